@@ -126,13 +126,17 @@ spdba_status make_pass(Pass<T>* out, int64_t L, int sign, int mode, long long O,
     if ((L - 1) * (isJ > osJ ? isJ : osJ) + 4096 * (isI > osI ? isI : osI) > 0x7fffffffLL)
         return fail(SPDBA_ERR_UNSUPPORTED, "FFT pass with a tile span beyond 2^31 elements");
     KernelInfo ki;
+    if (mode == PASS_CH_CHAIN) {
+        if (!loadp || !storep || isO != osO || isJ != osJ || !get_chain_kernel<T>(L, &ki) || I % ki.P != 0)
+            return fail(SPDBA_ERR_UNSUPPORTED, "no step chain kernel for length %lld", (long long)L);
+    } else
     // the tile size depends only on (T, L); ask once to learn P
     if (!get_pass_kernel<T>(L, sign, mode, loadp, storep, true, &ki))
         return fail(SPDBA_ERR_UNSUPPORTED, "no FFT pass kernel for length %lld (mode %d)", (long long)L, mode);
     const bool generic = (I % ki.P) != 0;
-    if (!get_pass_kernel<T>(L, sign, mode, loadp, storep, generic, &ki))
+    if (mode != PASS_CH_CHAIN && !get_pass_kernel<T>(L, sign, mode, loadp, storep, generic, &ki))
         return fail(SPDBA_ERR_UNSUPPORTED, "no FFT pass kernel for length %lld (mode %d)", (long long)L, mode);
-    spdba_status s = ensure_smem_attr(ki.func, ki.smem, ki.pipe);
+    spdba_status s = ensure_smem_attr(ki.func, ki.smem, ki.pipe || mode == PASS_CH_CHAIN);
     if (s != SPDBA_OK) return s;
     long long ntiles = (O * I + ki.P - 1) / ki.P;
     long long grid = ntiles;

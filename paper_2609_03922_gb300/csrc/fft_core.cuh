@@ -249,23 +249,21 @@ __device__ __forceinline__ void load_tile(cx_t<T>* sm, const PassParams<T>& a, l
 // pair of a row contiguous, so complex64 moves in 16-byte pieces; the padded
 // layout A moves complex64 one element (8 bytes) at a time.
 template <typename T, int L, int P, int NT, bool PFAST, class LY>
-__device__ __forceinline__ void issue_tile(cx_t<T>* sm, const PassParams<T>& a, long long q0) {
+__device__ __forceinline__ void issue_tile_at(cx_t<T>* sm, const cx_t<T>* base, long long sI, long long sJ) {
     using C = cx_t<T>;
-    const long long o = a.fd_I.div((uint32_t)q0), i0 = q0 - o * a.I;
-    const C* base = a.in + o * a.isO + i0 * a.isI;
     if constexpr (sizeof(C) == 8 && PFAST) {
         constexpr int UNITS = P * L / 2;
 #pragma unroll 4
         for (int u = threadIdx.x; u < UNITS; u += NT) {
             int j = u / (P / 2), p = (u % (P / 2)) * 2;
-            cp_async16(sm + LY::idx(p, j), base + (long long)p * a.isI + (long long)j * a.isJ);
+            cp_async16(sm + LY::idx(p, j), base + (long long)p * sI + (long long)j * sJ);
         }
     } else if constexpr (sizeof(C) == 8) {
         constexpr int UNITS = P * L;
 #pragma unroll 4
         for (int u = threadIdx.x; u < UNITS; u += NT) {
             int p = u / L, j = u % L;
-            cp_async8(sm + LY::idx(p, j), base + (long long)p * a.isI + (long long)j * a.isJ);
+            cp_async8(sm + LY::idx(p, j), base + (long long)p * sI + (long long)j * sJ);
         }
     } else {
         constexpr int UNITS = P * L;
@@ -274,9 +272,14 @@ __device__ __forceinline__ void issue_tile(cx_t<T>* sm, const PassParams<T>& a, 
             int p, j;
             if constexpr (PFAST) { j = u / P; p = u % P; }
             else { p = u / L; j = u % L; }
-            cp_async16(sm + LY::idx(p, j), base + (long long)p * a.isI + (long long)j * a.isJ);
+            cp_async16(sm + LY::idx(p, j), base + (long long)p * sI + (long long)j * sJ);
         }
     }
+}
+template <typename T, int L, int P, int NT, bool PFAST, class LY>
+__device__ __forceinline__ void issue_tile(cx_t<T>* sm, const PassParams<T>& a, long long q0) {
+    const long long o = a.fd_I.div((uint32_t)q0), i0 = q0 - o * a.I;
+    issue_tile_at<T, L, P, NT, PFAST, LY>(sm, a.in + o * a.isO + i0 * a.isI, a.isI, a.isJ);
 }
 
 // Asynchronous load of a z-pencil tile of a 3-D field from its half array
@@ -802,6 +805,9 @@ enum PassMode : int {
     PASS_UPD_HALF = 6,   // forward z-transform of the half array, then the CH update of c_hat
     // PASS_MIRROR with one transform per half pencil for x frequencies kx and N2 - kx
     PASS_PAIR_MIRROR = 7,
+    // PASS_CH_UPDATE, then the inverse transform of the updated c_hat: the last pass of a
+    // step and the first of the next in one (fft_chain_kernel)
+    PASS_CH_CHAIN = 8,
 };
 constexpr bool is_update_mode(int m) { return m == PASS_CH_UPDATE || m == PASS_UPD_HALF; }
 constexpr bool reads_half(int m) { return m == PASS_MIRROR || m == PASS_UPD_HALF; }
@@ -1261,6 +1267,112 @@ __global__ void __launch_bounds__(NT, PipeOcc<T, L, MODE, PFAST>::value) fft_pas
         t = tn;
     }
     cp_async_wait<0>();
+}
+
+// ---------------------------------------------------------------- step chain
+// The pass along the field's first axis of two consecutive steps in one kernel:
+// forward transform of g, the update of c_hat, and the inverse transform of the
+// updated c_hat that the next step starts with.  Run apart, these are two
+// passes over the workspace and two over c_hat (read by the update and again by
+// the inverse); here a tile's pencils of g and of c_hat are read once, the
+// non-frozen rows of c_hat written, and the inverse transform stored over g.
+// The update sits between the two transforms in registers where the last radix
+// equals the first (fused_mid_stage), with the same arithmetic as the separate
+// kernels, bit for bit.
+//
+// One tile per CTA and no second buffer: the c_hat tile takes its place in
+// shared memory, and the other resident CTAs cover a CTA's loads (the passes run
+// at the same rate with either, as HBM and L2 bound them).  A tile whose blocks
+// are all FROZEN reads no g and is only inverse-transformed.
+template <typename T, int L, int P, int NT, class LY> struct ChainMid {
+    using C = cx_t<T>;
+    static_assert(NT % P == 0, "each thread keeps one pencil");
+    const CHFuse<T>& f;
+    const uint8_t* tab;   // shared per-tile table
+    const T* kp;          // shared |k|^2 table of the pass axis
+    const C* cs;          // c_hat tile
+    C* cb;                // c_hat of (this thread's pencil, j = 0)
+    int nbx, bxs, lx, l_out, osJ;
+    bool d3;
+    T kx, kc;
+    __device__ __forceinline__ ChainMid(const PassParams<T>& a, const UpdTile& u, const uint8_t* tab_, const T* kp_,
+                                        const C* cs_)
+        : f(a.fu), tab(tab_), kp(kp_), cs(cs_) {
+        d3 = f.g.ndim == 3;
+        nbx = u.nbx;
+        const int p = (int)(threadIdx.x % P);
+        const int x = u.x0 + p, bx = (int)f.fd_b2.div((uint32_t)x);
+        bxs = bx - u.bx0;
+        lx = x - bx * f.g.b[2];
+        kx = f.k2ax[2][x];
+        kc = d3 ? f.k2ax[1][u.cy] : f.k2ax[0][u.cy];
+        l_out = u.l_out;
+        cb = f.c_hat + ((long long)u.o * a.osO + (long long)(u.i0 + p) * a.osI);
+        osJ = (int)a.osJ;
+    }
+    __device__ __forceinline__ C operator()(int p, int m, C gv) {
+        const C c = cs[LY::idx(p, m)];
+        const int bp = (int)f.fd_bp.div((uint32_t)m);
+        const unsigned e = tab[bp * nbx + bxs];
+        const int st = (int)(e & 3u);
+        if (st == SPDBA_FROZEN) return c;
+        // same association as the staged kernels: (k_outer + k_pass) then + k_x
+        const T k01 = d3 ? kp[m] + kc : kc + kp[m];
+        C nv = ch_new(c, gv, k01 + kx, f.dt, f.dtkappa);
+        if (st == SPDBA_TRANSITION) {
+            const int lj = m - bp * (d3 ? f.g.b[0] : f.g.b[1]);
+            nv = d3 ? ch_blend<T>(c, nv, f.taper, f.g, e >> 2, lj, l_out, lx)
+                    : ch_blend<T>(c, nv, f.taper, f.g, e >> 2, 0, lj, lx);
+        }
+        cb[m * osJ] = nv;
+        return nv;
+    }
+};
+
+// Resident CTAs per SM the chain kernel is compiled for.
+template <typename T, int L, int NT> struct ChainOcc {
+    static constexpr int value = sizeof(T) != 4 ? 1 : 512 / NT;
+};
+
+template <typename T, int L, int P, int NT>
+__global__ void __launch_bounds__(NT, ChainOcc<T, L, NT>::value) fft_chain_kernel(PassParams<T> a) {
+    using C = cx_t<T>;
+    using LY = PipeLayout<L, P, true>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    C* const sm = reinterpret_cast<C*>(smem_raw);
+    C* const cs = sm + LY::SIZE;
+    __shared__ uint8_t s_tab[kUpdTable];
+    __shared__ T s_kp[L];
+    constexpr bool STW = sizeof(T) == 4;   // twiddles in shared memory, as in the pipelined kernel
+    __shared__ C s_tw[STW ? L : 1];
+    const CHFuse<T>& f = a.fu;
+    const long long q0 = (long long)blockIdx.x * P;
+    const UpdTile u = upd_tile<T, P>(a, (int)q0);
+    issue_tile_at<T, L, P, NT, true, LY>(cs, f.c_hat + ((long long)u.o * a.osO + (long long)u.i0 * a.osI), a.osI,
+                                         a.osJ);
+    ch_update_stats<T, NT>(f, f.dense);
+    const T* kpg = f.g.ndim == 3 ? f.k2ax[0] : f.k2ax[1];
+    for (int j = threadIdx.x; j < L; j += NT) s_kp[j] = kpg[j];
+    if constexpr (STW)
+        for (int j = threadIdx.x; j < L; j += NT) s_tw[j] = a.tw[j];
+    const C* const tw = STW ? s_tw : a.tw;
+    const int nent = (int)(f.g.ndim == 3 ? f.g.nb[0] : f.g.nb[1]) * u.nbx;
+    ch_update_table<T, L, P, NT>(s_tab, a, u);
+    __syncthreads();
+    int any = 0;
+    for (int k = threadIdx.x; k < nent; k += NT) any |= (s_tab[k] & 3) != SPDBA_FROZEN;
+    const bool live = __syncthreads_or(any) != 0;
+    if (live) issue_tile<T, L, P, NT, true, LY>(sm, a, q0);
+    cp_async_commit();
+    cp_async_wait<0>();
+    __syncthreads();
+    PlainOut<T, L> out(a, q0);
+    if (live) {
+        ChainMid<T, L, P, NT, LY> mid(a, u, s_tab, s_kp, cs);
+        transform_pair<T, L, P, NT, -1, +1, LY>(sm, tw, mid, out);
+    } else {
+        run_stages_out<T, L, P, NT, +1, LY>(cs, tw, out);
+    }
 }
 
 }  // namespace spdba

@@ -11,6 +11,8 @@ struct KernelInfo {
 // generic: the pencil count is not a multiple of the tile (simple kernel only)
 template <typename T>
 bool get_pass_kernel(int64_t L, int sign, int mode, bool loadp, bool storep, bool generic, KernelInfo* ki);
+// the step chain (PASS_CH_CHAIN) along the first axis
+template <typename T> bool get_chain_kernel(int64_t L, KernelInfo* ki);
 // complex64 half-spectrum passes (PASS_HERM_INV, PASS_NL_HALF, PASS_MIRROR,
 // PASS_UPD_HALF); nhp = half row length (PASS_NL_HALF shared memory)
 bool get_half_kernel(int64_t L, int mode, int nhp, KernelInfo* ki);

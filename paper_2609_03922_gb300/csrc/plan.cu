@@ -165,6 +165,11 @@ template <typename T> struct Group {
     bool fused_update = false;      // the last forward pass carries the update (upd_pass)
     bool has_fused = false;         // upd_pass exists (else only the staged form)
     Pass<T> upd_pass;               // forward pass of the first axis with the update fused
+    // step chain: upd_pass and the next step's first inverse pass in one kernel, used
+    // between two steps of one call where the fused update is in force
+    Pass<T> chain;
+    bool has_chain = false;
+    bool pre_done = false;          // `work` holds the first inverse pass of c_hat (set by the chain, within a call)
     FftEngine<T> fft1;              // one run's transforms for set/get_field
     // NLS
     HPair<T>* H = nullptr;
@@ -219,10 +224,10 @@ template <typename T> struct Group {
 using namespace spdba;
 
 enum ProfKind { K_FFT_PASS = 0, K_FUSED_NL, K_UPDATE_DENSE, K_UPDATE_LIST, K_ASSESS, K_NLS_STEP, K_NLS_ROW, K_NLS_COL,
-                K_FFT_UPDATE, K_FFT_ZFWD, K_RCD_FFT, K_RCD_REACTION, K_FFT_YFWD, K_PREDICT, K_COUNT };
+                K_FFT_UPDATE, K_FFT_ZFWD, K_RCD_FFT, K_RCD_REACTION, K_FFT_YFWD, K_PREDICT, K_FFT_CHAIN, K_COUNT };
 static const char* kProfName[K_COUNT] = {"fft_pass", "fft_fused_nl", "update_dense", "update_list", "assess",
                                          "nls_step", "nls_row", "nls_col", "fft_update", "fft_z_forward",
-                                         "rcd_fft", "rcd_reaction", "fft_y_forward_pruned", "predict"};
+                                         "rcd_fft", "rcd_reaction", "fft_y_forward_pruned", "predict", "fft_update_inverse"};
 
 struct ProfRec {
     int kind;
@@ -254,6 +259,18 @@ struct MultiForm {
     MultiPhase inv, nl, upd;   // inverse along axis 0; nonlinearity along axis 1; forward + update along axis 0
 };
 
+// A captured segment of steps.
+struct SegGraph {
+    cudaGraphExec_t exec = nullptr;
+    long long launches = 0;
+    long long list_updates = 0;   // list-driven updates in the segment
+    bool chain_out = false;       // its last step chained into the next
+    void release() {
+        if (exec) cudaGraphExecDestroy(exec);
+        exec = nullptr;
+    }
+};
+
 struct spdba_plan {
     spdba_options opt;
     MultiForm multi[2];     // tile tables of 4096 and 2048 elements
@@ -280,12 +297,12 @@ struct spdba_plan {
     std::vector<RunRef> runs;
     TwiddleCache<float> tw32;
     TwiddleCache<double> tw64;
-    cudaGraphExec_t seg_exec = nullptr;   // one reassessment segment (R steps of every group)
+    // one reassessment segment (R steps of every group): bit 0 chained into by the
+    // step before, bit 1 chained out of into the step after
+    SegGraph seg[4];
     spdba_predictor* pred = nullptr;
     int horizon = 0, judge_every = 0;
     float prob_thr = 0.5f;
-    long long seg_launches = 0;
-    long long seg_list_updates = 0;   // list-driven updates in one captured segment
     // groups step concurrently on their own streams, forked from and joined to st
     std::vector<cudaStream_t> gstreams;
     std::vector<cudaEvent_t> gevents;
@@ -402,6 +419,23 @@ template <typename T> static void fill_fuse(const spdba_plan* p, const Group<T>&
     f.fd_b2.init((uint32_t)r.g.b[2]);
     f.fd_b1.init((uint32_t)r.g.b[1]);
     f.fd_n2.init((uint32_t)r.g.n[2]);
+}
+
+// The step chain along the first axis of a CH group's spectrum of extents d
+// (r.has_chain stays false where no kernel fits): its tiles lie within one row
+// of the last axis, and their state table fits the kernel's.
+template <typename T>
+static spdba_status setup_chain(spdba_plan* p, Group<T>& r, int ndim, const int64_t* d, long long batch) {
+    Pass<T> c;
+    spdba_status s = make_axis_pass<T>(&c, ndim, d, batch, 0, -1, PASS_CH_CHAIN, twc<T>(p), p->st);
+    if (s == SPDBA_ERR_UNSUPPORTED) return SPDBA_OK;
+    if (s != SPDBA_OK) return s;
+    const int64_t bpass = ndim == 3 ? r.g.b[0] : r.g.b[1];
+    if (d[ndim - 1] % c.P != 0 || (d[0] / bpass) * (int64_t)upd_table_cols(c.P, r.g.b[2]) > kUpdTable) return SPDBA_OK;
+    fill_fuse<T>(p, r, c.p.fu);
+    r.chain = c;
+    r.has_chain = true;
+    return SPDBA_OK;
 }
 
 // Half-spectrum passes of a 3-D complex64 group; SPDBA_ERR_UNSUPPORTED (and
@@ -537,6 +571,7 @@ static spdba_status group_init_ch_hs(spdba_plan* p, Group<float>& r, const int64
         r.h_upd = up;
         r.has_fused = true;
         r.fused_update = p->opt.fuse_update != 0;
+        if ((s = setup_chain<float>(p, r, 3, dh, 1)) != SPDBA_OK) return s;
     } else if (s != SPDBA_OK && s != SPDBA_ERR_UNSUPPORTED) {
         return s;
     }
@@ -611,6 +646,7 @@ static spdba_status group_init_ch(spdba_plan* p, Group<T>& r, int ndim, const in
                 r.upd_pass = ps;
                 r.has_fused = true;
                 r.fused_update = true;
+                if ((s = setup_chain<T>(p, r, ndim, dims, batch)) != SPDBA_OK) return s;
             } else if (sf != SPDBA_ERR_UNSUPPORTED) {
                 return sf;
             }
@@ -855,10 +891,26 @@ static void prof_select(spdba_plan* p, long long step) {
 
 template <typename T> static spdba_status ch_staged_update(spdba_plan* p, Group<T>& r, int dense);
 
-template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>& r) {
+// The last pass of a step with the update, chained into the next step's first inverse pass.
+template <typename T> static spdba_status ch_chain(spdba_plan* p, Group<T>& r, int dense, double bytes) {
+    Pass<T> ps = r.chain;
+    ps.p.fu.dense = dense;
+    ProfScope pr(p, K_FFT_CHAIN, bytes);
+    spdba_status s = launch_pass<T>(ps, r.work, r.work, p->st);
+    if (s != SPDBA_OK) return s;
+    p->launches += 1;
+    r.pre_done = true;
+    r.step += 1;
+    return SPDBA_OK;
+}
+
+// more: another step of this group follows in the same call (or captured segment).
+template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>& r, bool more) {
     cudaStream_t st = p->st;
     spdba_status s;
     prof_select(p, r.step);
+    // between two steps the fused update runs as a chain into the next step's first inverse pass
+    const bool chain = more && r.has_chain && r.fused_update && !r.use_half;
     const bool adaptive = p->opt.mode == SPDBA_MODE_ADAPTIVE;
     const int interval = p->pred ? p->horizon : p->reassess;
     const bool reassess = adaptive && (!r.assessed || r.step % interval == 0);
@@ -889,10 +941,12 @@ template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>&
         // the stored half, then the update (fused into the z forward or staged).
         // Profiled bytes are algorithmic: x frequencies 0 .. N2/2.
         const double hb = sizeof(cx_t<T>) * (double)(r.dims[0] * r.dims[1] * (r.dims[2] / 2 + 1));
-        {
+        if (!r.pre_done) {
             ProfScope pr(p, K_FFT_PASS, 2.0 * hb);
             if ((s = launch_pass<T>(r.h_inv_z, r.c_hat, r.work, st)) != SPDBA_OK) return s;
+            p->launches += 1;
         }
+        r.pre_done = false;
         {
             ProfScope pr(p, K_FFT_PASS, 2.0 * hb);
             if ((s = launch_pass<T>(r.h_inv_y, r.work, r.work, st)) != SPDBA_OK) return s;
@@ -915,7 +969,8 @@ template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>&
             ProfScope pr(p, dense ? K_FFT_PASS : K_FFT_YFWD, 2.0 * hb);
             if ((s = launch_pass<T>(yf, r.work, r.work, st)) != SPDBA_OK) return s;
         }
-        p->launches += 5;
+        p->launches += 4;
+        if (chain) return ch_chain<T>(p, r, dense, 4.0 * hb);
         if (r.fused_update) {
             Pass<T> ps = r.h_upd;
             ps.p.fu.dense = dense;
@@ -995,12 +1050,18 @@ template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>&
     // pre-update: c = Re(IFFT(c_hat)), g = c^3 - c, g_hat = FFT(g)
     const double pass_bytes = 2.0 * sizeof(cx_t<T>) * (double)(r.batch * r.n);
     const cx_t<T>* src = r.c_hat;
-    for (auto& ps : r.pre_inv) {
+    for (size_t k = 0; k < r.pre_inv.size(); ++k) {
+        const Pass<T>& ps = r.pre_inv[k];
+        if (k == 0 && r.pre_done) {
+            src = r.work;
+            continue;
+        }
         ProfScope pr(p, K_FFT_PASS, pass_bytes);
         if ((s = launch_pass<T>(ps, src, r.work, st)) != SPDBA_OK) return s;
         p->launches += 1;
         src = r.work;
     }
+    r.pre_done = false;
     Pass<T> fused = r.fused;
     if (reassess) {
         fused.p.mass = &r.stats[0].mass;
@@ -1014,6 +1075,7 @@ template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>&
     }
     for (size_t k = 0; k < r.pre_fwd.size(); ++k) {
         const bool last_fused = r.fused_update && k + 1 == r.pre_fwd.size();
+        if (last_fused && chain) return ch_chain<T>(p, r, dense, 2.0 * pass_bytes);
         if (last_fused) {
             // forward transform of the first axis + update; traffic depends on the states
             Pass<T> ps = r.upd_pass;
@@ -1335,10 +1397,11 @@ static spdba_status multi_ch_step(spdba_plan* p, const MultiForm& mf) {
     return SPDBA_OK;
 }
 
-template <typename T> static spdba_status group_steps(spdba_plan* p, Group<T>& g, int64_t n) {
+template <typename T> static spdba_status group_steps(spdba_plan* p, Group<T>& g, int64_t n, bool more) {
     if (p->opt.model == SPDBA_MODEL_NLS) return group_nls_steps<T>(p, g, n);
     for (int64_t i = 0; i < n; ++i) {
-        spdba_status s = p->opt.model == SPDBA_MODEL_RCD ? group_rcd_step<T>(p, g) : group_ch_step<T>(p, g);
+        spdba_status s = p->opt.model == SPDBA_MODEL_RCD ? group_rcd_step<T>(p, g)
+                                                         : group_ch_step<T>(p, g, more || i + 1 < n);
         if (s != SPDBA_OK) return s;
     }
     return SPDBA_OK;
@@ -1359,7 +1422,8 @@ static spdba_status ensure_group_streams(spdba_plan* p, size_t ngroups) {
     return SPDBA_OK;
 }
 
-template <typename T> static spdba_status direct_steps(spdba_plan* p, int64_t n) {
+// n steps of every group; more: other steps follow these in the same call.
+template <typename T> static spdba_status direct_steps(spdba_plan* p, int64_t n, bool more) {
     auto& gs = groups<T>(p);
     if constexpr (std::is_same<T, float>::value) {
         if (p->multi_sel > 0 && p->opt.model == SPDBA_MODEL_CH) {
@@ -1382,7 +1446,7 @@ template <typename T> static spdba_status direct_steps(spdba_plan* p, int64_t n)
         for (size_t i = 0; i < gs.size() && s == SPDBA_OK; ++i) {
             SPDBA_CUDA(cudaStreamWaitEvent(p->gstreams[i], p->fork_ev, 0));
             p->st = p->gstreams[i];
-            s = group_steps<T>(p, *gs[i], n);
+            s = group_steps<T>(p, *gs[i], n, more);
             p->st = main;
             cudaError_t e = cudaEventRecord(p->gevents[i], p->gstreams[i]);
             if (s == SPDBA_OK && e != cudaSuccess) s = cuda_fail(e, "cudaEventRecord(group)");
@@ -1403,7 +1467,8 @@ template <typename T> static spdba_status direct_steps(spdba_plan* p, int64_t n)
     }
     for (int64_t i = 0; i < n; ++i) {
         for (auto& g : gs) {
-            spdba_status s = p->opt.model == SPDBA_MODEL_RCD ? group_rcd_step<T>(p, *g) : group_ch_step<T>(p, *g);
+            spdba_status s = p->opt.model == SPDBA_MODEL_RCD ? group_rcd_step<T>(p, *g)
+                                                             : group_ch_step<T>(p, *g, more || i + 1 < n);
             if (s != SPDBA_OK) return s;
         }
     }
@@ -1426,18 +1491,31 @@ template <typename T> static bool segment_ready(spdba_plan* p) {
     return true;
 }
 
+// Whether every CH group holds its first inverse pass (a chain ended the last step).
+template <typename T> static bool chained(spdba_plan* p) {
+    for (auto& g : groups<T>(p))
+        if (g->pre_done) return true;
+    return false;
+}
+
 template <typename T> static spdba_status plan_step(spdba_plan* p, int64_t n) {
+    // nothing is carried over from an earlier call: the workspace may have been used since
+    for (auto& g : groups<T>(p)) g->pre_done = false;
     // graphs need a capturable (non-legacy) stream; a profile of every step records
     // events per kernel (a sampled one keeps graphs for unsampled segments)
-    if (!p->opt.use_graph || (p->prof && p->prof_every <= 1) || p->st == 0) return direct_steps<T>(p, n);
+    if (!p->opt.use_graph || (p->prof && p->prof_every <= 1) || p->st == 0) return direct_steps<T>(p, n, false);
     const int R = p->reassess;
     int64_t i = 0;
     while (i < n) {
         if (n - i >= R && segment_ready<T>(p)) {
-            if (!p->seg_exec) {
+            // the launches differ with the step before (chained into this segment or not)
+            // and with whether steps follow: one graph each
+            const bool more = n - i > R;
+            SegGraph& sg = p->seg[(chained<T>(p) ? 1 : 0) + (more ? 2 : 0)];
+            if (!sg.exec) {
                 const long long l0 = p->launches, u0 = p->list_updates;
                 SPDBA_CUDA(cudaStreamBeginCapture(p->st, cudaStreamCaptureModeThreadLocal));
-                spdba_status s = direct_steps<T>(p, R);
+                spdba_status s = direct_steps<T>(p, R, more);
                 cudaGraph_t graph = nullptr;
                 cudaError_t e = cudaStreamEndCapture(p->st, &graph);
                 if (s != SPDBA_OK) {
@@ -1445,28 +1523,30 @@ template <typename T> static spdba_status plan_step(spdba_plan* p, int64_t n) {
                     return s;
                 }
                 if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
-                e = cudaGraphInstantiate(&p->seg_exec, graph, 0);
+                e = cudaGraphInstantiate(&sg.exec, graph, 0);
                 cudaGraphDestroy(graph);
                 if (e != cudaSuccess) {
-                    p->seg_exec = nullptr;
+                    sg.exec = nullptr;
                     return cuda_fail(e, "cudaGraphInstantiate");
                 }
-                p->seg_launches = p->launches - l0;
-                p->seg_list_updates = p->list_updates - u0;
+                sg.launches = p->launches - l0;
+                sg.list_updates = p->list_updates - u0;
+                sg.chain_out = chained<T>(p);
                 // the capture advanced the host-side step counters; run what it recorded
-                SPDBA_CUDA(cudaGraphLaunch(p->seg_exec, p->st));
+                SPDBA_CUDA(cudaGraphLaunch(sg.exec, p->st));
             } else {
-                SPDBA_CUDA(cudaGraphLaunch(p->seg_exec, p->st));
+                SPDBA_CUDA(cudaGraphLaunch(sg.exec, p->st));
                 for (auto& g : groups<T>(p)) {
                     g->step += R;
                     if (p->opt.mode == SPDBA_MODE_ADAPTIVE) g->assessed = true;
+                    g->pre_done = sg.chain_out && g->has_chain && g->fused_update && !g->use_half;
                 }
-                p->launches += p->seg_launches;
-                p->list_updates += p->seg_list_updates;
+                p->launches += sg.launches;
+                p->list_updates += sg.list_updates;
             }
             i += R;
         } else {
-            spdba_status s = direct_steps<T>(p, 1);
+            spdba_status s = direct_steps<T>(p, 1, i + 1 < n);
             if (s != SPDBA_OK) return s;
             ++i;
         }
@@ -1784,7 +1864,7 @@ extern "C" void spdba_plan_destroy(spdba_plan* p) {
     p->tw32.release();
     p->tw64.release();
     for (cudaEvent_t e : p->ev_pool) cudaEventDestroy(e);
-    if (p->seg_exec) cudaGraphExecDestroy(p->seg_exec);
+    for (SegGraph& sg : p->seg) sg.release();
     for (cudaStream_t gs : p->gstreams) {
         cudaStreamSynchronize(gs);
         cudaStreamDestroy(gs);
@@ -1884,10 +1964,7 @@ template <typename T> static void apply_config(spdba_plan* p, int fuse, int grap
     p->multi_sel = (multi > 0 && fuse && p->multi[multi - 1].ok) ? multi : 0;
     p->opt.multi_pass = p->multi_sel;
     p->opt.use_graph = graph;
-    if (p->seg_exec) {
-        cudaGraphExecDestroy(p->seg_exec);
-        p->seg_exec = nullptr;
-    }
+    for (SegGraph& sg : p->seg) sg.release();
 }
 
 // ------------------------------------------------------------------ tuning cache
