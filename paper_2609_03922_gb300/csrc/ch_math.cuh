@@ -6,6 +6,15 @@
 
 namespace spdba {
 
+// 1 / x by the hardware approximation, for normal x (the update's denominators
+// lie in [1, 2^126)): the value of __fdividef(1, x) there, bit for bit, without
+// its handling of subnormal x.
+__device__ __forceinline__ float rcp_approx(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 // Evaluation order is pinned with explicit fma so that the Regular and the
 // sp-DBA kernels produce bit-identical values for the same mode.  The FP32
 // reciprocal is the hardware approximation (at most 2 ulp), far inside the

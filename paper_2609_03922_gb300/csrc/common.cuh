@@ -11,6 +11,52 @@ template <> struct Cx<float> { using type = float2; };
 template <> struct Cx<double> { using type = double2; };
 template <typename T> using cx_t = typename Cx<T>::type;
 
+// Two FP32 values in one 64-bit register, for the packed FP32 instructions of
+// sm_100 and later (one issue slot for two rounded operations, the same bits as
+// two scalar ones).  Used as the element type of transforms that carry two
+// pencils per thread: Cx<f32x2>::type holds (re0, re1), (im0, im1).
+__host__ __device__ constexpr unsigned long long f32x2_dup(float a) {
+    const unsigned u = __builtin_bit_cast(unsigned, a);
+    return ((unsigned long long)u << 32) | u;
+}
+struct f32x2 {
+    unsigned long long v;
+    f32x2() = default;
+    __host__ __device__ constexpr explicit f32x2(double a) : v(f32x2_dup((float)a)) {}
+    __host__ __device__ constexpr explicit f32x2(float a) : v(f32x2_dup(a)) {}
+    __host__ __device__ constexpr explicit f32x2(int a) : v(f32x2_dup((float)a)) {}
+    __device__ __forceinline__ f32x2(float a, float b) { asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b)); }
+    __device__ __forceinline__ float lo() const {
+        return __uint_as_float((unsigned)v);
+    }
+    __device__ __forceinline__ float hi() const {
+        return __uint_as_float((unsigned)(v >> 32));
+    }
+};
+__device__ __forceinline__ f32x2 operator+(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f32x2 operator-(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f32x2 operator-(f32x2 a) { return f32x2(0.f) - a; }
+__device__ __forceinline__ f32x2 mul_rn(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma_rn(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+struct alignas(16) cf32x2 { f32x2 x, y; };
+template <> struct Cx<f32x2> { using type = cf32x2; };
+
 template <typename C> __device__ __forceinline__ C mk(decltype(C::x) a, decltype(C::x) b) {
     C r; r.x = a; r.y = b; return r;
 }
@@ -58,8 +104,8 @@ template <int M, int SIGN, typename C> __device__ __forceinline__ C twiddle16(C 
     else if constexpr (m == 8) return mk<C>(-x.x, -x.y);
     else if constexpr (m == 12) return cmul_si<-SIGN>(x);
     else {
-        constexpr T c = (T)cos16(m);
-        constexpr T s = (T)(SIGN * sin16(m));
+        constexpr double cd = cos16(m), sd = SIGN * sin16(m);
+        const T c = (T)cd, s = (T)sd;
         return mk<C>(fma_rn(x.x, c, -mul_rn(x.y, s)), fma_rn(x.x, s, mul_rn(x.y, c)));
     }
 }
@@ -76,23 +122,25 @@ template <int SIGN, typename C> struct Dft<2, SIGN, C> {
 template <int SIGN, typename C> struct Dft<3, SIGN, C> {
     static __device__ __forceinline__ void run(C* v) {
         using T = decltype(C::x);
-        const T h = (T)0.5;
-        const T r3 = (T)(SIGN * 0.86602540378443865);   // SIGN * sqrt(3)/2
+        const T nh = (T)-0.5;
+        const T r3 = (T)(SIGN * 0.86602540378443865), nr3 = (T)(-SIGN * 0.86602540378443865);   // SIGN * sqrt(3)/2
         C t1 = cadd(v[1], v[2]);
-        C t2 = mk<C>(fma_rn(-h, t1.x, v[0].x), fma_rn(-h, t1.y, v[0].y));
+        C t2 = mk<C>(fma_rn(nh, t1.x, v[0].x), fma_rn(nh, t1.y, v[0].y));
         C d = csub(v[1], v[2]);
-        C t3 = mk<C>(mul_rn(-r3, d.y), mul_rn(r3, d.x));   // i * r3 * (v1 - v2)
+        // t2 +- i r3 d, as fused multiply-adds in every element type
         v[0] = cadd(v[0], t1);
-        v[1] = cadd(t2, t3);
-        v[2] = csub(t2, t3);
+        v[1] = mk<C>(fma_rn(nr3, d.y, t2.x), fma_rn(r3, d.x, t2.y));
+        v[2] = mk<C>(fma_rn(r3, d.y, t2.x), fma_rn(nr3, d.x, t2.y));
     }
 };
 template <int SIGN, typename C> struct Dft<4, SIGN, C> {
     static __device__ __forceinline__ void run(C* v) {
+        // t1 +- SIGN i d as sums and differences (no negated copy of d)
         C t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]);
-        C t2 = cadd(v[1], v[3]), t3 = cmul_si<SIGN>(csub(v[1], v[3]));
+        C t2 = cadd(v[1], v[3]), d = csub(v[1], v[3]);
+        const C p = mk<C>(t1.x - d.y, t1.y + d.x), m = mk<C>(t1.x + d.y, t1.y - d.x);
         v[0] = cadd(t0, t2); v[2] = csub(t0, t2);
-        v[1] = cadd(t1, t3); v[3] = csub(t1, t3);
+        v[1] = SIGN > 0 ? p : m; v[3] = SIGN > 0 ? m : p;
     }
 };
 
@@ -130,6 +178,19 @@ template <int A, int B, int SIGN, typename C> struct DftAB {
 #pragma unroll
             for (int k2 = 0; k2 < B; ++k2) v[k1 + A * k2] = t[k2];
         }
+    }
+};
+// Length 6 as 2 x 3 by the prime-factor map (no twiddles): input n = (3 a + 2 b)
+// mod 6, output k = (3 k1 + 4 k2) mod 6, for which n k / 6 = a k1 / 2 + b k2 / 3
+// up to whole turns.
+template <int SIGN, typename C> struct Dft<6, SIGN, C> {
+    static __device__ __forceinline__ void run(C* v) {
+        C t[2][3] = {{v[0], v[2], v[4]}, {v[3], v[5], v[1]}};
+        Dft<3, SIGN, C>::run(t[0]);
+        Dft<3, SIGN, C>::run(t[1]);
+        v[0] = cadd(t[0][0], t[1][0]); v[3] = csub(t[0][0], t[1][0]);
+        v[4] = cadd(t[0][1], t[1][1]); v[1] = csub(t[0][1], t[1][1]);
+        v[2] = cadd(t[0][2], t[1][2]); v[5] = csub(t[0][2], t[1][2]);
     }
 };
 template <int SIGN, typename C> struct Dft<8, SIGN, C> {

@@ -117,7 +117,7 @@ static spdba_status ensure_smem_attr(const void* f, int smem, bool max_carveout)
 template <typename T>
 spdba_status make_pass(Pass<T>* out, int64_t L, int sign, int mode, long long O, long long I, long long isO,
                        long long isI, long long isJ, long long osO, long long osI, long long osJ,
-                       TwiddleCache<T>& tw, cudaStream_t st) {
+                       TwiddleCache<T>& tw, cudaStream_t st, bool fourstep) {
     bool loadp = (isJ != 1), storep = (osJ != 1);
     if (loadp && isI != 1) return fail(SPDBA_ERR_UNSUPPORTED, "pass without a unit-stride input direction");
     if (storep && osI != 1) return fail(SPDBA_ERR_UNSUPPORTED, "pass without a unit-stride output direction");
@@ -126,24 +126,34 @@ spdba_status make_pass(Pass<T>* out, int64_t L, int sign, int mode, long long O,
     if ((L - 1) * (isJ > osJ ? isJ : osJ) + 4096 * (isI > osI ? isI : osI) > 0x7fffffffLL)
         return fail(SPDBA_ERR_UNSUPPORTED, "FFT pass with a tile span beyond 2^31 elements");
     KernelInfo ki;
-    if (mode == PASS_CH_CHAIN) {
-        if (!loadp || !storep || isO != osO || isJ != osJ || !get_chain_kernel<T>(L, &ki) || I % ki.P != 0)
-            return fail(SPDBA_ERR_UNSUPPORTED, "no step chain kernel for length %lld", (long long)L);
-    } else
-    // the tile size depends only on (T, L); ask once to learn P
-    if (!get_pass_kernel<T>(L, sign, mode, loadp, storep, true, &ki))
-        return fail(SPDBA_ERR_UNSUPPORTED, "no FFT pass kernel for length %lld (mode %d)", (long long)L, mode);
-    const bool generic = (I % ki.P) != 0;
-    if (mode != PASS_CH_CHAIN && !get_pass_kernel<T>(L, sign, mode, loadp, storep, generic, &ki))
-        return fail(SPDBA_ERR_UNSUPPORTED, "no FFT pass kernel for length %lld (mode %d)", (long long)L, mode);
-    spdba_status s = ensure_smem_attr(ki.func, ki.smem, ki.pipe || mode == PASS_CH_CHAIN);
+    int nsm = 0, dev = 0;
+    SPDBA_CUDA(cudaGetDevice(&dev));
+    SPDBA_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const bool chain = mode == PASS_CH_CHAIN;
+    if (chain && (!loadp || !storep || isO != osO || isJ != osJ))
+        return fail(SPDBA_ERR_UNSUPPORTED, "the step chain runs in place along a strided axis");
+    auto get = [&](TileKind kind) {
+        if (chain) return kind != TILE_GENERIC && get_chain_kernel<T>(L, kind == TILE_NARROW, &ki);
+        return get_pass_kernel<T>(L, sign, mode, loadp, storep, kind, fourstep, &ki);
+    };
+    // A pass of fewer wide tiles than SMs takes narrow ones (128 x 128: 8 against
+    // 32 tiles).  complex128 passes, bound by the SMs' FP64 rate, do so up to four
+    // wide tiles an SM, to spread evenly.
+    const long long few = (sizeof(T) == 8 ? 4 : 1) * (long long)nsm;
+    bool ok = get(TILE_WIDE);
+    if (ok && O * I < few * ki.P) {
+        const KernelInfo wide = ki;
+        if (!get(TILE_NARROW) || I % ki.P != 0) ki = wide;
+    }
+    const bool generic = !ok || I % ki.P != 0;
+    if (generic) ok = get(TILE_GENERIC);
+    if (!ok) return fail(SPDBA_ERR_UNSUPPORTED, "no FFT pass kernel for length %lld (mode %d)", (long long)L, mode);
+    spdba_status s = ensure_smem_attr(ki.func, ki.smem, !generic);
     if (s != SPDBA_OK) return s;
     long long ntiles = (O * I + ki.P - 1) / ki.P;
     long long grid = ntiles;
     if (ki.pipe) {
-        int per_sm = 0, nsm = 0, dev = 0;
-        SPDBA_CUDA(cudaGetDevice(&dev));
-        SPDBA_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+        int per_sm = 0;
         SPDBA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ki.func, ki.NT, ki.smem));
         if (per_sm < 1) per_sm = 1;
         long long resident = (long long)per_sm * nsm;
@@ -170,6 +180,17 @@ spdba_status make_pass(Pass<T>* out, int64_t L, int sign, int mode, long long O,
     ps.p.nl_scale = (T)1;
     ps.p.mass = nullptr;
     *out = ps;
+    return SPDBA_OK;
+}
+
+spdba_status set_pass_kernel(Pass<float>* ps, const KernelInfo& ki) {
+    spdba_status s = ensure_smem_attr(ki.func, ki.smem, true);
+    if (s != SPDBA_OK) return s;
+    ps->func = ki.func;
+    ps->nt = ki.NT;
+    ps->P = ki.P;
+    ps->smem = ki.smem;
+    ps->grid = ps->p.O * ps->p.I / ki.P;
     return SPDBA_OK;
 }
 
@@ -217,7 +238,7 @@ spdba_status FftEngine<T>::init(int nd, const int64_t* d, int64_t b, TwiddleCach
         for (int dir = 0; dir < 2; ++dir) {
             int sign = dir == 0 ? -1 : +1;
             Pass<T> p1, p2;
-            s = make_pass<T>(&p1, n1, sign, PASS_PLAIN, b, n2, n, 1, n2, n, 1, n2, tw, st);
+            s = make_pass<T>(&p1, n1, sign, PASS_PLAIN, b, n2, n, 1, n2, n, 1, n2, tw, st, true);
             if (s != SPDBA_OK) return s;
             p1.p.tw4 = t4;
             p1.p.n4 = n;
@@ -281,10 +302,10 @@ template struct FftEngine<float>;
 template struct FftEngine<double>;
 template spdba_status make_pass<float>(Pass<float>*, int64_t, int, int, long long, long long, long long, long long,
                                        long long, long long, long long, long long, TwiddleCache<float>&,
-                                       cudaStream_t);
+                                       cudaStream_t, bool);
 template spdba_status make_pass<double>(Pass<double>*, int64_t, int, int, long long, long long, long long, long long,
                                         long long, long long, long long, long long, TwiddleCache<double>&,
-                                        cudaStream_t);
+                                        cudaStream_t, bool);
 // Half-spectrum passes of a 3-D complex64 field (see fft_half.cuh).
 spdba_status make_half_pass(Pass<float>* out, int mode, const HalfGeo& hg, TwiddleCache<float>& tw, cudaStream_t st) {
     const bool rows = mode == PASS_NL_HALF;
@@ -329,7 +350,7 @@ spdba_status make_half_pass(Pass<float>* out, int mode, const HalfGeo& hg, Twidd
     SPDBA_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     SPDBA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ki.func, ki.NT, ki.smem));
     if (per_sm < 1) return fail(SPDBA_ERR_UNSUPPORTED, "half-spectrum kernel does not fit an SM");
-    ps.grid = std::min<long long>(ntiles, (long long)per_sm * nsm);
+    ps.grid = ki.pipe ? std::min<long long>(ntiles, (long long)per_sm * nsm) : ntiles;
     ps.func = ki.func;
     ps.nt = ki.NT;
     ps.P = ki.P;
@@ -346,6 +367,7 @@ spdba_status make_half_pass(Pass<float>* out, int mode, const HalfGeo& hg, Twidd
     a.mass_ppr = (long long)hg.N0 * hg.N1;
     a.fd_I.init((uint32_t)a.I);
     a.hg = hg;
+    a.hg.fd_HN.init((uint32_t)(hg.NHP / 2));
     *out = ps;
     return SPDBA_OK;
 }

@@ -30,6 +30,7 @@ namespace spdba {
 // Twiddle load: from a CTA's shared copy of the table (the compiler sees the
 // shared address space after inlining) or through the read-only cache.
 template <class C> __device__ __forceinline__ C tw_load(const C* p) { return __isShared(p) ? *p : __ldg(p); }
+__device__ __forceinline__ cf32x2 tw_load(const cf32x2* p) { return *p; }   // always a shared table
 
 // Radix schedule per pencil length (product of radices == L).
 template <int L> struct Radices;
@@ -38,9 +39,9 @@ template <> struct Radices<16> { using type = RList<16>; };
 template <> struct Radices<32> { using type = RList<8, 4>; };
 template <> struct Radices<64> { using type = RList<8, 8>; };
 template <> struct Radices<128> { using type = RList<16, 8>; };
-template <> struct Radices<192> { using type = RList<16, 4, 3>; };
+template <> struct Radices<192> { using type = RList<8, 3, 8>; };
 template <> struct Radices<256> { using type = RList<16, 16>; };
-template <> struct Radices<384> { using type = RList<16, 8, 3>; };
+template <> struct Radices<384> { using type = RList<8, 6, 8>; };
 template <> struct Radices<512> { using type = RList<8, 8, 8>; };
 template <> struct Radices<1024> { using type = RList<16, 16, 4>; };
 template <> struct Radices<2048> { using type = RList<16, 16, 8>; };
@@ -115,7 +116,7 @@ struct HalfGeo {
     // as a complex-to-real transform does (their planes need not be
     // conjugate-symmetric within themselves)
     int r2c = 0;
-    FastDiv fd_N2, fd_NHP, fd_M;   // fd_M: division by N2 / 2
+    FastDiv fd_N2, fd_NHP, fd_M, fd_HN;   // fd_M: division by N2 / 2; fd_HN: by NHP / 2
 };
 
 template <typename T> struct PassParams {
@@ -144,6 +145,7 @@ template <typename T> struct PassParams {
     // tile is skipped when none of its columns is marked (the outputs of
     // unmarked columns are never read), or null to transform every tile
     const uint8_t* col_live = nullptr;
+    int stream_chat = 0;   // step chain: c_hat is streamed past the L2
 };
 
 // Address of element (p, j) of the tile starting at pencil q0.
@@ -375,8 +377,12 @@ __device__ __forceinline__ void store_tile(const cx_t<T>* sm, const PassParams<T
 // to (j / NS) NS R + (j mod NS) + r NS (autosorting; natural order after the
 // last stage).
 // Reader of a stage's input element m of pencil p: the tile itself by default.
+// EXT: the inputs do not come from the buffer the stage writes, so no barrier
+// is needed between its reads and its writes.  before_write() runs between the two.
 template <typename T, class LY> struct SmemIn {
+    static constexpr bool EXT = false;
     const cx_t<T>* sm;
+    __device__ __forceinline__ void before_write() const {}
     __device__ __forceinline__ cx_t<T> operator()(int p, int m) const { return sm[LY::idx(p, m)]; }
 };
 
@@ -408,7 +414,8 @@ __device__ __forceinline__ void stockham_stage_in(cx_t<T>* sm, const cx_t<T>* __
             Dft<R, SIGN, C>::run(v[k]);
         }
     }
-    __syncthreads();
+    in.before_write();
+    if constexpr (!IN::EXT) __syncthreads();
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
         int b = threadIdx.x + k * NT;
@@ -535,6 +542,7 @@ template <typename T, int L, class LY, class MID> struct MidOut {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int m = j + r * (L / R);
+            if (r == 0) mid.begin(p, j);
             sm[LY::idx(p, m)] = mid(p, m, v[r]);
         }
     }
@@ -543,9 +551,10 @@ template <typename T, int L, class LY, class MID> struct MidOut {
 // c = Re(x) / N, g = c^3 - c (the CH nonlinearity), with the sum of c kept.
 template <typename T> struct ChNlMid {
     T scale, msum;
+    __device__ __forceinline__ void begin(int, int) {}
     __device__ __forceinline__ cx_t<T> operator()(int, int, cx_t<T> x) {
         const T c = mul_rn(x.x, scale);
-        msum += c;
+        msum = msum + c;
         return mk<cx_t<T>>(fma_rn(mul_rn(c, c), c, -c), (T)0);
     }
 };
@@ -610,7 +619,8 @@ template <typename T, int L, int R, class LY> struct FirstStageOut {
 // stage of the next (sign SB) of the same pencil, when both have radix R: the
 // first's butterfly j yields exactly the elements j + r L/R (natural order)
 // that the second's butterfly j reads, so both butterflies and an elementwise
-// step between them (mid(p, m, x) for element m) run in registers.  The
+// step between them (mid(p, m, x) for element m = j + r L/R, after mid.begin(p, j))
+// run in registers.  The
 // second stage's outputs go to `out` (j R + r for a stage that others follow).
 template <typename T, int L, int P, int NT, int SA, int SB, int NS, int R, class LY, class MID, class OUT>
 __device__ __forceinline__ void fused_mid_stage(cx_t<T>* sm, const cx_t<T>* __restrict__ tw, MID& mid, OUT& out) {
@@ -638,6 +648,7 @@ __device__ __forceinline__ void fused_mid_stage(cx_t<T>* sm, const cx_t<T>* __re
                     v[k][r] = cmul(v[k][r], w);
                 }
             }
+            mid.begin(p, j);
             Dft<R, SA, C>::run(v[k]);
 #pragma unroll
             for (int r = 0; r < R; ++r) v[k][r] = mid(p, j + r * Q, v[k][r]);
@@ -1142,18 +1153,20 @@ __global__ void __launch_bounds__(NT) fft_pass_kernel(PassParams<T> a) {
 // Resident CTAs per SM the pipelined kernel is compiled for (register budget).
 // (chosen from the compiler's register counts: the largest count of CTAs at
 // which the kernel does not spill)
-template <typename T, int L, int MODE, bool PFAST> struct PipeOcc {
+template <typename T, int L, int MODE, bool PFAST, int NT = 256> struct PipeOcc {
     static constexpr bool PLAINISH = MODE == PASS_PLAIN || MODE == PASS_MIRROR;
-    static constexpr int value = sizeof(T) != 4 || L > 512     ? 1
-                                 : L == 384 || L == 512        ? ((PLAINISH && (PFAST || L == 512)) ? 2 : 1)
-                                 : L == 192                    ? (MODE == PASS_CH_NL ? 1 : 2)
-                                 : is_update_mode(MODE)        ? 2
-                                                               : 3;
+    static constexpr int per256 = sizeof(T) != 4 || L > 512     ? 1
+                                  : L == 384 || L == 512        ? ((PLAINISH && (PFAST || L == 512)) ? 2 : 1)
+                                  : L == 192                    ? 2
+                                  : is_update_mode(MODE)        ? 2
+                                                                : 3;
+    static constexpr int value = sizeof(T) != 4 ? 1 : per256 * 256 / NT;   // the same registers a thread at any NT
 };
 
 // Shared-memory layout of the pipelined kernels' tiles.
+// (a row-major tile of one pencil is a pencil-major one, and padded as such)
 template <int L, int P, bool PFAST>
-using PipeLayout = typename std::conditional<PFAST, LayoutB<L, P>, LayoutA<L, P, true>>::type;
+using PipeLayout = typename std::conditional<PFAST && P >= 2, LayoutB<L, P>, LayoutA<L, P, true>>::type;
 
 // Start the asynchronous load of the tile at pencil q0 (one cp.async group is
 // committed by the caller).
@@ -1229,7 +1242,7 @@ __device__ __forceinline__ void pipe_tile(cx_t<T>* sm, cx_t<T>* chat, const Pass
 }
 
 template <typename T, int L, int P, int NT, int SIGN, int MODE, bool PFAST>
-__global__ void __launch_bounds__(NT, PipeOcc<T, L, MODE, PFAST>::value) fft_pass_pipe_kernel(PassParams<T> a) {
+__global__ void __launch_bounds__(NT, PipeOcc<T, L, MODE, PFAST, NT>::value) fft_pass_pipe_kernel(PassParams<T> a) {
     using C = cx_t<T>;
     using LY = PipeLayout<L, P, PFAST>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1310,6 +1323,7 @@ template <typename T, int L, int P, int NT, class LY> struct ChainMid {
         cb = f.c_hat + ((long long)u.o * a.osO + (long long)(u.i0 + p) * a.osI);
         osJ = (int)a.osJ;
     }
+    __device__ __forceinline__ void begin(int, int) {}
     __device__ __forceinline__ C operator()(int p, int m, C gv) {
         const C c = cs[LY::idx(p, m)];
         const int bp = (int)f.fd_bp.div((uint32_t)m);

@@ -105,6 +105,8 @@ __device__ __forceinline__ void issue_herm_mirror(cx_t<T>* smb, const PassParams
 
 // (direct + conj(mirror)) / 2 of element m of pencil p
 template <typename T, int L, int P, class LY> struct HermIn {
+    static constexpr bool EXT = false;   // the mirror buffer is refilled after the stage's barrier
+    __device__ __forceinline__ void before_write() const {}
     const cx_t<T>* a;
     const cx_t<T>* b;
     __device__ __forceinline__ cx_t<T> operator()(int p, int m) const {
@@ -169,6 +171,7 @@ __global__ void __launch_bounds__(NT, 2) fft_herm_inv_kernel(PassParams<T> a) {
 // G1[k] = (W[k] + conj W[-k]) / 2, G2[k] = (W[k] - conj W[-k]) / (2i), k <= N2/2.
 template <typename T> struct ChNlPairMid {
     T scale, msum;
+    __device__ __forceinline__ void begin(int, int) {}
     __device__ __forceinline__ cx_t<T> operator()(int, int, cx_t<T> x) {
         const T c0 = mul_rn(x.x, scale), c1 = mul_rn(x.y, scale);
         msum += c0 + c1;
@@ -193,6 +196,8 @@ template <typename T, int L, class LY> struct SmemOut {
 // 2 pp and 2 pp + 1, extended past N2/2 by conjugate symmetry (with r2c, the
 // imaginary parts at k = 0 and N2/2 dropped).
 template <typename T, int L> struct PairPackIn {
+    static constexpr bool EXT = false;
+    __device__ __forceinline__ void before_write() const {}
     const cx_t<T>* rw;
     int nhp;
     bool r2c;

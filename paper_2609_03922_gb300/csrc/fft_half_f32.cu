@@ -54,11 +54,9 @@ template <int L> static bool pick_pair(KernelInfo* ki) {
     return true;
 }
 
-// real rows per tile of the x pass (two rows per transform pencil)
-template <int N2> struct NlHalfRows { static constexpr int value = N2 <= 256 ? 4096 / N2 : 16; };
-
+// the x pass of the lengths without a kernel of two pencils per thread
 template <int N2> static bool pick_x(int nhp, KernelInfo* ki) {
-    constexpr int P = NlHalfRows<N2>::value, NT = N2 <= 256 ? 128 : 256;
+    constexpr int P = 16, NT = 256;   // real rows per tile (two rows per transform pencil)
     ki->P = P;
     ki->NT = NT;
     ki->pipe = true;
@@ -69,14 +67,7 @@ template <int N2> static bool pick_x(int nhp, KernelInfo* ki) {
 
 bool get_half_kernel(int64_t L, int mode, int nhp, KernelInfo* ki) {
     if (mode == PASS_NL_HALF) {   // L = N2, the full row length
-        switch (L) {
-            case 64: return pick_x<64>(nhp, ki);
-            case 128: return pick_x<128>(nhp, ki);
-            case 256: return pick_x<256>(nhp, ki);
-            case 384: return pick_x<384>(nhp, ki);
-            case 512: return pick_x<512>(nhp, ki);
-            default: return false;
-        }
+        return L == 512 ? pick_x<512>(nhp, ki) : get_nl_half2_kernel(L, nhp, ki);
     }
     if (mode == PASS_PAIR_MIRROR) {
         switch (L) {

@@ -28,6 +28,8 @@ namespace spdba {
 
 // (direct + conj(mirror)) / 2 of element m of pencil p, from the tensor-box tiles
 template <int L, int P> struct HermInBox {
+    static constexpr bool EXT = false;
+    __device__ __forceinline__ void before_write() const {}
     const float2* a;    // direct tile, row-major [z][p]
     const float2* b;    // mirror tile, [z][P + 2]
     const float2* c;    // kx = 0 columns of row -ky, [z][2] (tiles with kx0 = 0)

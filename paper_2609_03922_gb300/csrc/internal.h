@@ -11,6 +11,7 @@
 #include "fft_core.cuh"
 
 namespace spdba {
+struct KernelInfo;
 
 // ------------------------------------------------------------------ errors
 void set_error(const char* fmt, ...);
@@ -56,12 +57,18 @@ template <typename T> struct Pass {
     PassParams<T> p{};
 };
 
-// Build a pass of length L over pencils (O, I) with the given strides.
+// Build a pass of length L over pencils (O, I) with the given strides; fourstep: the
+// caller adds four-step twiddles.
 template <typename T>
 spdba_status make_pass(Pass<T>* out, int64_t L, int sign, int mode, long long O, long long I,
                        long long isO, long long isI, long long isJ, long long osO, long long osI,
-                       long long osJ, TwiddleCache<T>& tw, cudaStream_t st);
+                       long long osJ, TwiddleCache<T>& tw, cudaStream_t st, bool fourstep = false);
 template <typename T> spdba_status launch_pass(const Pass<T>& ps, const void* in, void* out, cudaStream_t st);
+
+// Puts another kernel under a pass (same pencils, one CTA per tile).
+spdba_status set_pass_kernel(Pass<float>* ps, const KernelInfo& ki);
+// Element step of the last stage of the two-pencil step chain of length L.
+int chain2_step(int64_t L);
 
 // A complete transform: list of passes (forward and inverse), scratch for the
 // out-of-place four-step second pass.
@@ -94,8 +101,6 @@ spdba_status launch_half_col_live(const Geom& g, const uint8_t* states, int N2, 
                                   cudaStream_t st);
 // Tiles of a paired z forward pass.
 long long pair_tile_count(const Pass<float>& ps);
-// Pencils per tile of the pass kernels of length L (0 if none).
-template <typename T> int pass_tile_pencils(int64_t L);
 
 // ------------------------------------------------------------------ TMA z inverse
 // The Hermitian z inverse of the half-spectrum form with its tiles moved as

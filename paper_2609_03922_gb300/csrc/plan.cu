@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "blocks.h"
+#include "kernel_table.h"
 #include "nls.h"
 #include "rcd.h"
 
@@ -431,8 +432,23 @@ static spdba_status setup_chain(spdba_plan* p, Group<T>& r, int ndim, const int6
     if (s == SPDBA_ERR_UNSUPPORTED) return SPDBA_OK;
     if (s != SPDBA_OK) return s;
     const int64_t bpass = ndim == 3 ? r.g.b[0] : r.g.b[1];
+    if constexpr (std::is_same<T, float>::value) {
+        // two pencils per thread: blocks of an even edge along the rows, and of an edge along
+        // the pass axis that divides the last stage's element step
+        KernelInfo k2;
+        if (get_chain2_kernel(d[0], c.P < 8, &k2) && r.g.b[2] % 2 == 0 && d[ndim - 1] % k2.P == 0 &&
+            chain2_step(d[0]) % bpass == 0) {
+            if ((s = set_pass_kernel(&c, k2)) != SPDBA_OK) return s;
+        }
+    }
     if (d[ndim - 1] % c.P != 0 || (d[0] / bpass) * (int64_t)upd_table_cols(c.P, r.g.b[2]) > kUpdTable) return SPDBA_OK;
     fill_fuse<T>(p, r, c.p.fu);
+    // c_hat past the L2 where the workspace fits it but not both
+    int l2 = 0, dev = 0;
+    SPDBA_CUDA(cudaGetDevice(&dev));
+    SPDBA_CUDA(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
+    const long long field = (long long)sizeof(cx_t<T>) * c.p.O * c.p.I * d[0];
+    c.p.stream_chat = field <= l2 && 2 * field > l2;
     r.chain = c;
     r.has_chain = true;
     return SPDBA_OK;
@@ -444,9 +460,11 @@ static spdba_status setup_half(spdba_plan* p, Group<float>& r, const int64_t* di
     cudaStream_t st = p->st;
     const int64_t N0 = dims[0], N1 = dims[1], N2 = dims[2];
     if (N2 % 2 != 0 || N0 > 4096 || N1 > 4096 || N2 > 4096) return SPDBA_ERR_UNSUPPORTED;
-    const int Py = pass_tile_pencils<float>(N1);
-    if (Py == 0) return SPDBA_ERR_UNSUPPORTED;
+    if (!tile_length_supported(N1)) return SPDBA_ERR_UNSUPPORTED;
     const int64_t M = N2 / 2;
+    // rows of whole y pass tiles (16 pencils), and of whole tiles of the z passes
+    // for cubes of 128 and below, whose z tiles are wider
+    const int Py = N1 <= 128 ? (int)(4096 / N1) : 16;
     const int64_t NHP = ((M + 1 + Py - 1) / Py) * Py;
     if (4 * NHP > 3 * N2) return SPDBA_ERR_UNSUPPORTED;   // under a quarter saved: keep the full form
     HalfGeo hg;
@@ -525,8 +543,8 @@ static spdba_status group_init_ch_hs(spdba_plan* p, Group<float>& r, const int64
     if (B2 < 1 || N2 % (2 * B2) != 0)
         return fail(SPDBA_ERR_UNSUPPORTED, "half-spectrum storage needs 2 B2 | N2 (B2 = %d, N2 = %lld)", B2,
                     (long long)N2);
-    const int Py = pass_tile_pencils<float>(N1);
-    if (Py == 0) return fail(SPDBA_ERR_UNSUPPORTED, "no y pass for %lld points", (long long)N1);
+    if (!tile_length_supported(N1)) return fail(SPDBA_ERR_UNSUPPORTED, "no y pass for %lld points", (long long)N1);
+    const int Py = 16;             // pencils of a wide tile
     int64_t q = Py;
     while (q % B2 != 0) q += Py;   // a multiple of both
     const int64_t M = N2 / 2;
