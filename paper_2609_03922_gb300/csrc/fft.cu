@@ -71,6 +71,7 @@ bool tile_length_supported(int64_t L) {
 
 // ------------------------------------------------------------------ twiddles
 template <typename T> __global__ void twiddle_kernel(cx_t<T>* t, long long n) {
+    pdl_wait();
     long long m = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (m < n) {
         double s, c;
@@ -85,7 +86,7 @@ template <typename T> cx_t<T>* TwiddleCache<T>::get(int64_t n, cudaStream_t st, 
     cx_t<T>* p = nullptr;
     cudaError_t e = dev_alloc((void**)&p, sizeof(cx_t<T>) * (size_t)n);
     if (e != cudaSuccess) { *err = cuda_fail(e, "device allocation (twiddle table)"); return nullptr; }
-    twiddle_kernel<T><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(p, (long long)n);
+    pdl_launch(twiddle_kernel<T>, (unsigned)((n + 255) / 256), 256, 0, st, p, (long long)n);
     e = cudaGetLastError();
     if (e != cudaSuccess) { dev_free(p); *err = cuda_fail(e, "twiddle_kernel"); return nullptr; }
     tables[n] = p;
@@ -199,7 +200,7 @@ template <typename T> spdba_status launch_pass(const Pass<T>& ps, const void* in
     p.in = reinterpret_cast<const cx_t<T>*>(in);
     p.out = reinterpret_cast<cx_t<T>*>(out);
     void* args[] = {&p};
-    SPDBA_CUDA(cudaLaunchKernel(ps.func, dim3((unsigned)ps.grid), dim3(ps.nt), args, (size_t)ps.smem, st));
+    SPDBA_CUDA(pdl_launch_ptr(ps.func, dim3((unsigned)ps.grid), dim3(ps.nt), args, (size_t)ps.smem, st));
     return SPDBA_OK;
 }
 

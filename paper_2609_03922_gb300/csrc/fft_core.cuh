@@ -1136,6 +1136,7 @@ __device__ __forceinline__ void tile_body(cx_t<T>* sm, const PassParams<T>& a, l
 // (generic addressing) and the transposing store of the four-step second pass.
 template <typename T, int L, int P, int NT, int SIGN, int MODE, bool LOADP, bool STOREP>
 __global__ void __launch_bounds__(NT) fft_pass_kernel(PassParams<T> a) {
+    pdl_wait();
     using C = cx_t<T>;
     using LY = LayoutA<L, P, true>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1243,6 +1244,7 @@ __device__ __forceinline__ void pipe_tile(cx_t<T>* sm, cx_t<T>* chat, const Pass
 
 template <typename T, int L, int P, int NT, int SIGN, int MODE, bool PFAST>
 __global__ void __launch_bounds__(NT, PipeOcc<T, L, MODE, PFAST, NT>::value) fft_pass_pipe_kernel(PassParams<T> a) {
+    pdl_wait();
     using C = cx_t<T>;
     using LY = PipeLayout<L, P, PFAST>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1350,6 +1352,7 @@ template <typename T, int L, int NT> struct ChainOcc {
 
 template <typename T, int L, int P, int NT>
 __global__ void __launch_bounds__(NT, ChainOcc<T, L, NT>::value) fft_chain_kernel(PassParams<T> a) {
+    pdl_wait();
     using C = cx_t<T>;
     using LY = PipeLayout<L, P, true>;
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -88,6 +88,7 @@ template <int L> struct GlobalPairOut {
 // 384 points over 384 x 384 x 208: 143 us (8-pencil tiles) and 87 us.
 template <int L, int P, int NT, int SIGN, int OCC>
 __global__ void __launch_bounds__(NT, OCC) fft_pipe2_kernel(PassParams<float> a) {
+    pdl_wait();
     constexpr int H = P / 2;
     using LY = LayoutB<L, H>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -217,6 +218,7 @@ template <int L, int H, int Q> struct ChainMid2 {
 
 template <int L, int P, int NT, int OCC>
 __global__ void __launch_bounds__(NT, OCC) fft_chain2_kernel(PassParams<float> a) {
+    pdl_wait();
     constexpr int H = P / 2;
     using LY = LayoutB<L, H>;
     static_assert(NT % H == 0, "each thread keeps one pencil pair");
@@ -302,6 +304,7 @@ template <int L> struct RowPairOut {
 // nonlinear 70.2 -> 60.1, 455 -> 285, 10.0 -> 7.5 us.
 template <int L, int P, int NT, int SIGN, int MODE, int OCC>
 __global__ void __launch_bounds__(NT, OCC) fft_rows2_kernel(PassParams<float> a) {
+    pdl_wait();
     constexpr int H = P / 2;
     using LY = RowLayout<L, H>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -373,6 +376,7 @@ template <int L, class LY> struct SmemOut2 {
 // them); else the packed elements are read from global memory, each row twice.
 template <int L, int P, int NT, int OCC, bool ST>
 __global__ void __launch_bounds__(NT, OCC) fft_nl_half2_kernel(PassParams<float> a) {
+    pdl_wait();
     constexpr int H = P / 4, M = L / 2;
     using LY = RowLayout<L, H>;
     extern __shared__ __align__(16) unsigned char smem_raw[];

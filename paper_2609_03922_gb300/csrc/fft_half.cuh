@@ -117,6 +117,7 @@ template <typename T, int L, int P, class LY> struct HermIn {
 
 template <typename T, int L, int P, int NT>
 __global__ void __launch_bounds__(NT, 2) fft_herm_inv_kernel(PassParams<T> a) {
+    pdl_wait();
     using C = cx_t<T>;
     using LY = LayoutB<L, P>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -223,6 +224,7 @@ template <typename T, int L> struct PairPackIn {
 // rows of NHP entries.  a.tw: stage twiddles of N2.
 template <typename T, int L, int P, int NT>
 __global__ void __launch_bounds__(NT, L == 384 ? 1 : 512 / NT) fft_nl_half_kernel(PassParams<T> a) {
+    pdl_wait();
     using C = cx_t<T>;
     constexpr int PP = P / 2;
     constexpr int M = L / 2;
@@ -389,6 +391,7 @@ __device__ __forceinline__ bool pair_live(const PassParams<T>& a, bool masked, i
 // to its CTAs (liveness clusters in the spectrum).
 template <typename T, int P>
 __global__ void __launch_bounds__(256) pair_live_list_kernel(PassParams<T> a, int* list, int* count) {
+    pdl_wait();
     const int ntm = a.hg.N1 * (a.hg.N2 >> 1) / P, nt = ntm + a.hg.N1 / P;
     const int t = (int)(blockIdx.x * 8 + (threadIdx.x >> 5));
     if (t >= nt) return;   // warp-uniform
@@ -509,6 +512,7 @@ __device__ __forceinline__ void pair_column(const cx_t<T>* sm, const PassParams<
 constexpr int kPairBufs = 3;
 template <typename T, int L, int P, int NT>
 __global__ void __launch_bounds__(NT, 512 / NT) fft_pair_kernel(PassParams<T> a) {
+    pdl_wait();
     using C = cx_t<T>;
     using LY = LayoutBP<L, P>;
     static_assert(NT % P == 0 && NT % (P / 2) == 0, "each thread keeps one pencil");

@@ -97,8 +97,8 @@ spdba_status launch_pair_live_list(const Pass<float>& ps, int* list, int* count,
     const unsigned grid = (unsigned)((nt + 7) / 8);   // a warp per tile, 8 per CTA
     SPDBA_CUDA(cudaMemsetAsync(count, 0, sizeof(int), st));
     switch (ps.P) {
-        case 8: pair_live_list_kernel<float, 8><<<grid, 256, 0, st>>>(ps.p, list, count); break;
-        case 16: pair_live_list_kernel<float, 16><<<grid, 256, 0, st>>>(ps.p, list, count); break;
+        case 8: pdl_launch(pair_live_list_kernel<float, 8>, grid, 256, 0, st, ps.p, list, count); break;
+        case 16: pdl_launch(pair_live_list_kernel<float, 16>, grid, 256, 0, st, ps.p, list, count); break;
         default: return SPDBA_ERR_UNSUPPORTED;
     }
     SPDBA_CUDA(cudaGetLastError());
@@ -115,6 +115,7 @@ namespace spdba {
 // are never read.
 __global__ void __launch_bounds__(1024) half_col_live_kernel(const uint8_t* __restrict__ states, int nrows, int nb2,
                                                              int B2, int N2, int NHP, uint8_t* __restrict__ col_live) {
+    pdl_wait();
     __shared__ uint8_t s_col[64];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int bx = warp; bx < nb2; bx += 32) {
@@ -141,6 +142,7 @@ __global__ void __launch_bounds__(1024) half_col_live_kernel(const uint8_t* __re
 __global__ void __launch_bounds__(256) hs_live_kernel(const uint8_t* __restrict__ states, int nb0, int nb1, int nb2,
                                                       int B1, int B2, int N1, int NHP, uint8_t* __restrict__ zlive,
                                                       uint8_t* __restrict__ xlive) {
+    pdl_wait();
     const long long n = (long long)N1 * NHP;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const int y = (int)(i / NHP), x = (int)(i - (long long)y * NHP);
@@ -157,7 +159,7 @@ spdba_status launch_hs_live(const Geom& g, const uint8_t* states, uint8_t* zlive
     const long long n = g.n[1] * g.n[2];
     SPDBA_CUDA(cudaMemsetAsync(xlive, 0, (size_t)g.n[2], st));
     const long long grid = std::min<long long>((n + 255) / 256, 152 * 8);
-    hs_live_kernel<<<(unsigned)grid, 256, 0, st>>>(states, (int)g.nb[0], (int)g.nb[1], (int)g.nb[2], g.b[1], g.b[2],
+    pdl_launch(hs_live_kernel, (unsigned)grid, 256, 0, st, states, (int)g.nb[0], (int)g.nb[1], (int)g.nb[2], g.b[1], g.b[2],
                                                    (int)g.n[1], (int)g.n[2], zlive, xlive);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
@@ -166,7 +168,7 @@ spdba_status launch_hs_live(const Geom& g, const uint8_t* states, uint8_t* zlive
 spdba_status launch_half_col_live(const Geom& g, const uint8_t* states, int N2, int NHP, uint8_t* col_live,
                                   cudaStream_t st) {
     if (g.nb[2] > 64) return fail(SPDBA_ERR_UNSUPPORTED, "more than 64 block columns");
-    half_col_live_kernel<<<1, 1024, 0, st>>>(states, (int)(g.nb[0] * g.nb[1]), (int)g.nb[2], g.b[2], N2, NHP,
+    pdl_launch(half_col_live_kernel, 1, 1024, 0, st, states, (int)(g.nb[0] * g.nb[1]), (int)g.nb[2], g.b[2], N2, NHP,
                                              col_live);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;

@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(NT, 2)
     fft_herm_inv_tma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                             const __grid_constant__ CUtensorMap map_c, PassParams<float> a,
                             unsigned long long* timeouts, long long spin_limit, int stall) {
+    pdl_wait();
     using C = float2;
     using LY = LayoutB<L, P>;
     constexpr int ZB = L <= 256 ? L : L / 2;   // z extent of one box
@@ -221,7 +222,7 @@ spdba_status launch_herm_inv_tma(const HermTma& ht, const Pass<float>& zinv, con
     long long spin = wait_limit();
     int stall = stall_waits();
     void* args[] = {(void*)&ht.map[0], (void*)&ht.map[1], (void*)&ht.map[2], &p, &timeouts, &spin, &stall};
-    SPDBA_CUDA(cudaLaunchKernel(ht.func, dim3((unsigned)ht.grid), dim3(kHermTmaNT), args, ht.smem, st));
+    SPDBA_CUDA(pdl_launch_ptr(ht.func, dim3((unsigned)ht.grid), dim3(kHermTmaNT), args, ht.smem, st));
     return SPDBA_OK;
 }
 

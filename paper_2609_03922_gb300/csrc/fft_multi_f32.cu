@@ -75,6 +75,7 @@ template <typename T, int TILE, int SIGN, int MODE, bool PFAST>
 __global__ void __launch_bounds__(kMultiNT, MultiOcc<MODE>::value)
     fft_multi_kernel(const MultiGroup<T>* __restrict__ gs, int ng, unsigned total, unsigned dense_mask,
                      unsigned mass_mask) {
+    pdl_wait();
     using C = cx_t<T>;
     constexpr int NT = kMultiNT;
     constexpr int BUF = MultiBuf<TILE, PFAST>::SIZE;
@@ -212,7 +213,7 @@ spdba_status launch_multi(const void* func, int smem, long long grid, const Mult
                           unsigned total, unsigned dense_mask, unsigned mass_mask, cudaStream_t st) {
     if (total == 0 || grid < 1) return SPDBA_OK;
     void* args[] = {&groups, &ng, &total, &dense_mask, &mass_mask};
-    SPDBA_CUDA(cudaLaunchKernel(func, dim3((unsigned)grid), dim3(kMultiNT), args, (size_t)smem, st));
+    SPDBA_CUDA(pdl_launch_ptr(func, dim3((unsigned)grid), dim3(kMultiNT), args, (size_t)smem, st));
     return SPDBA_OK;
 }
 

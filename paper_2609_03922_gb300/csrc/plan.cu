@@ -23,6 +23,7 @@ namespace spdba {
 
 // ------------------------------------------------------------------ small kernels
 template <typename T> __global__ void real_to_complex_kernel(const T* __restrict__ r, cx_t<T>* __restrict__ c, long long n) {
+    pdl_wait();
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         c[i] = mk<cx_t<T>>(r[i], (T)0);
 }
@@ -31,6 +32,7 @@ template <typename T> __global__ void real_to_complex_kernel(const T* __restrict
 template <typename T>
 __global__ void half_storage_extend_kernel(const cx_t<T>* __restrict__ h, cx_t<T>* __restrict__ full, int N0, int N1,
                                            int N2, int NHP) {
+    pdl_wait();
     const long long n = (long long)N0 * N1 * N2;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(i % N2);
@@ -49,14 +51,17 @@ __global__ void half_storage_extend_kernel(const cx_t<T>* __restrict__ h, cx_t<T
 }
 
 template <typename T> __global__ void complex_real_part_kernel(const cx_t<T>* __restrict__ c, T* __restrict__ r, long long n) {
+    pdl_wait();
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         r[i] = c[i].x;
 }
 __global__ void zero_strided_kernel(double* p, long long n, int stride) {
+    pdl_wait();
     for (long long i = threadIdx.x; i < n; i += blockDim.x) p[i * stride] = 0.0;
 }
 // per-run share of non-frozen blocks for one step (1 on all-active steps)
 __global__ void ratio_kernel(DevStats* stats, long long nruns, long long bpr, long long bmodes, int dense) {
+    pdl_wait();
     for (long long r = threadIdx.x; r < nruns; r += blockDim.x) {
         double nf = dense ? (double)bpr : (double)(stats[r].n_active + stats[r].n_transition);
         stats[r].ratio_sum += nf / (double)bpr;
@@ -69,6 +74,7 @@ __global__ void ratio_kernel(DevStats* stats, long long nruns, long long bpr, lo
 }
 // Statistics of runs [0, n) reset, with the threshold coefficient in force set to eps.
 __global__ void stats_reset_kernel(DevStats* stats, long long n, double eps) {
+    pdl_wait();
     for (long long r = threadIdx.x; r < n; r += blockDim.x) {
         stats[r] = DevStats{};
         stats[r].eps = eps;
@@ -91,6 +97,7 @@ __device__ __forceinline__ double control_decision(double eps, double r, double 
 // rounding in the quotient); the interval restarts.  Runs without an adaptive
 // step in the interval keep their coefficient.
 __global__ void control_kernel(DevStats* stats, long long nruns, long long bpr, double r_tar, double eta) {
+    pdl_wait();
     for (long long r = threadIdx.x; r < nruns; r += blockDim.x) {
         DevStats& s = stats[r];
         if (s.ctl_steps == 0) continue;
@@ -396,7 +403,7 @@ template <typename T> static spdba_status group_buffers(spdba_plan* p, Group<T>&
     if ((s = r.alloc(&r.scratch, classify_scratch_bytes(nb))) != SPDBA_OK) return s;
     if ((s = r.alloc(&r.stats, sizeof(DevStats) * r.batch)) != SPDBA_OK) return s;
     SPDBA_CUDA(cudaMemsetAsync(r.c_hat, 0, sizeof(cx_t<T>) * tot, st));
-    stats_reset_kernel<<<1, 256, 0, st>>>(r.stats, r.batch, p->threshold);
+    pdl_launch(stats_reset_kernel, 1, 256, 0, st, r.stats, r.batch, p->threshold);
     SPDBA_CUDA(cudaGetLastError());
     SPDBA_CUDA(cudaMemsetAsync(r.gmax, 0, sizeof(double) * 2 * r.batch, st));
     SPDBA_CUDA(cudaMemsetAsync(r.states, SPDBA_ACTIVE, nb, st));
@@ -840,13 +847,14 @@ template <typename T> static spdba_status group_assess(spdba_plan* p, Group<T>& 
 // blocks the exact states mark non-frozen while the prediction in force had them frozen
 __global__ void missed_kernel(const uint8_t* __restrict__ exact, const uint8_t* __restrict__ pred, long long nb,
                               DevStats* stats) {
+    pdl_wait();
     unsigned long long c = 0;
     for (long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x; b < nb; b += (long long)gridDim.x * blockDim.x)
         c += (exact[b] != 0 && pred[b] == 0) ? 1ull : 0ull;
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(&stats->missed, c);
 }
-__global__ void count_prediction_kernel(DevStats* stats) { stats->predictions += 1; }
+__global__ void count_prediction_kernel(DevStats* stats) { pdl_wait(); stats->predictions += 1; }
 
 // Reassessment with an attached predictor (3-D CH, one run): exact judge or prediction.
 template <typename T> static spdba_status group_assess_predicted(spdba_plan* p, Group<T>& r) {
@@ -857,7 +865,7 @@ template <typename T> static spdba_status group_assess_predicted(spdba_plan* p, 
     if (judge) {
         if ((s = group_assess<T>(p, r)) != SPDBA_OK) return s;
         if (r.has_pred) {
-            missed_kernel<<<grid_for(nb, 256), 256, 0, st>>>(r.states, r.pstates, nb, r.stats);
+            pdl_launch(missed_kernel, grid_for(nb, 256), 256, 0, st, r.states, r.pstates, nb, r.stats);
             p->launches += 1;
         }
         SPDBA_CUDA(cudaMemcpyAsync(r.snap_maxsq, r.maxsq, sizeof(double) * nb, cudaMemcpyDeviceToDevice, st));
@@ -874,7 +882,7 @@ template <typename T> static spdba_status group_assess_predicted(spdba_plan* p, 
                              r.chi, r.list, r.count, r.scratch, r.stats, st)) != SPDBA_OK)
         return s;
     SPDBA_CUDA(cudaMemcpyAsync(r.pstates, r.states, nb, cudaMemcpyDeviceToDevice, st));
-    count_prediction_kernel<<<1, 1, 0, st>>>(r.stats);
+    pdl_launch(count_prediction_kernel, 1, 1, 0, st, r.stats);
     p->launches += 10;
     r.has_pred = true;
     r.assessed = true;
@@ -896,7 +904,7 @@ static bool all_active_step(const spdba_plan* p, int64_t step) {
 
 // The control decision of a group's runs, before the step's reassessment.
 template <typename T> static spdba_status group_control(spdba_plan* p, Group<T>& r) {
-    control_kernel<<<1, 256, 0, p->st>>>(r.stats, r.batch, r.g.live_bpr(), p->opt.target_ratio, p->opt.control_eta);
+    pdl_launch(control_kernel, 1, 256, 0, p->st, r.stats, r.batch, r.g.live_bpr(), p->opt.target_ratio, p->opt.control_eta);
     SPDBA_CUDA(cudaGetLastError());
     p->launches += 1;
     return SPDBA_OK;
@@ -972,7 +980,7 @@ template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>&
         Pass<T> nl = r.h_nl;
         if (reassess) {
             nl.p.mass = &r.stats[0].mass;
-            zero_strided_kernel<<<1, 256, 0, st>>>(&r.stats[0].mass, r.batch, nl.p.mass_stride);
+            pdl_launch(zero_strided_kernel, 1, 256, 0, st, &r.stats[0].mass, r.batch, nl.p.mass_stride);
             p->launches += 1;
         }
         {
@@ -1030,7 +1038,7 @@ template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>&
         Pass<T> nl = r.h_nl;
         if (reassess) {
             nl.p.mass = &r.stats[0].mass;
-            zero_strided_kernel<<<1, 256, 0, st>>>(&r.stats[0].mass, r.batch, nl.p.mass_stride);
+            pdl_launch(zero_strided_kernel, 1, 256, 0, st, &r.stats[0].mass, r.batch, nl.p.mass_stride);
             p->launches += 1;
         }
         {
@@ -1083,7 +1091,7 @@ template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>&
     Pass<T> fused = r.fused;
     if (reassess) {
         fused.p.mass = &r.stats[0].mass;
-        zero_strided_kernel<<<1, 256, 0, st>>>(&r.stats[0].mass, r.batch, fused.p.mass_stride);
+        pdl_launch(zero_strided_kernel, 1, 256, 0, st, &r.stats[0].mass, r.batch, fused.p.mass_stride);
         p->launches += 1;
     }
     {
@@ -1211,21 +1219,21 @@ template <typename T> static spdba_status group_nls_steps(spdba_plan* p, Group<T
             NLSArgs<T> c = a;
             c.tw = r.tw_col;
             if (reassess) {
-                zero_strided_kernel<<<1, 256, 0, st>>>(&r.stats[0].mass, r.batch, a.power_stride);
+                pdl_launch(zero_strided_kernel, 1, 256, 0, st, &r.stats[0].mass, r.batch, a.power_stride);
                 c.power = &r.stats[0].mass;
             }
             if ((s = col_pass<T>(p, r, c, 1, 1, 1)) != SPDBA_OK) return s;
         } else {
             if (reassess && (s = group_assess<T>(p, r)) != SPDBA_OK) return s;
             if (reassess) {
-                zero_strided_kernel<<<1, 256, 0, st>>>(&r.stats[0].mass, r.batch, a.power_stride);
+                pdl_launch(zero_strided_kernel, 1, 256, 0, st, &r.stats[0].mass, r.batch, a.power_stride);
                 a.power = &r.stats[0].mass;
             }
             ProfScope pr(p, K_NLS_STEP, 2.0 * sizeof(cx_t<T>) * (double)(r.batch * r.n));
             if ((s = nls_small_step<T>(a, r.nl, st)) != SPDBA_OK) return s;
             p->launches += 1;
         }
-        ratio_kernel<<<1, 256, 0, st>>>(r.stats, r.batch, r.g.bpr(), r.g.block_modes(), dense);
+        pdl_launch(ratio_kernel, 1, 256, 0, st, r.stats, r.batch, r.g.bpr(), r.g.block_modes(), dense);
         SPDBA_CUDA(cudaGetLastError());
         p->launches += 1;
         prev_dense = dense;
@@ -1382,7 +1390,7 @@ static spdba_status multi_ch_step(spdba_plan* p, const MultiForm& mf) {
         if (control_step(p, r.step) && (s = group_control<float>(p, r)) != SPDBA_OK) return s;
         if (reassess) {
             if ((s = group_assess<float>(p, r)) != SPDBA_OK) return s;
-            zero_strided_kernel<<<1, 256, 0, st>>>(&r.stats[0].mass, r.batch, r.fused.p.mass_stride);
+            pdl_launch(zero_strided_kernel, 1, 256, 0, st, &r.stats[0].mass, r.batch, r.fused.p.mass_stride);
             p->launches += 1;
             mass_mask |= 1u << i;
         }
@@ -1582,11 +1590,11 @@ static spdba_status run_set_field(spdba_plan* p, Group<T>& r, long long sub, con
     if (p->opt.model == SPDBA_MODEL_RCD) {
         const long long tot = r.n * r.ncomp;
         SPDBA_CUDA(cudaMemcpyAsync(r.real, src, sizeof(T) * tot, kind, st));
-        real_to_complex_kernel<T><<<grid_for(tot, 256), 256, 0, st>>>(r.real, r.work, tot);
+        pdl_launch(real_to_complex_kernel<T>, grid_for(tot, 256), 256, 0, st, r.real, r.work, tot);
         if ((s = r.rcd_fft.exec(r.work, r.c_hat, SPDBA_FORWARD, st)) != SPDBA_OK) return s;
     } else if (p->opt.model == SPDBA_MODEL_CH) {
         SPDBA_CUDA(cudaMemcpyAsync(r.real, src, sizeof(T) * r.n, kind, st));
-        real_to_complex_kernel<T><<<grid_for(r.n, 256), 256, 0, st>>>(r.real, wslot, r.n);
+        pdl_launch(real_to_complex_kernel<T>, grid_for(r.n, 256), 256, 0, st, r.real, wslot, r.n);
         if ((s = r.fft1.exec(wslot, slot, SPDBA_FORWARD, st)) != SPDBA_OK) return s;
         if (r.hs) {
             // keep the half kx = 0 .. N2/2 of the full spectrum, rows padded with zeros
@@ -1616,7 +1624,7 @@ static spdba_status run_set_field(spdba_plan* p, Group<T>& r, long long sub, con
     r.assessed = false;
     r.has_snap = false;
     r.has_pred = false;
-    stats_reset_kernel<<<1, 32, 0, st>>>(r.stats + sub, 1, p->threshold);
+    pdl_launch(stats_reset_kernel, 1, 32, 0, st, r.stats + sub, 1, p->threshold);
     SPDBA_CUDA(cudaGetLastError());
     SPDBA_CUDA(cudaMemsetAsync(r.states + sub * r.g.bpr(), SPDBA_ACTIVE, r.g.bpr(), st));
     return SPDBA_OK;
@@ -1632,17 +1640,17 @@ static spdba_status run_get_field(spdba_plan* p, Group<T>& r, long long sub, voi
     if (p->opt.model == SPDBA_MODEL_RCD) {
         const long long tot = r.n * r.ncomp;
         if ((s = r.rcd_fft.exec(r.c_hat, r.work, SPDBA_INVERSE, st)) != SPDBA_OK) return s;
-        complex_real_part_kernel<T><<<grid_for(tot, 256), 256, 0, st>>>(r.work, r.real, tot);
+        pdl_launch(complex_real_part_kernel<T>, grid_for(tot, 256), 256, 0, st, r.work, r.real, tot);
         SPDBA_CUDA(cudaMemcpyAsync(dst, r.real, sizeof(T) * tot, kind, st));
     } else if (p->opt.model == SPDBA_MODEL_CH) {
         if (r.hs) {
-            half_storage_extend_kernel<T><<<grid_for(r.n, 256), 256, 0, st>>>(
+            pdl_launch(half_storage_extend_kernel<T>, grid_for(r.n, 256), 256, 0, st, 
                 r.c_hat, r.work, (int)r.dims[0], (int)r.dims[1], (int)r.dims[2], (int)r.hs_nhp);
             if ((s = r.fft1.exec(r.work, wslot, SPDBA_INVERSE, st)) != SPDBA_OK) return s;
         } else if ((s = r.fft1.exec(slot, wslot, SPDBA_INVERSE, st)) != SPDBA_OK) {
             return s;
         }
-        complex_real_part_kernel<T><<<grid_for(r.n, 256), 256, 0, st>>>(wslot, r.real, r.n);
+        pdl_launch(complex_real_part_kernel<T>, grid_for(r.n, 256), 256, 0, st, wslot, r.real, r.n);
         SPDBA_CUDA(cudaMemcpyAsync(dst, r.real, sizeof(T) * r.n, kind, st));
     } else if (!r.long_nls) {
         if ((s = r.fft1.exec(slot, wslot, SPDBA_INVERSE, st)) != SPDBA_OK) return s;

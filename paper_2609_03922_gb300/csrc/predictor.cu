@@ -156,6 +156,7 @@ __global__ void __launch_bounds__(128) conv_kernel(MapDims m, TileGrid tg, const
                                                    const bf16* __restrict__ Wt, const float* __restrict__ bias,
                                                    float* __restrict__ out_pre, const float* __restrict__ mask_pre,
                                                    bf16* __restrict__ out) {
+    pdl_wait();
     constexpr int K = 27 * CIN, KP = kpad(K), NT = COUT / 8, KC = KP / 16, VS = VoxStride<CIN>::value;
     __shared__ __align__(16) bf16 sX[kHalo * VS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
@@ -255,6 +256,7 @@ template <int CIN, int COUT>
 __global__ void __launch_bounds__(kWgNT) wgrad_kernel(MapDims m, TileGrid tg, const bf16* __restrict__ dA,
                                                       const bf16* __restrict__ X, float* __restrict__ dW,
                                                       float* __restrict__ dbias) {
+    pdl_wait();
     constexpr int K = 27 * CIN, VS = VoxStride<CIN>::value, DS = VoxStride<COUT>::value;
     constexpr int NACC = CIN == 2 ? 1 : 3 * CIN / 8;
     __shared__ __align__(16) bf16 sX[kHalo * VS];
@@ -361,6 +363,7 @@ __global__ void __launch_bounds__(kHeadNT) head_kernel(long long nvox, const bf1
                                                        const float* __restrict__ labels, double inv_n,
                                                        bf16* __restrict__ da3, float* __restrict__ grads,
                                                        double* __restrict__ loss) {
+    pdl_wait();
     const float* wh = params + OFF_WH;
     const float bh = params[OFF_BH];
     float gw[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -430,6 +433,7 @@ __global__ void __launch_bounds__(kHeadNT) head_kernel(long long nvox, const bf1
 // input-gradient layout Wd[ci][k'] (k' = tap'*COUT + co, tap' = 26 - tap).
 __global__ void convert_weights_kernel(const float* __restrict__ P, int off, int cin, int cout, bf16* __restrict__ Wt,
                                        bf16* __restrict__ Wd) {
+    pdl_wait();
     const int K = 27 * cin, KP = kpad(K), Kd = 27 * cout, KPd = kpad(Kd);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < cout * KP; i += gridDim.x * blockDim.x) {
         int co = i / KP, k = i % KP;
@@ -451,6 +455,7 @@ __global__ void convert_weights_kernel(const float* __restrict__ P, int off, int
 // x[v][0] = clamp(log10(A_B / tau) / 8, -1, 1), x[v][1] = 1 if the block is not FROZEN.
 __global__ void features_kernel(long long V, int nmaps, const double* __restrict__ maxsq, const double* __restrict__ tau,
                                 const uint8_t* __restrict__ states, bf16* __restrict__ x) {
+    pdl_wait();
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < V * nmaps;
          i += (long long)gridDim.x * blockDim.x) {
         const long long mp = i / V;
@@ -465,6 +470,7 @@ __global__ void features_kernel(long long V, int nmaps, const double* __restrict
 
 __global__ void adam_kernel(float* __restrict__ P, const float* __restrict__ G, float* __restrict__ M,
                             float* __restrict__ Vv, int n, float lr, float b1, float b2, float eps, float c1, float c2) {
+    pdl_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         float g = G[i];
         float m = b1 * M[i] + (1.f - b1) * g;
@@ -476,6 +482,7 @@ __global__ void adam_kernel(float* __restrict__ P, const float* __restrict__ G, 
 }
 
 __global__ void prob_to_measure_kernel(const float* __restrict__ p, double* __restrict__ out, long long n) {
+    pdl_wait();
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         out[i] = (double)p[i];
 }
@@ -511,9 +518,9 @@ static unsigned grid_of(long long n, int nt) {
 }
 
 static spdba_status refresh_weights(spdba_predictor* pr, cudaStream_t st) {
-    convert_weights_kernel<<<32, 256, 0, st>>>(pr->P, OFF_W1, 2, 8, pr->W1t, nullptr);
-    convert_weights_kernel<<<32, 256, 0, st>>>(pr->P, OFF_W2, 8, 16, pr->W2t, pr->W2d);
-    convert_weights_kernel<<<32, 256, 0, st>>>(pr->P, OFF_W3, 16, 8, pr->W3t, pr->W3d);
+    pdl_launch(convert_weights_kernel, 32, 256, 0, st, pr->P, OFF_W1, 2, 8, pr->W1t, nullptr);
+    pdl_launch(convert_weights_kernel, 32, 256, 0, st, pr->P, OFF_W2, 8, 16, pr->W2t, pr->W2d);
+    pdl_launch(convert_weights_kernel, 32, 256, 0, st, pr->P, OFF_W3, 16, 8, pr->W3t, pr->W3d);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
 }
@@ -522,11 +529,11 @@ static spdba_status refresh_weights(spdba_predictor* pr, cudaStream_t st) {
 static spdba_status forward(spdba_predictor* pr, const bf16* x, int nmaps, bool keep_pre, cudaStream_t st) {
     const TileGrid tg = tile_grid(pr->m, nmaps);
     const unsigned g = (unsigned)tg.tiles;
-    conv_kernel<2, 8, CONV_FWD><<<g, 128, 0, st>>>(pr->m, tg, x, pr->W1t, pr->P + OFF_B1,
+    pdl_launch(conv_kernel<2, 8, CONV_FWD>, g, 128, 0, st, pr->m, tg, x, pr->W1t, pr->P + OFF_B1,
                                                    keep_pre ? pr->a1 : nullptr, nullptr, pr->h1);
-    conv_kernel<8, 16, CONV_FWD><<<g, 128, 0, st>>>(pr->m, tg, pr->h1, pr->W2t, pr->P + OFF_B2,
+    pdl_launch(conv_kernel<8, 16, CONV_FWD>, g, 128, 0, st, pr->m, tg, pr->h1, pr->W2t, pr->P + OFF_B2,
                                                     keep_pre ? pr->a2 : nullptr, nullptr, pr->h2);
-    conv_kernel<16, 8, CONV_FWD><<<g, 128, 0, st>>>(pr->m, tg, pr->h2, pr->W3t, pr->P + OFF_B3,
+    pdl_launch(conv_kernel<16, 8, CONV_FWD>, g, 128, 0, st, pr->m, tg, pr->h2, pr->W3t, pr->P + OFF_B3,
                                                     keep_pre ? pr->a3 : nullptr, nullptr, pr->h3);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
@@ -538,7 +545,7 @@ template <int CIN, int COUT>
 static void wgrad(spdba_predictor* pr, const TileGrid& tg, const bf16* dA, const bf16* X, int offW, int offB,
                   cudaStream_t st) {
     const unsigned g = (unsigned)std::min<long long>(tg.tiles, 152 * 3);
-    wgrad_kernel<CIN, COUT><<<g, kWgNT, 0, st>>>(pr->m, tg, dA, X, pr->G + offW, pr->G + offB);
+    pdl_launch(wgrad_kernel<CIN, COUT>, g, kWgNT, 0, st, pr->m, tg, dA, X, pr->G + offW, pr->G + offB);
 }
 
 static spdba_status backward(spdba_predictor* pr, const bf16* x, const float* labels, int nmaps, cudaStream_t st) {
@@ -547,12 +554,12 @@ static spdba_status backward(spdba_predictor* pr, const bf16* x, const float* la
     const unsigned g = (unsigned)tg.tiles;
     SPDBA_CUDA(cudaMemsetAsync(pr->G, 0, sizeof(float) * NPARAM, st));
     SPDBA_CUDA(cudaMemsetAsync(pr->loss, 0, sizeof(double), st));
-    head_kernel<<<head_grid(nvox), kHeadNT, 0, st>>>(nvox, pr->h3, pr->a3, pr->P, pr->prob, labels,
-                                                     1.0 / (double)nvox, pr->da3, pr->G, pr->loss);
+    pdl_launch(head_kernel, head_grid(nvox), kHeadNT, 0, st, nvox, pr->h3, pr->a3, pr->P, pr->prob, labels,
+               1.0 / (double)nvox, pr->da3, pr->G, pr->loss);
     wgrad<16, 8>(pr, tg, pr->da3, pr->h2, OFF_W3, OFF_B3, st);
-    conv_kernel<8, 16, CONV_DGRAD><<<g, 128, 0, st>>>(pr->m, tg, pr->da3, pr->W3d, nullptr, nullptr, pr->a2, pr->da2);
+    pdl_launch(conv_kernel<8, 16, CONV_DGRAD>, g, 128, 0, st, pr->m, tg, pr->da3, pr->W3d, nullptr, nullptr, pr->a2, pr->da2);
     wgrad<8, 16>(pr, tg, pr->da2, pr->h1, OFF_W2, OFF_B2, st);
-    conv_kernel<16, 8, CONV_DGRAD><<<g, 128, 0, st>>>(pr->m, tg, pr->da2, pr->W2d, nullptr, nullptr, pr->a1, pr->da1);
+    pdl_launch(conv_kernel<16, 8, CONV_DGRAD>, g, 128, 0, st, pr->m, tg, pr->da2, pr->W2d, nullptr, nullptr, pr->a1, pr->da1);
     wgrad<2, 8>(pr, tg, pr->da1, x, OFF_W1, OFF_B1, st);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
@@ -642,8 +649,8 @@ extern "C" spdba_status spdba_predictor_features(spdba_predictor* pr, const doub
                                                  const uint8_t* states, int32_t nmaps, void* x_bf16, void* stream) {
     if (!pr || !maxsq || !tau || !states || !x_bf16 || nmaps < 1 || nmaps > pr->max_batch)
         return fail(SPDBA_ERR_ARG, "spdba_predictor_features: bad arguments");
-    features_kernel<<<grid_of(pr->m.V * nmaps, 256), 256, 0, (cudaStream_t)stream>>>(pr->m.V, nmaps, maxsq, tau, states,
-                                                                                      (bf16*)x_bf16);
+    pdl_launch(features_kernel, grid_of(pr->m.V * nmaps, 256), 256, 0, (cudaStream_t)stream, pr->m.V, nmaps, maxsq, tau,
+               states, (bf16*)x_bf16);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
 }
@@ -656,8 +663,8 @@ extern "C" spdba_status spdba_predictor_forward(spdba_predictor* pr, const void*
     const long long nvox = pr->m.V * nmaps;
     spdba_status s = forward(pr, (const bf16*)x_bf16, nmaps, false, st);
     if (s != SPDBA_OK) return s;
-    head_kernel<<<head_grid(nvox), kHeadNT, 0, st>>>(nvox, pr->h3, pr->a3, pr->P, prob, nullptr, 0.0, nullptr, nullptr,
-                                                    nullptr);
+    pdl_launch(head_kernel, head_grid(nvox), kHeadNT, 0, st, nvox, pr->h3, pr->a3, pr->P, prob, nullptr, 0.0, nullptr,
+               nullptr, nullptr);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
 }
@@ -686,7 +693,7 @@ extern "C" spdba_status spdba_predictor_train_step(spdba_predictor* pr, const vo
     pr->adam_t += 1;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f - powf(b1, (float)pr->adam_t), c2 = 1.f - powf(b2, (float)pr->adam_t);
-    adam_kernel<<<grid_of(NPARAM, 256), 256, 0, st>>>(pr->P, pr->G, pr->M, pr->Vv, NPARAM, lr, b1, b2, 1e-8f, c1, c2);
+    pdl_launch(adam_kernel, grid_of(NPARAM, 256), 256, 0, st, pr->P, pr->G, pr->M, pr->Vv, NPARAM, lr, b1, b2, 1e-8f, c1, c2);
     SPDBA_CUDA(cudaGetLastError());
     if ((s = refresh_weights(pr, st)) != SPDBA_OK) return s;
     if (loss_out) {
@@ -704,7 +711,7 @@ spdba_status spdba_predictor_states_internal(spdba_predictor* pr, const double* 
     if (s != SPDBA_OK) return s;
     if ((s = spdba_predictor_forward(pr, x_scratch, nmaps, pr->prob, st)) != SPDBA_OK) return s;
     const long long n = pr->m.V * nmaps;
-    prob_to_measure_kernel<<<grid_of(n, 256), 256, 0, st>>>(pr->prob, measure_out, n);
+    pdl_launch(prob_to_measure_kernel, grid_of(n, 256), 256, 0, st, pr->prob, measure_out, n);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
 }

@@ -22,6 +22,7 @@ constexpr int RCD_RX_NT = 256;
 template <typename T>
 __global__ void __launch_bounds__(RCD_RX_NT) rcd_reaction_kernel(cx_t<T>* __restrict__ w, long long n, int M, T r, T a,
                                                                  T alpha, T beta) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* su = reinterpret_cast<T*>(smem_raw);
     const int tid = threadIdx.x;
@@ -56,7 +57,7 @@ spdba_status launch_rcd_reaction(cx_t<T>* work, long long n, int M, T r, T a, T 
     const int smem = M * RCD_RX_NT * (int)sizeof(T);
     long long grid = (n + RCD_RX_NT - 1) / RCD_RX_NT;
     if (grid > 152 * 8) grid = 152 * 8;
-    rcd_reaction_kernel<T><<<(unsigned)grid, RCD_RX_NT, smem, st>>>(work, n, M, r, a, alpha, beta);
+    pdl_launch(rcd_reaction_kernel<T>, (unsigned)grid, RCD_RX_NT, smem, st, work, n, M, r, a, alpha, beta);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
 }
@@ -121,6 +122,7 @@ template <> __device__ __forceinline__ double rcd_mode_sq<double2>(const double2
 template <typename T>
 __global__ void rcd_activity_kernel(Geom g, const cx_t<T>* __restrict__ q, int M, long long n, double* maxsq,
                                     double* gmax) {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
     const long long nb = g.blocks();
@@ -159,7 +161,7 @@ spdba_status launch_rcd_activity(const Geom& g, const cx_t<T>* u_hat, int M, dou
     const long long nb = g.blocks();
     long long grid = (nb + 7) / 8;
     if (grid > 152 * 16) grid = 152 * 16;
-    rcd_activity_kernel<T><<<(unsigned)grid, 256, 0, st>>>(g, u_hat, M, g.modes(), maxsq, gmax);
+    pdl_launch(rcd_activity_kernel<T>, (unsigned)grid, 256, 0, st, g, u_hat, M, g.modes(), maxsq, gmax);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
 }
@@ -207,6 +209,7 @@ template <typename T, int MM> struct RcdOcc {
 
 template <typename T, int MM>
 __global__ void __launch_bounds__(RCD_NT, RcdOcc<T, MM>::value) rcd_update_kernel(Geom g, RcdArgs<T> a, int dense) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* sVt = reinterpret_cast<T*>(smem_raw);   // sVt[j * MM + i] = V[i][j] (zero padded)
     T* sV = sVt + MM * MM;                     // sV[i * MM + j] = V[i][j]
@@ -367,7 +370,7 @@ template <typename T, int MM> static spdba_status update_go(const Geom& g, const
     long long grid = (long long)RcdShape<T, MM>::per_sm * RcdShape<T, MM>::nsm;
     if (grid > items) grid = items;
     if (grid < 1) grid = 1;
-    rcd_update_kernel<T, MM><<<(unsigned)grid, RCD_NT, smem, st>>>(g, a, dense);
+    pdl_launch(rcd_update_kernel<T, MM>, (unsigned)grid, RCD_NT, smem, st, g, a, dense);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
 }

@@ -50,6 +50,7 @@ __device__ __forceinline__ void store2(double2* p, double2 a, double2 b) { p[0] 
 // Regular: every mode, two consecutive modes per thread along the fast axis.
 template <typename T>
 __global__ void ch_dense_kernel(Geom g, CHUpdateArgs<T> a) {
+    pdl_wait();
     const long long npairs = g.modes() / 2;
     if (blockIdx.x == 0 && a.stats)
         for (long long r = threadIdx.x; r < g.runs(); r += blockDim.x) a.stats[r].ratio_sum += 1.0;
@@ -77,6 +78,7 @@ __global__ void ch_dense_kernel(Geom g, CHUpdateArgs<T> a) {
 template <typename T>
 __global__ void ch_list_kernel(Geom g, CHUpdateArgs<T> a, FastDiv fd_h, FastDiv fd_b1, FastDiv fd_nb2,
                                FastDiv fd_nb1) {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const long long warp0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -132,6 +134,7 @@ __global__ void ch_list_kernel(Geom g, CHUpdateArgs<T> a, FastDiv fd_h, FastDiv 
 // independent row loads of ĉ and ĝ at a fixed stride, and no index is divided
 // at run time.  The same arithmetic as ch_list_kernel, bit for bit.
 __global__ void __launch_bounds__(256) ch_list8_kernel(Geom g, CHUpdateArgs<float> a) {
+    pdl_wait();
     constexpr int B = 8;
     const int lane = threadIdx.x & 31;
     const long long warp0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -186,7 +189,7 @@ template <typename T> spdba_status launch_ch_update(const Geom& g, const CHUpdat
         long long npairs = g.modes() / 2;
         long long grid = (npairs + 255) / 256;
         if (grid > 152 * 16) grid = 152 * 16;
-        ch_dense_kernel<T><<<(unsigned)grid, 256, 0, st>>>(g, a);
+        pdl_launch(ch_dense_kernel<T>, (unsigned)grid, 256, 0, st, g, a);
     } else {
         long long nb = g.blocks();
         long long grid = (nb * 32 + 255) / 256;
@@ -195,7 +198,7 @@ template <typename T> spdba_status launch_ch_update(const Geom& g, const CHUpdat
         if constexpr (std::is_same<T, float>::value) {
             fixed8 = g.ndim == 3 && g.runs() == 1 && g.b[0] == 8 && g.b[1] == 8 && g.b[2] == 8 &&
                      g.blocks() < 0x7fffffffLL;
-            if (fixed8) ch_list8_kernel<<<(unsigned)grid, 256, 0, st>>>(g, a);
+            if (fixed8) pdl_launch(ch_list8_kernel, (unsigned)grid, 256, 0, st, g, a);
         }
         if (!fixed8) {
             FastDiv fd_h, fd_b1, fd_nb2, fd_nb1;
@@ -203,7 +206,7 @@ template <typename T> spdba_status launch_ch_update(const Geom& g, const CHUpdat
             fd_b1.init((uint32_t)g.b[1]);
             fd_nb2.init((uint32_t)g.nb[2]);
             fd_nb1.init((uint32_t)g.nb[1]);
-            ch_list_kernel<T><<<(unsigned)grid, 256, 0, st>>>(g, a, fd_h, fd_b1, fd_nb2, fd_nb1);
+            pdl_launch(ch_list_kernel<T>, (unsigned)grid, 256, 0, st, g, a, fd_h, fd_b1, fd_nb2, fd_nb1);
         }
     }
     SPDBA_CUDA(cudaGetLastError());

@@ -35,6 +35,7 @@ __global__ void __launch_bounds__(TMA_NT) ch_list_tma_kernel(const __grid_consta
                                                              const __grid_constant__ CUtensorMap map_g, Geom g,
                                                              CHUpdateArgs<float> a, long long spin_limit,
                                                              int stall) {
+    pdl_wait();
     extern __shared__ __align__(128) unsigned char smem_tma[];
     // input stages (128-byte aligned), then two output boxes, then the barriers
     TmaStage* stage = reinterpret_cast<TmaStage*>(smem_tma);
@@ -203,7 +204,7 @@ spdba_status launch_ch_update_tma(const void* map_c, const void* map_g, const Ge
     const long long cap = g.blocks();
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
-    ch_list_tma_kernel<<<(unsigned)grid, TMA_NT, tma_update_smem(), st>>>(
+    pdl_launch(ch_list_tma_kernel, (unsigned)grid, TMA_NT, tma_update_smem(), st,
         *reinterpret_cast<const CUtensorMap*>(map_c), *reinterpret_cast<const CUtensorMap*>(map_g), g, a,
         wait_limit(), stall_waits());
     SPDBA_CUDA(cudaGetLastError());
