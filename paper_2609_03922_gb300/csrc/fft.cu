@@ -80,6 +80,17 @@ template <typename T> __global__ void twiddle_kernel(cx_t<T>* t, long long n) {
     }
 }
 
+// Four-step twiddles exp(-2 pi i m i / n), m < n / 512, i < 512, at m * 512 + i.
+template <typename T> __global__ void fourstep_twiddle_kernel(cx_t<T>* t, long long n) {
+    pdl_wait();
+    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e < n) {
+        double s, c;
+        sincospi(2.0 * (double)((e >> 9) * (e & 511)) / (double)n, &s, &c);   // the product stays below n
+        t[e] = mk<cx_t<T>>((T)c, (T)(-s));
+    }
+}
+
 template <typename T> cx_t<T>* TwiddleCache<T>::get(int64_t n, cudaStream_t st, spdba_status* err) {
     auto it = tables.find(n);
     if (it != tables.end()) return it->second;
@@ -146,7 +157,17 @@ spdba_status make_pass(Pass<T>* out, int64_t L, int sign, int mode, long long O,
         const KernelInfo wide = ki;
         if (!get(TILE_NARROW) || I % ki.P != 0) ki = wide;
     }
-    const bool generic = !ok || I % ki.P != 0;
+    bool generic = !ok || I % ki.P != 0;
+    if (sizeof(T) == 4 && !chain && mode == PASS_PLAIN && !loadp && storep) {
+        // rows in, columns out (the second pass of a four-step transform)
+        const KernelInfo simple = ki;
+        if (get_transpose2_kernel(L, sign, &ki) && I % ki.P == 0) {
+            ok = true;
+            generic = false;
+        } else {
+            ki = simple;
+        }
+    }
     if (generic) ok = get(TILE_GENERIC);
     if (!ok) return fail(SPDBA_ERR_UNSUPPORTED, "no FFT pass kernel for length %lld (mode %d)", (long long)L, mode);
     spdba_status s = ensure_smem_attr(ki.func, ki.smem, !generic);
@@ -174,7 +195,6 @@ spdba_status make_pass(Pass<T>* out, int64_t L, int sign, int mode, long long O,
     ps.p.osO = osO; ps.p.osI = osI; ps.p.osJ = osJ;
     ps.p.tw = t;
     ps.p.tw4 = nullptr;
-    ps.p.n4 = 1;
     ps.p.scale = (T)1;
     ps.p.generic = generic;
     ps.p.fd_I.init((uint32_t)I);
@@ -233,16 +253,18 @@ spdba_status FftEngine<T>::init(int nd, const int64_t* d, int64_t b, TwiddleCach
         long long n2 = 512, n1 = n / n2;
         if (n % 512 != 0 || !tile_length_supported(n1) || n1 > 512)
             return fail(SPDBA_ERR_UNSUPPORTED, "1-D length %lld not supported", n);
-        s = SPDBA_OK;
-        cx_t<T>* t4 = tw.get(n, st, &s);
-        if (!t4) return s;
+        if (!tw4) {
+            cudaError_t e = dev_alloc((void**)&tw4, sizeof(cx_t<T>) * (size_t)n);
+            if (e != cudaSuccess) return cuda_fail(e, "device allocation (four-step twiddles)");
+            pdl_launch(fourstep_twiddle_kernel<T>, (unsigned)((n + 255) / 256), 256, 0, st, tw4, n);
+            SPDBA_CUDA(cudaGetLastError());
+        }
         for (int dir = 0; dir < 2; ++dir) {
             int sign = dir == 0 ? -1 : +1;
             Pass<T> p1, p2;
             s = make_pass<T>(&p1, n1, sign, PASS_PLAIN, b, n2, n, 1, n2, n, 1, n2, tw, st, true);
             if (s != SPDBA_OK) return s;
-            p1.p.tw4 = t4;
-            p1.p.n4 = n;
+            p1.p.tw4 = tw4;
             s = make_pass<T>(&p2, n2, sign, PASS_PLAIN, b, n1, n, n2, 1, n, 1, n1, tw, st);
             if (s != SPDBA_OK) return s;
             if (sign > 0) p2.p.scale = (T)(1.0 / (double)n);
@@ -294,7 +316,9 @@ spdba_status FftEngine<T>::exec(const cx_t<T>* in, cx_t<T>* out, int direction, 
 
 template <typename T> void FftEngine<T>::release() {
     if (scratch) dev_free(scratch);
+    if (tw4) dev_free(tw4);
     scratch = nullptr;
+    tw4 = nullptr;
 }
 
 template struct TwiddleCache<float>;
@@ -359,8 +383,6 @@ spdba_status make_half_pass(Pass<float>* out, int mode, const HalfGeo& hg, Twidd
     s = SPDBA_OK;
     if (!(a.tw = tw.get(L, st, &s))) return s;
     a.tw4 = nullptr;
-
-    a.n4 = 1;
     a.scale = 1.f;
     a.generic = 0;
     a.nl_scale = (float)(1.0 / ((double)hg.N0 * hg.N1 * hg.N2));

@@ -126,8 +126,7 @@ template <typename T> struct PassParams {
     long long isO, isI, isJ;              // input strides (elements)
     long long osO, osI, osJ;              // output strides
     const cx_t<T>* tw;                    // exp(-2 pi i m / L), m < L
-    const cx_t<T>* tw4;                   // four-step twiddles exp(-2 pi i m / N4), or null
-    long long n4;
+    const cx_t<T>* tw4;                   // four-step twiddles exp(-2 pi i i m / (I L)) at m * I + i, or null
     T scale;                              // multiply on store (1 = none)
     int generic;                          // 1: I % P != 0, per-pencil address arithmetic
     // CH nonlinearity fused between the inverse and forward x transforms
@@ -786,23 +785,38 @@ template <typename T, int L> struct PlainOut {
 };
 
 
-// Four-step twiddle: element (pencil i, output index j) *= W_N^{i j}.
-template <typename T, int L, int P, int NT, int SIGN, class LY>
-__device__ __forceinline__ void apply_fourstep_twiddle(cx_t<T>* sm, const PassParams<T>& a, long long q0) {
+// Plain pass output of the first pass of a four-step transform: element (pencil i,
+// output index m) times W_N^{i m}, read from the table tw4 at m * I + i, which
+// consecutive lanes (pencils) read side by side.  (Forming the index modulo N in 64
+// bits per element, in a pass of its own over the tile, took two thirds of the
+// kernel: 128 us for 32 x 512 x 512.)
+template <typename T, int L, int SIGN> struct FourStepOut {
     using C = cx_t<T>;
-    for (int e = threadIdx.x; e < P * L; e += NT) {
-        int p, j;
-        if constexpr (LY::PMAP) { p = e % P; j = e / P; }
-        else { p = e / L; j = e % L; }
-        long long q = q0 + p;
-        long long i = q % a.I;
-        long long m = (i * (long long)j) % a.n4;
-        C w = __ldg(a.tw4 + m);
-        if constexpr (SIGN > 0) w.y = -w.y;
-        sm[LY::idx(p, j)] = cmul(sm[LY::idx(p, j)], w);
+    static constexpr bool SYNC = false;
+    C* base;
+    const C* tw;   // (output 0, pencil 0 of the tile)
+    int osI, osJ, I;
+    __device__ __forceinline__ FourStepOut(const PassParams<T>& a, long long q0) {
+        const long long o = a.fd_I.div((uint32_t)q0), i0 = q0 - o * a.I;
+        base = a.out + (o * a.osO + i0 * a.osI);
+        tw = a.tw4 + i0;
+        osI = (int)a.osI;
+        osJ = (int)a.osJ;
+        I = (int)a.I;
     }
-    __syncthreads();
-}
+    __device__ __forceinline__ void pre() {}
+    __device__ __forceinline__ void begin(int, int, int) {}
+    template <int R> __device__ __forceinline__ void emit(int, int p, int j, C (&v)[R]) {
+        C* po = base + (p * osI + j * osJ);
+        const C* t = tw + (p + j * I);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            C w = __ldg(t + r * (L / R) * I);
+            if constexpr (SIGN > 0) w.y = -w.y;
+            po[r * (L / R) * osJ] = cmul(v[r], w);
+        }
+    }
+};
 
 // Pass modes
 enum PassMode : int {
@@ -1104,7 +1118,6 @@ __device__ __forceinline__ void tile_body(cx_t<T>* sm, const PassParams<T>& a, l
     using C = cx_t<T>;
     if constexpr (MODE == PASS_PLAIN) {
         run_stages<T, L, P, NT, SIGN, LY>(sm, a.tw);
-        if (a.tw4 != nullptr) apply_fourstep_twiddle<T, L, P, NT, SIGN, LY>(sm, a, q0);
     } else if constexpr (MODE == PASS_CH_UPDATE) {
         run_stages<T, L, P, NT, -1, LY>(sm, a.tw);
     } else if constexpr (MODE == PASS_CH_NL) {
@@ -1194,6 +1207,13 @@ __device__ __forceinline__ void pipe_tile(cx_t<T>* sm, cx_t<T>* chat, const Pass
     // (the radix-3 tails of 192 and 384 hold too many registers to emit directly)
     constexpr bool DIRECT = (LY::PMAP || (L / Radices_last<L>::value) * (int)sizeof(C) >= 32) &&
                             Radices_last<L>::value != 3;
+    if constexpr (MODE == PASS_PLAIN && PFAST) {
+        if (a.tw4 != nullptr) {
+            FourStepOut<T, L, SIGN> out(a, q0);
+            run_stages_out<T, L, P, NT, SIGN, LY>(sm, tw, out);
+            return;
+        }
+    }
     if constexpr (MODE == PASS_MIRROR) {
         MirrorPlainOut<T, L, P> out(a, q0);
         run_stages_out<T, L, P, NT, SIGN, LY>(sm, tw, out);
@@ -1202,14 +1222,8 @@ __device__ __forceinline__ void pipe_tile(cx_t<T>* sm, cx_t<T>* chat, const Pass
         tile_body<T, L, P, NT, SIGN, MODE, LY>(sm, a, q0);
         store_tile<T, L, P, NT, PFAST, LY>(sm, a, q0);
     } else if constexpr (MODE == PASS_PLAIN) {
-        if (a.tw4 != nullptr) {
-            // first pass of a four-step transform: twiddle in shared memory
-            tile_body<T, L, P, NT, SIGN, MODE, LY>(sm, a, q0);
-            store_tile<T, L, P, NT, PFAST, LY>(sm, a, q0);
-        } else {
-            PlainOut<T, L> out(a, q0);
-            run_stages_out<T, L, P, NT, SIGN, LY>(sm, tw, out);
-        }
+        PlainOut<T, L> out(a, q0);
+        run_stages_out<T, L, P, NT, SIGN, LY>(sm, tw, out);
     } else if constexpr (MODE == PASS_CH_NL) {
         // inverse transform, the nonlinearity, forward transform (last stage storing)
         ChNlMid<T> mid{a.nl_scale, (T)0};

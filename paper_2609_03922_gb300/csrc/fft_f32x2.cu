@@ -60,6 +60,18 @@ bool get_pass2_kernel(int64_t L, int sign, int mode, bool strided_axis, bool nar
     }
 }
 
+bool get_transpose2_kernel(int64_t L, int sign, KernelInfo* ki) {
+    if (L != 512) return false;   // the row length of every four-step transform
+    constexpr int P = 16, NT = 256, OCC = 2;
+    ki->P = P;
+    ki->NT = NT;
+    ki->pipe = false;
+    ki->smem = LayoutA<512, P / 2, true>::SIZE * (int)sizeof(cf32x2);
+    ki->func = sign < 0 ? (const void*)fft_rows_transpose2_kernel<512, P, NT, -1, OCC>
+                        : (const void*)fft_rows_transpose2_kernel<512, P, NT, +1, OCC>;
+    return true;
+}
+
 template <int L, int P, int NT, int OCC> static bool chain(KernelInfo* ki) {
     ki->P = P;
     ki->NT = NT;

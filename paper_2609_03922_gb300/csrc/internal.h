@@ -80,6 +80,7 @@ template <typename T> struct FftEngine {
     std::vector<Pass<T>> fwd, inv;
     std::vector<int> fwd_scratch_out, inv_scratch_out;  // 1 if the pass writes to scratch
     cx_t<T>* scratch = nullptr;
+    cx_t<T>* tw4 = nullptr;   // four-step twiddles of a long 1-D transform
     spdba_status init(int ndim, const int64_t* dims, int64_t batch, TwiddleCache<T>& tw, cudaStream_t st);
     spdba_status exec(const cx_t<T>* in, cx_t<T>* out, int direction, cudaStream_t st);
     void release();

@@ -17,6 +17,8 @@ bool get_pass_kernel(int64_t L, int sign, int mode, bool loadp, bool storep, Til
                      KernelInfo* ki);
 // complex64 kernels with two pencils per thread (fft_f32x2.cuh), where they are the faster ones
 bool get_pass2_kernel(int64_t L, int sign, int mode, bool strided, bool narrow, KernelInfo* ki);
+// rows in, transposed out (unit-stride pencils on the output)
+bool get_transpose2_kernel(int64_t L, int sign, KernelInfo* ki);
 bool get_chain2_kernel(int64_t L, bool narrow, KernelInfo* ki);
 bool get_nl_half2_kernel(int64_t L, int nhp, KernelInfo* ki);
 // the step chain (PASS_CH_CHAIN) along the first axis
