@@ -145,6 +145,10 @@ template <typename T> struct PassParams {
     // unmarked columns are never read), or null to transform every tile
     const uint8_t* col_live = nullptr;
     int stream_chat = 0;   // step chain: c_hat is streamed past the L2
+    // plain passes whose outer index o (strided) or row (rows) runs over fields of
+    // seg_n such indices: a tile is skipped when its entries of seg_live are zero
+    const uint8_t* seg_live = nullptr;
+    FastDiv fd_seg;        // division by seg_n
 };
 
 // Address of element (p, j) of the tile starting at pencil q0.
@@ -898,6 +902,10 @@ __device__ __forceinline__ UpdTile upd_tile(const PassParams<T>& a, int q0) {
 template <typename T, int P, int MODE>
 __device__ __forceinline__ bool tile_live(const PassParams<T>& a, long long q0) {
     if constexpr (MODE == PASS_PLAIN) {
+        if (a.seg_live != nullptr) {
+            const uint32_t o = a.fd_I.div((uint32_t)q0);
+            if (a.seg_live[o - a.fd_seg.div(o) * a.fd_seg.d] == 0) return false;
+        }
         if (a.col_live == nullptr) return true;
         const long long i0 = q0 - (long long)a.fd_I.div((uint32_t)q0) * a.I;
         bool live = false;

@@ -99,15 +99,8 @@ __global__ void __launch_bounds__(NT, OCC) fft_pipe2_kernel(PassParams<float> a)
     const int p = (int)(threadIdx.x % H), j0 = (int)(threadIdx.x / H);
     static_assert(NT % H == 0, "each thread copies one pencil pair");
     auto next_live = [&](int t) {
-        if (a.col_live == nullptr) return t;
-        for (; t < ntiles; t += G) {
-            const long long q0 = (long long)t * P;
-            const long long i0 = q0 - (long long)a.fd_I.div((uint32_t)q0) * a.I;
-            bool live = false;
-#pragma unroll
-            for (int k = 0; k < P; ++k) live |= a.col_live[i0 + k] != 0;
-            if (live) break;
-        }
+        if (a.col_live == nullptr && a.seg_live == nullptr) return t;
+        while (t < ntiles && !tile_live<float, P, PASS_PLAIN>(a, (long long)t * P)) t += G;
         return t;
     };
     auto issue = [&](cf32x2* b, int t) {
@@ -312,6 +305,14 @@ __global__ void __launch_bounds__(NT, OCC) fft_rows2_kernel(PassParams<float> a)
     __shared__ cf32x2 s_tw[L];
     const long long q0 = (long long)blockIdx.x * P;
     const long long o = a.fd_I.div((uint32_t)q0), i0 = q0 - o * a.I;
+    if (MODE == PASS_PLAIN && a.seg_live != nullptr) {
+        // P rows of one field (its rows are a whole number of tiles)
+        const uint32_t r0 = (uint32_t)q0 - a.fd_seg.div((uint32_t)q0) * a.fd_seg.d;
+        bool live = false;
+#pragma unroll
+        for (int p = 0; p < P; ++p) live |= a.seg_live[r0 + p] != 0;
+        if (!live) return;
+    }
     dup_twiddles<L, NT>(s_tw, a.tw);
     RowPairIn in{a.in + (o * a.isO + i0 * a.isI), (int)a.isI};
     RowPairOut<L> out{a.out + (o * a.osO + i0 * a.osI), (int)a.osI, f32x2(a.scale)};
@@ -351,7 +352,6 @@ __global__ void __launch_bounds__(NT, OCC) fft_rows_transpose2_kernel(PassParams
     pdl_wait();
     constexpr int H = P / 2;
     using LY = LayoutA<L, H, true>;
-    constexpr int NST = NSTAGES<L>::value;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cf32x2* const sm = reinterpret_cast<cf32x2*>(smem_raw);
     __shared__ cf32x2 s_tw[L];

@@ -193,6 +193,12 @@ template <typename T> struct Group {
     T* rcd_V = nullptr;             // eigenvectors of D, row-major V[i * M + j]
     T* rcd_lam = nullptr;           // eigenvalues of D
     FftEngine<T> rcd_fft;           // transforms of the ncomp fields (one batch)
+    RcdPack rcd_pack;               // two components per complex field between the update and itself (complex64)
+    std::vector<Pass<T>> rcd_inv, rcd_fwd;   // ... its remaining inverse passes and its forward passes
+    bool rcd_prune = false;         // ... skipping, on adaptive steps, planes (and rows) that no non-frozen
+    bool rcd_prune_rows = false;    // block reads
+    uint8_t* rcd_row_live = nullptr;
+    uint8_t* rcd_plane_live = nullptr;
     // TMA form of the list-driven update (3-D complex64, 8^3 blocks): tensor maps of c_hat and work
     alignas(64) unsigned char tma_map_c[128] = {};
     alignas(64) unsigned char tma_map_g[128] = {};
@@ -820,6 +826,32 @@ static spdba_status group_init_rcd(spdba_plan* p, Group<T>& r, int ndim, const i
     rcd_eigen_host(M, p->opt.rcd_d_diag, p->opt.rcd_d_cross, V, lam);
     if ((s = upload(r, &r.rcd_V, std::vector<T>(V.begin(), V.end()), st)) != SPDBA_OK) return s;
     if ((s = upload(r, &r.rcd_lam, std::vector<T>(lam.begin(), lam.end()), st)) != SPDBA_OK) return s;
+    if constexpr (std::is_same<T, float>::value) {
+        if ((s = rcd_pack_prepare(&r.rcd_pack, ndim, dims, M, p->tw32, st)) != SPDBA_OK) return s;
+        if (r.rcd_pack.ok) {
+            // inverse: rows (with the packing), then the other axes from the last; forward back
+            // in the reverse order, rows last, so that rows and planes no block reads drop out
+            const int Mh = r.rcd_pack.Mh;
+            for (int a = ndim - 2; a >= 0; --a) {
+                Pass<T> ps;
+                if ((s = make_axis_pass<T>(&ps, ndim, dims, Mh, a, +1, PASS_PLAIN, p->tw32, st)) != SPDBA_OK) return s;
+                r.rcd_inv.push_back(ps);
+            }
+            for (int a = 0; a < ndim; ++a) {
+                Pass<T> ps;
+                if ((s = make_axis_pass<T>(&ps, ndim, dims, Mh, a, -1, PASS_PLAIN, p->tw32, st)) != SPDBA_OK) return s;
+                r.rcd_fwd.push_back(ps);
+            }
+            const long long rows = r.g.n[0] * r.g.n[1];
+            r.rcd_prune = true;
+            // rows: the kernels with two rows per thread, whose tiles lie within one field
+            r.rcd_prune_rows = dims[ndim - 1] >= 64 && rows % 16 == 0 && !r.rcd_fwd.back().p.generic;
+            if ((s = r.alloc(&r.rcd_row_live, (size_t)rows)) != SPDBA_OK) return s;
+            if ((s = r.alloc(&r.rcd_plane_live, (size_t)r.g.n[0])) != SPDBA_OK) return s;
+            r.rcd_fwd.back().p.fd_seg.init((uint32_t)rows);
+            if (ndim == 3) r.rcd_fwd[1].p.fd_seg.init((uint32_t)r.g.n[0]);
+        }
+    }
     return rcd_prepare<T>(M);
 }
 
@@ -1246,6 +1278,39 @@ template <typename T> static spdba_status group_nls_steps(spdba_plan* p, Group<T
     return SPDBA_OK;
 }
 
+// u_hat -> packed fields -> R(u) -> packed transform in `work` (complex64).
+static spdba_status rcd_packed_passes(spdba_plan* p, Group<float>& r, int dense) {
+    cudaStream_t st = p->st;
+    spdba_status s;
+    const RcdPack& pk = r.rcd_pack;
+    const double half_b = sizeof(float2) * (double)(pk.Mh * r.n);
+    {
+        ProfScope pr(p, K_RCD_FFT, 2.0 * r.ndim * half_b + sizeof(float2) * (double)((pk.M - pk.Mh) * r.n));
+        if ((s = launch_rcd_pack(pk, r.c_hat, r.work, st)) != SPDBA_OK) return s;
+        for (auto& ps : r.rcd_inv)
+            if ((s = launch_pass<float>(ps, r.work, r.work, st)) != SPDBA_OK) return s;
+    }
+    {
+        ProfScope pr(p, K_RCD_REACTION, 2.0 * half_b);
+        const RcdParams& q = p->rcd;
+        if ((s = launch_rcd_reaction_packed(pk, r.work, (float)q.r, (float)q.a, (float)q.alpha, (float)q.beta, st)) !=
+            SPDBA_OK)
+            return s;
+    }
+    {
+        ProfScope pr(p, K_RCD_FFT, 2.0 * r.ndim * half_b);
+        for (int a = 0; a < r.ndim; ++a) {
+            Pass<float> ps = r.rcd_fwd[a];
+            if (!dense && r.rcd_prune) {
+                if (a == r.ndim - 1) ps.p.seg_live = r.rcd_prune_rows ? r.rcd_row_live : nullptr;
+                else if (a == 1) ps.p.seg_live = r.rcd_plane_live;
+            }
+            if ((s = launch_pass<float>(ps, r.work, r.work, st)) != SPDBA_OK) return s;
+        }
+    }
+    return SPDBA_OK;
+}
+
 // One RCD step (S4.2): state preparation at reassessments (component RMS
 // amplitude), u = IFFT(u_hat) of the M components, R(u) in real space, its
 // FFT, then the per-mode coupled update on the listed blocks (or every block).
@@ -1266,20 +1331,29 @@ template <typename T> static spdba_status group_rcd_step(spdba_plan* p, Group<T>
                                            r.scratch, r.stats, st)) != SPDBA_OK)
             return s;
         p->launches += 4;
+        if (r.rcd_prune) {
+            if ((s = launch_rcd_live(r.g, r.states, r.rcd_row_live, r.rcd_plane_live, st)) != SPDBA_OK) return s;
+            p->launches += 1;
+        }
         r.assessed = true;
     }
     const int dense = !adaptive || all_active_step(p, r.step);
-    {
+    bool packed = false;
+    if constexpr (std::is_same<T, float>::value) {
+        packed = r.rcd_pack.ok;
+        if (packed && (s = rcd_packed_passes(p, r, dense)) != SPDBA_OK) return s;
+    }
+    if (!packed) {
         ProfScope pr(p, K_RCD_FFT, 2.0 * r.ndim * field_b);
         if ((s = r.rcd_fft.exec(r.c_hat, r.work, SPDBA_INVERSE, st)) != SPDBA_OK) return s;
     }
-    {
+    if (!packed) {
         ProfScope pr(p, K_RCD_REACTION, 2.0 * field_b);
         const RcdParams& q = p->rcd;
         if ((s = launch_rcd_reaction<T>(r.work, r.n, M, (T)q.r, (T)q.a, (T)q.alpha, (T)q.beta, st)) != SPDBA_OK)
             return s;
     }
-    {
+    if (!packed) {
         ProfScope pr(p, K_RCD_FFT, 2.0 * r.ndim * field_b);
         if ((s = r.rcd_fft.exec(r.work, r.work, SPDBA_FORWARD, st)) != SPDBA_OK) return s;
     }
@@ -1296,6 +1370,7 @@ template <typename T> static spdba_status group_rcd_step(spdba_plan* p, Group<T>
     a.count = r.count;
     a.dt = (T)p->opt.dt;
     a.M = M;
+    a.packed = packed;
     a.n = r.n;
     a.stats = r.stats;
     {
@@ -1957,6 +2032,10 @@ template <typename T> static spdba_status snap_take(spdba_plan* p, Group<T>& r, 
     // between reassessments resumes with the states of the snapshot, so their
     // liveness is restored with them
     if (r.col_live) sn.bufs.push_back({r.col_live, (size_t)r.h_fwd_y.p.I});
+    if (r.rcd_prune) {
+        sn.bufs.push_back({r.rcd_row_live, (size_t)(r.g.n[0] * r.g.n[1])});
+        sn.bufs.push_back({r.rcd_plane_live, (size_t)r.g.n[0]});
+    }
     if (r.hs_zlive) {
         sn.bufs.push_back({r.hs_zlive, (size_t)(r.g.n[1] * r.g.n[2])});
         sn.bufs.push_back({r.hs_xlive, (size_t)r.g.n[2]});

@@ -258,12 +258,53 @@ __global__ void __launch_bounds__(RCD_NT, RcdOcc<T, MM>::value) rcd_update_kerne
         const int lt = threadIdx.x % RCD_TM, lm0 = threadIdx.x / RCD_TM;
         const int lo = ti * RCD_TM + lt;
         const bool lvalid = lo < bm;
-        long long lidx = 0;
+        long long lidx = 0, midx = 0;   // the mode and its mirror -k
         if (lvalid) {
             const int d2 = lo % B2, d1 = (lo / B2) % B1, d0 = lo / (B2 * B1);
-            lidx = ((b0 * B0 + d0) * g.n[1] + (b1 * B1 + d1)) * g.n[2] + (b2 * B2 + d2);
+            const long long kz = b0 * B0 + d0, ky = b1 * B1 + d1, kx = b2 * B2 + d2;
+            lidx = (kz * g.n[1] + ky) * g.n[2] + kx;
+            midx = ((kz == 0 ? 0 : g.n[0] - kz) * g.n[1] + (ky == 0 ? 0 : g.n[1] - ky)) * g.n[2] +
+                   (kx == 0 ? 0 : g.n[2] - kx);
         }
-        {
+        if (a.packed) {
+            // thread e takes component pairs e / RCD_TM, ...: both from W(k) and W(-k)
+            constexpr int PPER = (MM / 2 + LSTEP - 1) / LSTEP;
+            const int Mh = (M + 1) / 2;
+            cx_t<T> u0[PPER], u1[PPER], wk[PPER], wm[PPER];
+#pragma unroll
+            for (int k = 0; k < PPER; ++k) {
+                const int c = lm0 + LSTEP * k;
+                u0[k] = mk<cx_t<T>>((T)0, (T)0);
+                u1[k] = wk[k] = wm[k] = u0[k];
+                if (c < Mh && lvalid) {
+                    u0[k] = a.u_hat[(long long)(2 * c) * n + lidx];
+                    if (2 * c + 1 < M) u1[k] = a.u_hat[(long long)(2 * c + 1) * n + lidx];
+                    wk[k] = a.g_hat[(long long)c * n + lidx];
+                    wm[k] = a.g_hat[(long long)c * n + midx];
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < PPER; ++k) {
+                const int c = lm0 + LSTEP * k;
+                if (2 * c < MM) {
+                    const cx_t<T> w = wk[k], v = wm[k];
+                    // (W + conj V) / 2 and (W - conj V) / (2 i)
+                    const T g0x = (T)0.5 * (w.x + v.x), g0y = (T)0.5 * (w.y - v.y);
+                    const T g1x = (T)0.5 * (w.y + v.y), g1y = (T)-0.5 * (w.x - v.x);
+                    T* pu = sU + (2 * c) * RCD_COLS + 2 * lt;
+                    T* py = sY + (2 * c) * RCD_COLS + 2 * lt;
+                    pu[0] = u0[k].x;
+                    pu[1] = u0[k].y;
+                    py[0] = u0[k].x + a.dt * g0x;
+                    py[1] = u0[k].y + a.dt * g0y;
+                    const bool two = 2 * c + 1 < M;
+                    pu[RCD_COLS] = u1[k].x;
+                    pu[RCD_COLS + 1] = u1[k].y;
+                    py[RCD_COLS] = two ? u1[k].x + a.dt * g1x : (T)0;
+                    py[RCD_COLS + 1] = two ? u1[k].y + a.dt * g1y : (T)0;
+                }
+            }
+        } else {
             cx_t<T> u[LPER], gg[LPER];
 #pragma unroll
             for (int k = 0; k < LPER; ++k) {
