@@ -32,20 +32,34 @@ namespace spdba {
 template <class C> __device__ __forceinline__ C tw_load(const C* p) { return __isShared(p) ? *p : __ldg(p); }
 __device__ __forceinline__ cf32x2 tw_load(const cf32x2* p) { return *p; }   // always a shared table
 
-// Radix schedule per pencil length (product of radices == L).
-template <int L> struct Radices;
+// Radix schedule per element type and pencil length (product of radices == L).
+// FP32: few stages, as registers allow.  FP64: radices of at most 8.  An SM takes an
+// FP64 instruction of a warp in 16 cycles however few of its lanes are in use,
+// and a pencil of 128 points is 8 butterflies of radix 16 but 32 of radix 4; the
+// operation counts are the same (25 per point of 256 either way).
+template <typename T, int L> struct Radices;
 template <int... R> struct RList {};
-template <> struct Radices<16> { using type = RList<16>; };
-template <> struct Radices<32> { using type = RList<8, 4>; };
-template <> struct Radices<64> { using type = RList<8, 8>; };
-template <> struct Radices<128> { using type = RList<16, 8>; };
-template <> struct Radices<192> { using type = RList<8, 3, 8>; };
-template <> struct Radices<256> { using type = RList<16, 16>; };
-template <> struct Radices<384> { using type = RList<8, 6, 8>; };
-template <> struct Radices<512> { using type = RList<8, 8, 8>; };
-template <> struct Radices<1024> { using type = RList<16, 16, 4>; };
-template <> struct Radices<2048> { using type = RList<16, 16, 8>; };
-template <> struct Radices<4096> { using type = RList<16, 16, 16>; };
+template <int L> struct Radices32;
+template <> struct Radices32<16> { using type = RList<16>; };
+template <> struct Radices32<32> { using type = RList<8, 4>; };
+template <> struct Radices32<64> { using type = RList<8, 8>; };
+template <> struct Radices32<128> { using type = RList<16, 8>; };
+template <> struct Radices32<192> { using type = RList<8, 3, 8>; };
+template <> struct Radices32<256> { using type = RList<16, 16>; };
+template <> struct Radices32<384> { using type = RList<8, 6, 8>; };
+template <> struct Radices32<512> { using type = RList<8, 8, 8>; };
+template <> struct Radices32<1024> { using type = RList<16, 16, 4>; };
+template <> struct Radices32<2048> { using type = RList<16, 16, 8>; };
+template <> struct Radices32<4096> { using type = RList<16, 16, 16>; };
+template <int L> struct Radices64 : Radices32<L> {};
+template <> struct Radices64<16> { using type = RList<4, 4>; };
+template <> struct Radices64<32> { using type = RList<4, 2, 4>; };
+template <> struct Radices64<64> { using type = RList<4, 4, 4>; };
+template <> struct Radices64<128> { using type = RList<4, 8, 4>; };
+template <> struct Radices64<256> { using type = RList<4, 4, 4, 4>; };
+template <int L> struct Radices<float, L> : Radices32<L> {};
+template <int L> struct Radices<f32x2, L> : Radices32<L> {};
+template <int L> struct Radices<double, L> : Radices64<L> {};
 
 template <class RL> struct LastOf;
 template <int R0> struct LastOf<RList<R0>> { static constexpr int value = R0; };
@@ -54,20 +68,22 @@ template <int R0, int R1, int... Rs> struct LastOf<RList<R0, R1, Rs...>> {
 };
 template <class RL> struct CountOf;
 template <int... Rs> struct CountOf<RList<Rs...>> { static constexpr int value = sizeof...(Rs); };
-template <int L> struct NSTAGES { static constexpr int value = CountOf<typename Radices<L>::type>::value; };
+template <typename T, int L> struct NSTAGES { static constexpr int value = CountOf<typename Radices<T, L>::type>::value; };
 template <class RL> struct RArr;
 template <int... Rs> struct RArr<RList<Rs...>> {
     static constexpr int n = sizeof...(Rs);
     static constexpr int v[sizeof...(Rs)] = {Rs...};
 };
 // i-th radix of a length and the product of the radices before it
-template <int L> __host__ __device__ constexpr int radix_at(int i) { return RArr<typename Radices<L>::type>::v[i]; }
-template <int L> __host__ __device__ constexpr int ns_at(int i) {
+template <typename T, int L> __host__ __device__ constexpr int radix_at(int i) {
+    return RArr<typename Radices<T, L>::type>::v[i];
+}
+template <typename T, int L> __host__ __device__ constexpr int ns_at(int i) {
     int p = 1;
-    for (int k = 0; k < i; ++k) p *= radix_at<L>(k);
+    for (int k = 0; k < i; ++k) p *= radix_at<T, L>(k);
     return p;
 }
-template <int L> struct Radices_last { static constexpr int value = LastOf<typename Radices<L>::type>::value; };
+template <typename T, int L> struct Radices_last { static constexpr int value = LastOf<typename Radices<T, L>::type>::value; };
 
 // Layout A; ODD selects an odd pencil stride (needed when pencils are read
 // transposed, pencil-fastest), otherwise the stride stays even so that a pair
@@ -452,7 +468,7 @@ __device__ __forceinline__ void run_stages_list(cx_t<T>* sm, const cx_t<T>* tw, 
 // All stages of a length-L transform with kernel exp(SIGN 2 pi i n k / L).
 template <typename T, int L, int P, int NT, int SIGN, class LY>
 __device__ __forceinline__ void run_stages(cx_t<T>* sm, const cx_t<T>* tw) {
-    run_stages_list<T, L, P, NT, SIGN, LY>(sm, tw, typename Radices<L>::type{});
+    run_stages_list<T, L, P, NT, SIGN, LY>(sm, tw, typename Radices<T, L>::type{});
 }
 
 // Last stage with its outputs handed to `out` instead of written back to
@@ -529,7 +545,7 @@ __device__ __forceinline__ void run_stages_out_list(cx_t<T>* sm, const cx_t<T>* 
 // All stages of a length-L transform, the last one emitting through `out`.
 template <typename T, int L, int P, int NT, int SIGN, class LY, class OUT>
 __device__ __forceinline__ void run_stages_out(cx_t<T>* sm, const cx_t<T>* tw, OUT& out) {
-    run_stages_out_list<T, L, P, NT, SIGN, LY, OUT>(sm, tw, out, typename Radices<L>::type{});
+    run_stages_out_list<T, L, P, NT, SIGN, LY, OUT>(sm, tw, out, typename Radices<T, L>::type{});
 }
 
 // Last-stage outputs passed through an elementwise step and written back to
@@ -566,7 +582,7 @@ template <typename T> struct ChNlMid {
 template <typename T, int L, int P, int NT, int SIGN, class LY, int I, int E>
 __device__ __forceinline__ void run_stage_range(cx_t<T>* sm, const cx_t<T>* tw) {
     if constexpr (I < E) {
-        stockham_stage<T, L, P, NT, SIGN, ns_at<L>(I), radix_at<L>(I), LY>(sm, tw);
+        stockham_stage<T, L, P, NT, SIGN, ns_at<T, L>(I), radix_at<T, L>(I), LY>(sm, tw);
         run_stage_range<T, L, P, NT, SIGN, LY, I + 1, E>(sm, tw);
     }
 }
@@ -679,11 +695,11 @@ __device__ __forceinline__ void fused_mid_stage(cx_t<T>* sm, const cx_t<T>* __re
 // emits through `out` (at least two stages).
 template <typename T, int L, int P, int NT, int SIGN, class LY, class IN, class OUT>
 __device__ __forceinline__ void run_stages_in_out(cx_t<T>* sm, const cx_t<T>* tw, const IN& in, OUT& out) {
-    constexpr int NST = NSTAGES<L>::value;
+    constexpr int NST = NSTAGES<T, L>::value;
     static_assert(NST >= 2, "a separate first and last stage");
-    stockham_stage_in<T, L, P, NT, SIGN, 1, radix_at<L>(0), LY>(sm, tw, in);
+    stockham_stage_in<T, L, P, NT, SIGN, 1, radix_at<T, L>(0), LY>(sm, tw, in);
     run_stage_range<T, L, P, NT, SIGN, LY, 1, NST - 1>(sm, tw);
-    stockham_stage_out<T, L, P, NT, SIGN, ns_at<L>(NST - 1), radix_at<L>(NST - 1), LY>(sm, tw, out);
+    stockham_stage_out<T, L, P, NT, SIGN, ns_at<T, L>(NST - 1), radix_at<T, L>(NST - 1), LY>(sm, tw, out);
 }
 
 template <typename T, int L, int P, int NT, int SA, int SB, class LY, class MID, class OUT>
@@ -694,8 +710,8 @@ __device__ __forceinline__ void transform_pair(cx_t<T>* sm, const cx_t<T>* tw, M
 // three stages in all.
 template <typename T, int L, int P, int NT, int SA, int SB, class LY, class IN, class MID, class OUT>
 __device__ __forceinline__ void transform_pair_in(cx_t<T>* sm, const cx_t<T>* tw, const IN& in, MID& mid, OUT& out) {
-    constexpr int NST = NSTAGES<L>::value;
-    constexpr int R0 = radix_at<L>(0), RL = radix_at<L>(NST - 1);
+    constexpr int NST = NSTAGES<T, L>::value;
+    constexpr int R0 = radix_at<T, L>(0), RL = radix_at<T, L>(NST - 1);
     static_assert(NST >= 2, "the first stage must not be the meeting stage");
     stockham_stage_in<T, L, P, NT, SA, 1, R0, LY>(sm, tw, in);
     if constexpr (R0 == RL) {
@@ -704,11 +720,11 @@ __device__ __forceinline__ void transform_pair_in(cx_t<T>* sm, const cx_t<T>* tw
         fused_mid_stage<T, L, P, NT, SA, SB, L / R0, R0, LY>(sm, tw, mid, fo);
         __syncthreads();
         run_stage_range<T, L, P, NT, SB, LY, 1, NST - 1>(sm, tw);
-        stockham_stage_out<T, L, P, NT, SB, ns_at<L>(NST - 1), RL, LY>(sm, tw, out);
+        stockham_stage_out<T, L, P, NT, SB, ns_at<T, L>(NST - 1), RL, LY>(sm, tw, out);
     } else {
         run_stage_range<T, L, P, NT, SA, LY, 1, NST - 1>(sm, tw);
         MidOut<T, L, LY, MID> mo{sm, mid};
-        stockham_stage_out<T, L, P, NT, SA, ns_at<L>(NST - 1), RL, LY>(sm, tw, mo);
+        stockham_stage_out<T, L, P, NT, SA, ns_at<T, L>(NST - 1), RL, LY>(sm, tw, mo);
         __syncthreads();
         run_stages_out<T, L, P, NT, SB, LY>(sm, tw, out);
     }
@@ -716,8 +732,8 @@ __device__ __forceinline__ void transform_pair_in(cx_t<T>* sm, const cx_t<T>* tw
 
 template <typename T, int L, int P, int NT, int SA, int SB, class LY, class MID, class OUT>
 __device__ __forceinline__ void transform_pair(cx_t<T>* sm, const cx_t<T>* tw, MID& mid, OUT& out) {
-    constexpr int NST = NSTAGES<L>::value;
-    constexpr int R0 = radix_at<L>(0), RL = radix_at<L>(NST - 1);
+    constexpr int NST = NSTAGES<T, L>::value;
+    constexpr int R0 = radix_at<T, L>(0), RL = radix_at<T, L>(NST - 1);
     if constexpr (R0 == RL) {
         run_stage_range<T, L, P, NT, SA, LY, 0, NST - 1>(sm, tw);
         if constexpr (NST == 1) {
@@ -727,7 +743,7 @@ __device__ __forceinline__ void transform_pair(cx_t<T>* sm, const cx_t<T>* tw, M
             fused_mid_stage<T, L, P, NT, SA, SB, L / R0, R0, LY>(sm, tw, mid, fo);
             __syncthreads();
             run_stage_range<T, L, P, NT, SB, LY, 1, NST - 1>(sm, tw);
-            stockham_stage_out<T, L, P, NT, SB, ns_at<L>(NST - 1), RL, LY>(sm, tw, out);
+            stockham_stage_out<T, L, P, NT, SB, ns_at<T, L>(NST - 1), RL, LY>(sm, tw, out);
         }
     } else {
         MidOut<T, L, LY, MID> mo{sm, mid};
@@ -978,7 +994,7 @@ __host__ __device__ __forceinline__ int upd_table_cols(int P, int bx) { return (
 // The update pass stages c_hat in a third tile buffer for row-major tiles of
 // L <= 256 whose last stage emits directly (not the radix-3 tail of 192).
 template <typename T, int L> __host__ __device__ constexpr bool upd_stages_chat() {
-    return L <= 256 && Radices_last<L>::value != 3;
+    return L <= 256 && Radices_last<T, L>::value != 3;
 }
 
 // Update emitted from the forward transform's last stage (tile within one row):
@@ -1213,8 +1229,8 @@ __device__ __forceinline__ void pipe_tile(cx_t<T>* sm, cx_t<T>* chat, const Pass
     // direct stores from the last stage stay coalesced when a warp's lanes
     // cover at least 32 contiguous bytes of each output row
     // (the radix-3 tails of 192 and 384 hold too many registers to emit directly)
-    constexpr bool DIRECT = (LY::PMAP || (L / Radices_last<L>::value) * (int)sizeof(C) >= 32) &&
-                            Radices_last<L>::value != 3;
+    constexpr bool DIRECT = (LY::PMAP || (L / Radices_last<T, L>::value) * (int)sizeof(C) >= 32) &&
+                            Radices_last<T, L>::value != 3;
     if constexpr (MODE == PASS_PLAIN && PFAST) {
         if (a.tw4 != nullptr) {
             FourStepOut<T, L, SIGN> out(a, q0);
@@ -1253,7 +1269,7 @@ __device__ __forceinline__ void pipe_tile(cx_t<T>* sm, cx_t<T>* chat, const Pass
             ch_update_table<T, L, P, NT>(tab, a, u);
             __syncthreads();
             issue_chat<T, L, P, NT, LY>(chat, a, u, tab);
-            UpdOut<T, L, P, NT, Radices_last<L>::value, true, LY, MODE == PASS_UPD_HALF> out(a, u, tab, kp, chat);
+            UpdOut<T, L, P, NT, Radices_last<T, L>::value, true, LY, MODE == PASS_UPD_HALF> out(a, u, tab, kp, chat);
             run_stages_out<T, L, P, NT, -1, LY>(sm, tw, out);
         } else {
             ch_update_table<T, L, P, NT>(tab, a, u);
@@ -1278,8 +1294,8 @@ __global__ void __launch_bounds__(NT, PipeOcc<T, L, MODE, PFAST, NT>::value) fft
         const T* kpg = a.fu.g.ndim == 3 ? a.fu.k2ax[0] : a.fu.k2ax[1];
         for (int j = threadIdx.x; j < L; j += NT) s_kp[j] = kpg[j];   // visible after the loop's first barrier
     }
-    // complex64 passes up to 512 points keep the twiddle table in shared memory
-    constexpr bool STW = sizeof(T) == 4 && L <= 512;
+    // passes up to 512 points keep the twiddle table in shared memory
+    constexpr bool STW = L <= 512;
     __shared__ C s_tw[STW ? L : 1];
     if constexpr (STW)
         for (int j = threadIdx.x; j < L; j += NT) s_tw[j] = a.tw[j];   // visible after the loop's first barrier
@@ -1382,8 +1398,7 @@ __global__ void __launch_bounds__(NT, ChainOcc<T, L, NT>::value) fft_chain_kerne
     C* const cs = sm + LY::SIZE;
     __shared__ uint8_t s_tab[kUpdTable];
     __shared__ T s_kp[L];
-    constexpr bool STW = sizeof(T) == 4;   // twiddles in shared memory, as in the pipelined kernel
-    __shared__ C s_tw[STW ? L : 1];
+    __shared__ C s_tw[L];   // twiddles in shared memory, as in the pipelined kernel
     const CHFuse<T>& f = a.fu;
     const long long q0 = (long long)blockIdx.x * P;
     const UpdTile u = upd_tile<T, P>(a, (int)q0);
@@ -1392,9 +1407,8 @@ __global__ void __launch_bounds__(NT, ChainOcc<T, L, NT>::value) fft_chain_kerne
     ch_update_stats<T, NT>(f, f.dense);
     const T* kpg = f.g.ndim == 3 ? f.k2ax[0] : f.k2ax[1];
     for (int j = threadIdx.x; j < L; j += NT) s_kp[j] = kpg[j];
-    if constexpr (STW)
-        for (int j = threadIdx.x; j < L; j += NT) s_tw[j] = a.tw[j];
-    const C* const tw = STW ? s_tw : a.tw;
+    for (int j = threadIdx.x; j < L; j += NT) s_tw[j] = a.tw[j];
+    const C* const tw = s_tw;
     const int nent = (int)(f.g.ndim == 3 ? f.g.nb[0] : f.g.nb[1]) * u.nbx;
     ch_update_table<T, L, P, NT>(s_tab, a, u);
     __syncthreads();

@@ -94,11 +94,11 @@ bool get_chain2_kernel(int64_t L, bool narrow, KernelInfo* ki) {
 
 int chain2_step(int64_t L) {
     switch (L) {
-        case 64: return 64 / Radices_last<64>::value;
-        case 128: return 128 / Radices_last<128>::value;
-        case 192: return 192 / Radices_last<192>::value;
-        case 256: return 256 / Radices_last<256>::value;
-        case 384: return 384 / Radices_last<384>::value;
+        case 64: return 64 / Radices_last<f32x2, 64>::value;
+        case 128: return 128 / Radices_last<f32x2, 128>::value;
+        case 192: return 192 / Radices_last<f32x2, 192>::value;
+        case 256: return 256 / Radices_last<f32x2, 256>::value;
+        case 384: return 384 / Radices_last<f32x2, 384>::value;
         default: return 1;
     }
 }

@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(NT, OCC) fft_chain2_kernel(PassParams<float> a
     GlobalPairOut<L> out{a.out + ((long long)u.o * a.osO + u.i0), (int)a.osJ, f32x2(1.f)};
     if (live) {
         GlobalPairInWait in{{a.in + ((long long)u.o * a.isO + u.i0), (int)a.isJ}};
-        ChainMid2<L, H, L / Radices_last<L>::value> mid(a, u, s_tab, s_kp, cs, pol);
+        ChainMid2<L, H, L / Radices_last<f32x2, L>::value> mid(a, u, s_tab, s_kp, cs, pol);
         transform_pair_in<f32x2, L, H, NT, -1, +1, LY>(sm, s_tw, in, mid, out);
     } else {
         cp_async_wait<0>();

@@ -149,12 +149,12 @@ __global__ void __launch_bounds__(NT, 2) fft_herm_inv_kernel(PassParams<T> a) {
         // between its reads and writes frees the mirror buffer
         PlainOut<T, L> out(a, t * P);
         HermIn<T, L, P, LY> in{sm, smB};
-        stockham_stage_in<T, L, P, NT, +1, 1, radix_at<L>(0), LY>(sm, tw, in);
+        stockham_stage_in<T, L, P, NT, +1, 1, radix_at<T, L>(0), LY>(sm, tw, in);
         // the mirror tile of the next tile streams in during the rest of the transform
         if (tn < ntiles) issue_herm_mirror<T, L, P, NT>(smB, a, tn * P);
         cp_async_commit();
-        run_stage_range<T, L, P, NT, +1, LY, 1, NSTAGES<L>::value - 1>(sm, tw);
-        stockham_stage_out<T, L, P, NT, +1, ns_at<L>(NSTAGES<L>::value - 1), radix_at<L>(NSTAGES<L>::value - 1), LY>(
+        run_stage_range<T, L, P, NT, +1, LY, 1, NSTAGES<T, L>::value - 1>(sm, tw);
+        stockham_stage_out<T, L, P, NT, +1, ns_at<T, L>(NSTAGES<T, L>::value - 1), radix_at<T, L>(NSTAGES<T, L>::value - 1), LY>(
             sm, tw, out);
         __syncthreads();
         buf ^= 1;
@@ -516,7 +516,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) fft_pair_kernel(PassParams<T> a)
     using C = cx_t<T>;
     using LY = LayoutBP<L, P>;
     static_assert(NT % P == 0 && NT % (P / 2) == 0, "each thread keeps one pencil");
-    static_assert(Radices_last<L>::value != 3, "the last stage emits directly");
+    static_assert(Radices_last<T, L>::value != 3, "the last stage emits directly");
     static_assert(kPairBufs == 3, "the loop keeps two tiles in flight");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // complex64 passes up to 512 points keep the twiddle table in shared memory
@@ -556,7 +556,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) fft_pair_kernel(PassParams<T> a)
         __syncthreads();
         C* sm = smb + slot * LY::SIZE;
         if (t < ntm) {
-            PairPlainOut<T, L, P, Radices_last<L>::value> out(a, t, masked, s_tab, s_tab + kPairTable);
+            PairPlainOut<T, L, P, Radices_last<T, L>::value> out(a, t, masked, s_tab, s_tab + kPairTable);
             run_stages_out<T, L, P, NT, -1, LY>(sm, tw, out);
         } else {
             run_stages<T, L, P, NT, -1, LY>(sm, tw);

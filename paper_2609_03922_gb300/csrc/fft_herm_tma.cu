@@ -143,14 +143,14 @@ __global__ void __launch_bounds__(NT, 2)
         HermInBox<L, P> in{sm, smB, smC, kx0, M};
         // the first stage reads the direct and mirror tiles; its barrier between
         // reads and writes frees the mirror buffer for the next tile's copy
-        stockham_stage_in<float, L, P, NT, +1, 1, radix_at<L>(0), LY>(sm, s_tw, in);
+        stockham_stage_in<float, L, P, NT, +1, 1, radix_at<float, L>(0), LY>(sm, s_tw, in);
         if (threadIdx.x == 0 && tn < ntiles) {
             fence_async_smem();
             issue_b(tn);
             out_b = true;
         }
-        run_stage_range<float, L, P, NT, +1, LY, 1, NSTAGES<L>::value - 1>(sm, s_tw);
-        stockham_stage_out<float, L, P, NT, +1, ns_at<L>(NSTAGES<L>::value - 1), radix_at<L>(NSTAGES<L>::value - 1),
+        run_stage_range<float, L, P, NT, +1, LY, 1, NSTAGES<float, L>::value - 1>(sm, s_tw);
+        stockham_stage_out<float, L, P, NT, +1, ns_at<float, L>(NSTAGES<float, L>::value - 1), radix_at<float, L>(NSTAGES<float, L>::value - 1),
                            LY>(sm, s_tw, out);
         __syncthreads();
         buf ^= 1;
