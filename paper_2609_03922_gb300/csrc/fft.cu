@@ -169,6 +169,7 @@ spdba_status make_pass(Pass<T>* out, int64_t L, int sign, int mode, long long O,
         }
     }
     if (generic) ok = get(TILE_GENERIC);
+    if (!ok && (mode == PASS_R2C || mode == PASS_C2R)) return SPDBA_ERR_UNSUPPORTED;   // the caller has another way
     if (!ok) return fail(SPDBA_ERR_UNSUPPORTED, "no FFT pass kernel for length %lld (mode %d)", (long long)L, mode);
     spdba_status s = ensure_smem_attr(ki.func, ki.smem, !generic);
     if (s != SPDBA_OK) return s;
@@ -333,7 +334,7 @@ template spdba_status make_pass<double>(Pass<double>*, int64_t, int, int, long l
                                         cudaStream_t, bool);
 // Half-spectrum passes of a 3-D complex64 field (see fft_half.cuh).
 spdba_status make_half_pass(Pass<float>* out, int mode, const HalfGeo& hg, TwiddleCache<float>& tw, cudaStream_t st) {
-    const bool rows = mode == PASS_NL_HALF;
+    const bool rows = mode == PASS_NL_HALF || mode == PASS_R2C_HALF || mode == PASS_C2R_HALF;
     const int64_t L = rows ? hg.N2 : hg.N0;
     KernelInfo ki;
     if (!get_half_kernel(L, mode, hg.NHP, &ki)) {

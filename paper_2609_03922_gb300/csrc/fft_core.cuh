@@ -853,6 +853,12 @@ enum PassMode : int {
     // PASS_CH_UPDATE, then the inverse transform of the updated c_hat: the last pass of a
     // step and the first of the next in one (fft_chain_kernel)
     PASS_CH_CHAIN = 8,
+    // rows of a real field in (forward) or out (inverse, real parts), the other side complex:
+    // full rows, or rows of the half array
+    PASS_R2C = 9,
+    PASS_C2R = 10,
+    PASS_R2C_HALF = 11,
+    PASS_C2R_HALF = 12,
 };
 constexpr bool is_update_mode(int m) { return m == PASS_CH_UPDATE || m == PASS_UPD_HALF; }
 constexpr bool reads_half(int m) { return m == PASS_MIRROR || m == PASS_UPD_HALF; }

@@ -24,6 +24,8 @@ template <int L, int P, int NT, int OCC> static bool rows(int sign, int mode, Ke
     ki->pipe = false;
     ki->smem = RowLayout<L, P / 2>::SIZE * (int)sizeof(cf32x2);
     ki->func = mode == PASS_CH_NL ? (const void*)fft_rows2_kernel<L, P, NT, -1, PASS_CH_NL, OCC>
+               : mode == PASS_R2C ? (const void*)fft_rows2_kernel<L, P, NT, -1, PASS_R2C, OCC>
+               : mode == PASS_C2R ? (const void*)fft_rows2_kernel<L, P, NT, +1, PASS_C2R, OCC>
                : sign < 0         ? (const void*)fft_rows2_kernel<L, P, NT, -1, PASS_PLAIN, OCC>
                                   : (const void*)fft_rows2_kernel<L, P, NT, +1, PASS_PLAIN, OCC>;
     return true;
@@ -36,7 +38,7 @@ bool get_pass2_kernel(int64_t L, int sign, int mode, bool strided_axis, bool nar
         if (L == 384) return strided<384, 16, 192, 2>(sign, ki);
         return false;
     }
-    if (mode != PASS_PLAIN && mode != PASS_CH_NL) return false;
+    if (mode != PASS_PLAIN && mode != PASS_CH_NL && mode != PASS_R2C && mode != PASS_C2R) return false;
     if (narrow) {
         // four rows a tile
         switch (L) {
@@ -103,21 +105,24 @@ int chain2_step(int64_t L) {
     }
 }
 
-template <int L, int P, int NT, int OCC, bool ST> static bool nl_half(int nhp, KernelInfo* ki) {
+template <int L, int P, int NT, int OCC, bool ST> static bool nl_half(int mode, int nhp, KernelInfo* ki) {
     ki->P = P;
     ki->NT = NT;
     ki->pipe = false;
     const int tile = RowLayout<L, P / 4>::SIZE * (int)sizeof(cf32x2);
-    ki->smem = ST ? std::max(tile, P * nhp * (int)sizeof(float2)) : tile;
-    ki->func = (const void*)fft_nl_half2_kernel<L, P, NT, OCC, ST>;
+    ki->smem = ST && mode != PASS_R2C_HALF ? std::max(tile, P * nhp * (int)sizeof(float2)) : tile;
+    ki->func = mode == PASS_NL_HALF    ? (const void*)fft_nl_half2_kernel<L, P, NT, OCC, ST, PASS_NL_HALF>
+               : mode == PASS_R2C_HALF ? (const void*)fft_nl_half2_kernel<L, P, NT, OCC, ST, PASS_R2C_HALF>
+                                       : (const void*)fft_nl_half2_kernel<L, P, NT, OCC, ST, PASS_C2R_HALF>;
     return true;
 }
-bool get_nl_half2_kernel(int64_t L, int nhp, KernelInfo* ki) {
+bool get_nl_half2_kernel(int64_t L, int mode, int nhp, KernelInfo* ki) {
     switch (L) {
-        case 64: return nl_half<64, 32, 64, 8, false>(nhp, ki);
-        case 128: return nl_half<128, 32, 64, 8, true>(nhp, ki);
-        case 256: return nl_half<256, 32, 128, 5, true>(nhp, ki);
-        case 384: return nl_half<384, 16, 64, 6, true>(nhp, ki);
+        case 64: return nl_half<64, 32, 64, 8, false>(mode, nhp, ki);
+        case 128: return nl_half<128, 32, 64, 8, true>(mode, nhp, ki);
+        case 256: return nl_half<256, 32, 128, 5, true>(mode, nhp, ki);
+        case 384: return nl_half<384, 16, 64, 6, true>(mode, nhp, ki);
+        case 512: return mode != PASS_NL_HALF && nl_half<512, 16, 128, 4, true>(mode, nhp, ki);
         default: return false;
     }
 }

@@ -291,7 +291,36 @@ template <int L> struct RowPairOut {
     }
 };
 
-// MODE: PASS_PLAIN, or PASS_CH_NL (inverse, c = Re / N and g = c^3 - c, forward).
+// Real rows in or out (base: the float field).
+struct RealRowPairIn {
+    static constexpr bool EXT = true;
+    const float* base;
+    int sI;
+    __device__ __forceinline__ void before_write() const {}
+    __device__ __forceinline__ cf32x2 operator()(int p, int m) const {
+        return mk<cf32x2>(f32x2(base[2 * p * sI + m], base[(2 * p + 1) * sI + m]), f32x2(0.f));
+    }
+};
+template <int L> struct RealRowPairOut {
+    static constexpr bool SYNC = false;
+    float* base;
+    int sI;
+    f32x2 scale;
+    __device__ __forceinline__ void pre() {}
+    __device__ __forceinline__ void begin(int, int, int) {}
+    template <int R> __device__ __forceinline__ void emit(int, int p, int j, cf32x2 (&v)[R]) {
+        float* pa = base + (2 * p * sI + j);
+        float* pb = pa + sI;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const f32x2 x = mul_rn(v[r].x, scale);
+            pa[r * (L / R)] = x.lo();
+            pb[r * (L / R)] = x.hi();
+        }
+    }
+};
+
+// MODE: PASS_PLAIN, PASS_R2C / PASS_C2R (real rows in / real parts out), or PASS_CH_NL (inverse, c = Re / N and g = c^3 - c, forward).
 // Measured (rows x length, in place; pipelined one-pencil kernel before): plain
 // 65536 x 256 56.8 -> 51.9 us, 147456 x 384 323 -> 194 us, 32768 x 64 7.6 -> 5.6 us;
 // nonlinear 70.2 -> 60.1, 455 -> 285, 10.0 -> 7.5 us.
@@ -323,6 +352,12 @@ __global__ void __launch_bounds__(NT, OCC) fft_rows2_kernel(PassParams<float> a)
             const double ms = warp_sum((double)mid.msum.lo() + (double)mid.msum.hi());
             if ((threadIdx.x & 31) == 0) atomicAdd(a.mass + (q0 / a.mass_ppr) * a.mass_stride, ms);
         }
+    } else if constexpr (MODE == PASS_R2C) {
+        RealRowPairIn rin{reinterpret_cast<const float*>(a.in) + i0 * a.isI, (int)a.isI};
+        run_stages_in_out<f32x2, L, H, NT, SIGN, LY>(sm, s_tw, rin, out);
+    } else if constexpr (MODE == PASS_C2R) {
+        RealRowPairOut<L> rout{reinterpret_cast<float*>(a.out) + i0 * a.osI, (int)a.osI, f32x2(a.scale)};
+        run_stages_in_out<f32x2, L, H, NT, SIGN, LY>(sm, s_tw, in, rout);
     } else {
         run_stages_in_out<f32x2, L, H, NT, SIGN, LY>(sm, s_tw, in, out);
     }
@@ -399,6 +434,38 @@ struct ChNlQuadMid {
         return mk<cf32x2>(fma_rn(mul_rn(c0, c0), c0, -c0), fma_rn(mul_rn(c1, c1), c1, -c1));
     }
 };
+// Four real rows in: rows 4p .. 4p + 3 as pencils (row, row + 1) of pair p.
+struct QuadRealIn {
+    static constexpr bool EXT = true;
+    const float* base;   // row 0 of the tile, rows of n
+    int n;
+    __device__ __forceinline__ void before_write() const {}
+    __device__ __forceinline__ cf32x2 operator()(int p, int m) const {
+        const float* q = base + (4 * p * n + m);
+        return mk<cf32x2>(f32x2(q[0], q[2 * n]), f32x2(q[n], q[3 * n]));
+    }
+};
+template <int L> struct QuadRealOut {
+    static constexpr bool SYNC = false;
+    float* base;
+    f32x2 scale;
+    __device__ __forceinline__ void pre() {}
+    __device__ __forceinline__ void begin(int, int, int) {}
+    template <int R> __device__ __forceinline__ void emit(int, int p, int j, cf32x2 (&v)[R]) {
+        float* q = base + (4 * p * L + j);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const float4 w = quad_of(cscale(v[r], scale));
+            q[r * (L / R)] = w.x;
+            q[r * (L / R) + L] = w.y;
+            q[r * (L / R) + 2 * L] = w.z;
+            q[r * (L / R) + 3 * L] = w.w;
+        }
+    }
+};
+
+// MODE: PASS_NL_HALF (half rows -> real -> g = c^3 - c -> half rows), PASS_R2C_HALF (real
+// rows -> half rows) or PASS_C2R_HALF (half rows -> real rows).
 // P real rows per tile, P / 4 pencils of the packed transform.  Measured (rows x
 // N2, in place, one thread one pencil before): 65536 x 256 35.3 -> 32.2 us,
 // 147456 x 384 233 -> 161 us, 65536 x 128 22.0 -> 18.7 us, 4096 x 64 3.7 -> 2.8 us;
@@ -406,7 +473,7 @@ struct ChNlQuadMid {
 // and fft_nl_half_kernel stays.
 // ST: the tile's rows are staged in shared memory (the transform then works over
 // them); else the packed elements are read from global memory, each row twice.
-template <int L, int P, int NT, int OCC, bool ST>
+template <int L, int P, int NT, int OCC, bool ST, int MODE = PASS_NL_HALF>
 __global__ void __launch_bounds__(NT, OCC) fft_nl_half2_kernel(PassParams<float> a) {
     pdl_wait();
     constexpr int H = P / 4, M = L / 2;
@@ -419,7 +486,7 @@ __global__ void __launch_bounds__(NT, OCC) fft_nl_half2_kernel(PassParams<float>
     dup_twiddles<L, NT>(s_tw, a.tw);
     const float2* src = a.in + q0 * NHP;
     float2* rows = reinterpret_cast<float2*>(smem_raw);
-    if constexpr (ST) {
+    if constexpr (ST && MODE != PASS_R2C_HALF) {
         for (int u = threadIdx.x; u < P * NHP / 2; u += NT) cp_async16(rows + 2 * u, src + 2 * u);
         cp_async_commit();
         cp_async_wait<0>();
@@ -429,7 +496,16 @@ __global__ void __launch_bounds__(NT, OCC) fft_nl_half2_kernel(PassParams<float>
     QuadPackIn<L, !ST> in{src, NHP, a.hg.r2c != 0};
     ChNlQuadMid mid{f32x2(a.nl_scale), f32x2(0.f)};
     SmemOut2<L, LY> so{sm};
-    transform_pair_in<f32x2, L, H, NT, +1, -1, LY>(sm, s_tw, in, mid, so);
+    if constexpr (MODE == PASS_C2R_HALF) {
+        QuadRealOut<L> out{reinterpret_cast<float*>(a.out) + q0 * L, f32x2(a.nl_scale)};
+        run_stages_in_out<f32x2, L, H, NT, +1, LY>(sm, s_tw, in, out);
+        return;
+    } else if constexpr (MODE == PASS_R2C_HALF) {
+        QuadRealIn rin{reinterpret_cast<const float*>(a.in) + q0 * L, L};
+        run_stages_in_out<f32x2, L, H, NT, -1, LY>(sm, s_tw, rin, so);
+    } else {
+        transform_pair_in<f32x2, L, H, NT, +1, -1, LY>(sm, s_tw, in, mid, so);
+    }
     __syncthreads();
     // the two rows' half spectra of each transform: G1[k] = (W[k] + conj W[-k]) / 2,
     // G2[k] = (W[k] - conj W[-k]) / (2i), two entries of four rows an item (padding

@@ -67,8 +67,9 @@ template <int N2> static bool pick_x(int nhp, KernelInfo* ki) {
 
 bool get_half_kernel(int64_t L, int mode, int nhp, KernelInfo* ki) {
     if (mode == PASS_NL_HALF) {   // L = N2, the full row length
-        return L == 512 ? pick_x<512>(nhp, ki) : get_nl_half2_kernel(L, nhp, ki);
+        return L == 512 ? pick_x<512>(nhp, ki) : get_nl_half2_kernel(L, mode, nhp, ki);
     }
+    if (mode == PASS_R2C_HALF || mode == PASS_C2R_HALF) return get_nl_half2_kernel(L, mode, nhp, ki);
     if (mode == PASS_PAIR_MIRROR) {
         switch (L) {
             case 64: return pick_pair<64>(ki);

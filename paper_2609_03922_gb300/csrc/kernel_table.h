@@ -20,7 +20,7 @@ bool get_pass2_kernel(int64_t L, int sign, int mode, bool strided, bool narrow, 
 // rows in, transposed out (unit-stride pencils on the output)
 bool get_transpose2_kernel(int64_t L, int sign, KernelInfo* ki);
 bool get_chain2_kernel(int64_t L, bool narrow, KernelInfo* ki);
-bool get_nl_half2_kernel(int64_t L, int nhp, KernelInfo* ki);
+bool get_nl_half2_kernel(int64_t L, int mode, int nhp, KernelInfo* ki);
 // the step chain (PASS_CH_CHAIN) along the first axis
 template <typename T> bool get_chain_kernel(int64_t L, bool narrow, KernelInfo* ki);
 // complex64 half-spectrum passes (PASS_HERM_INV, PASS_NL_HALF, PASS_MIRROR,

@@ -12,7 +12,8 @@ template <typename T> struct HPair {
 };
 
 template <typename T> struct NLSArgs {
-    cx_t<T>* S;                 // spectra of `batch` signals of n samples
+    cx_t<T>* S;                 // spectra of `batch` signals of n samples (a pass's output)
+    const cx_t<T>* in;          // a row or column pass's input (S within a step)
     const HPair<T>* H;          // n entries: natural order (short), H(k1 + n1 m) at k1 * 512 + m (long)
     const uint8_t* states;      // batch * nblk
     const uint8_t* chi;

@@ -27,29 +27,6 @@ template <typename T> __global__ void real_to_complex_kernel(const T* __restrict
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         c[i] = mk<cx_t<T>>(r[i], (T)0);
 }
-// Full spectrum (N0 x N1 x N2) of a half-stored one (kx = 0 .. N2/2 in rows of
-// NHP entries): kx > N2/2 from X(k) = conj X(-k) (Eq. S.4).
-template <typename T>
-__global__ void half_storage_extend_kernel(const cx_t<T>* __restrict__ h, cx_t<T>* __restrict__ full, int N0, int N1,
-                                           int N2, int NHP) {
-    pdl_wait();
-    const long long n = (long long)N0 * N1 * N2;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % N2);
-        const long long zy = i / N2;
-        const int y = (int)(zy % N1), z = (int)(zy / N1);
-        cx_t<T> v;
-        if (x <= N2 / 2) {
-            v = h[zy * NHP + x];
-        } else {
-            const int my = y == 0 ? 0 : N1 - y, mz = z == 0 ? 0 : N0 - z;
-            v = h[((long long)mz * N1 + my) * NHP + (N2 - x)];
-            v.y = -v.y;
-        }
-        full[i] = v;
-    }
-}
-
 template <typename T> __global__ void complex_real_part_kernel(const cx_t<T>* __restrict__ c, T* __restrict__ r, long long n) {
     pdl_wait();
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -73,8 +50,12 @@ __global__ void ratio_kernel(DevStats* stats, long long nruns, long long bpr, lo
     }
 }
 // Statistics of runs [0, n) reset, with the threshold coefficient in force set to eps.
-__global__ void stats_reset_kernel(DevStats* stats, long long n, double eps) {
+// and their block states, if given, all ACTIVE (nst of them).
+__global__ void stats_reset_kernel(DevStats* stats, long long n, double eps, uint8_t* states, long long nst) {
     pdl_wait();
+    for (long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x; b < nst; b += (long long)gridDim.x * blockDim.x)
+        states[b] = SPDBA_ACTIVE;
+    if (blockIdx.x != 0) return;
     for (long long r = threadIdx.x; r < n; r += blockDim.x) {
         stats[r] = DevStats{};
         stats[r].eps = eps;
@@ -179,6 +160,10 @@ template <typename T> struct Group {
     bool has_chain = false;
     bool pre_done = false;          // `work` holds the first inverse pass of c_hat (set by the chain, within a call)
     FftEngine<T> fft1;              // one run's transforms for set/get_field
+    // ... whose passes along the rows take the real field in and give it out (complex64; the
+    // half array's rows with half-spectrum storage)
+    Pass<T> r2c, c2r;
+    bool has_real_rows = false;
     // NLS
     HPair<T>* H = nullptr;
     T* ntaper = nullptr;
@@ -409,11 +394,24 @@ template <typename T> static spdba_status group_buffers(spdba_plan* p, Group<T>&
     if ((s = r.alloc(&r.scratch, classify_scratch_bytes(nb))) != SPDBA_OK) return s;
     if ((s = r.alloc(&r.stats, sizeof(DevStats) * r.batch)) != SPDBA_OK) return s;
     SPDBA_CUDA(cudaMemsetAsync(r.c_hat, 0, sizeof(cx_t<T>) * tot, st));
-    pdl_launch(stats_reset_kernel, 1, 256, 0, st, r.stats, r.batch, p->threshold);
+    pdl_launch(stats_reset_kernel, 1, 256, 0, st, r.stats, r.batch, p->threshold, nullptr, 0);
     SPDBA_CUDA(cudaGetLastError());
     SPDBA_CUDA(cudaMemsetAsync(r.gmax, 0, sizeof(double) * 2 * r.batch, st));
     SPDBA_CUDA(cudaMemsetAsync(r.states, SPDBA_ACTIVE, nb, st));
     SPDBA_CUDA(cudaMemsetAsync(r.chi, 0, nb, st));
+    return SPDBA_OK;
+}
+
+// The passes of set_field / get_field between a run's real field (runs fields of
+// extents d) and its complex rows, where kernels exist.
+static spdba_status setup_real_rows(spdba_plan* p, Group<float>& r, const FftEngine<float>& e, int nd, const int64_t* d,
+                                    long long fields) {
+    spdba_status s = make_axis_pass<float>(&r.r2c, nd, d, fields, nd - 1, -1, PASS_R2C, p->tw32, p->st);
+    if (s == SPDBA_OK) s = make_axis_pass<float>(&r.c2r, nd, d, fields, nd - 1, +1, PASS_C2R, p->tw32, p->st);
+    if (s == SPDBA_ERR_UNSUPPORTED) return SPDBA_OK;
+    if (s != SPDBA_OK) return s;
+    r.c2r.p.scale = e.inv.back().p.scale;
+    r.has_real_rows = true;
     return SPDBA_OK;
 }
 
@@ -581,13 +579,15 @@ static spdba_status group_init_ch_hs(spdba_plan* p, Group<float>& r, const int64
         if ((s = upload(r, &r.taper[ax], taper_table<float>(r.g.b[ax]), st)) != SPDBA_OK) return s;
     }
     TwiddleCache<float>& tw = p->tw32;
-    if ((s = r.fft1.init(3, dims, 1, tw, st)) != SPDBA_OK) return s;
     HalfGeo hg;
     hg.N0 = (int)N0; hg.N1 = (int)N1; hg.N2 = (int)N2; hg.NHP = (int)NHP;
     hg.fd_N2.init((uint32_t)N2);
     hg.fd_NHP.init((uint32_t)NHP);
     hg.fd_M.init((uint32_t)M);
     hg.r2c = 1;
+    if ((s = make_half_pass(&r.r2c, PASS_R2C_HALF, hg, tw, st)) != SPDBA_OK) return s;
+    if ((s = make_half_pass(&r.c2r, PASS_C2R_HALF, hg, tw, st)) != SPDBA_OK) return s;
+    r.has_real_rows = true;
     if ((s = make_axis_pass<float>(&r.h_inv_z, 3, dh, 1, 0, +1, PASS_PLAIN, tw, st)) != SPDBA_OK) return s;
     if ((s = make_axis_pass<float>(&r.h_inv_y, 3, dh, 1, 1, +1, PASS_PLAIN, tw, st)) != SPDBA_OK) return s;
     if ((s = make_half_pass(&r.h_nl, PASS_NL_HALF, hg, tw, st)) != SPDBA_OK) return s;
@@ -650,6 +650,8 @@ static spdba_status group_init_ch(spdba_plan* p, Group<T>& r, int ndim, const in
     }
     TwiddleCache<T>& tw = twc<T>(p);
     if ((s = r.fft1.init(ndim, dims, 1, tw, st)) != SPDBA_OK) return s;
+    if constexpr (std::is_same<T, float>::value)
+        if ((s = setup_real_rows(p, r, r.fft1, ndim, dims, 1)) != SPDBA_OK) return s;
     // inverse along axes 0..d-2, fused inverse/NL/forward along d-1, forward d-2..0
     for (int a = 0; a < ndim - 1; ++a) {
         Pass<T> ps;
@@ -827,6 +829,7 @@ static spdba_status group_init_rcd(spdba_plan* p, Group<T>& r, int ndim, const i
     if ((s = upload(r, &r.rcd_V, std::vector<T>(V.begin(), V.end()), st)) != SPDBA_OK) return s;
     if ((s = upload(r, &r.rcd_lam, std::vector<T>(lam.begin(), lam.end()), st)) != SPDBA_OK) return s;
     if constexpr (std::is_same<T, float>::value) {
+        if ((s = setup_real_rows(p, r, r.rcd_fft, ndim, dims, M)) != SPDBA_OK) return s;
         if ((s = rcd_pack_prepare(&r.rcd_pack, ndim, dims, M, p->tw32, st)) != SPDBA_OK) return s;
         if (r.rcd_pack.ok) {
             // inverse: rows (with the packing), then the other axes from the last; forward back
@@ -1190,6 +1193,7 @@ template <typename T> static spdba_status ch_staged_update(spdba_plan* p, Group<
 template <typename T> static NLSArgs<T> nls_args(spdba_plan* p, Group<T>& r, cx_t<T>* S, long long batch, int dense) {
     NLSArgs<T> a{};
     a.S = S;
+    a.in = S;
     a.H = r.H;
     a.states = r.states;
     a.chi = r.chi;
@@ -1662,46 +1666,60 @@ static spdba_status run_set_field(spdba_plan* p, Group<T>& r, long long sub, con
     cx_t<T>* slot = r.c_hat + sub * r.n;
     cx_t<T>* wslot = r.work + sub * r.n;
     const cudaMemcpyKind kind = on_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    if (p->opt.model == SPDBA_MODEL_RCD) {
+    if (p->opt.model != SPDBA_MODEL_NLS) {
+        const bool rcd = p->opt.model == SPDBA_MODEL_RCD;
         const long long tot = r.n * r.ncomp;
-        SPDBA_CUDA(cudaMemcpyAsync(r.real, src, sizeof(T) * tot, kind, st));
-        pdl_launch(real_to_complex_kernel<T>, grid_for(tot, 256), 256, 0, st, r.real, r.work, tot);
-        if ((s = r.rcd_fft.exec(r.work, r.c_hat, SPDBA_FORWARD, st)) != SPDBA_OK) return s;
-    } else if (p->opt.model == SPDBA_MODEL_CH) {
-        SPDBA_CUDA(cudaMemcpyAsync(r.real, src, sizeof(T) * r.n, kind, st));
-        pdl_launch(real_to_complex_kernel<T>, grid_for(r.n, 256), 256, 0, st, r.real, wslot, r.n);
-        if ((s = r.fft1.exec(wslot, slot, SPDBA_FORWARD, st)) != SPDBA_OK) return s;
-        if (r.hs) {
-            // keep the half kx = 0 .. N2/2 of the full spectrum, rows padded with zeros
-            const size_t es = sizeof(cx_t<T>);
-            const int64_t N2 = r.dims[2];
-            SPDBA_CUDA(cudaMemsetAsync(r.work, 0, es * (size_t)r.hs_n, st));
-            SPDBA_CUDA(cudaMemcpy2DAsync(r.work, es * (size_t)r.hs_nhp, r.c_hat, es * (size_t)N2,
-                                         es * (size_t)(N2 / 2 + 1), (size_t)(r.dims[0] * r.dims[1]),
-                                         cudaMemcpyDeviceToDevice, st));
-            SPDBA_CUDA(cudaMemcpyAsync(r.c_hat, r.work, es * (size_t)r.hs_n, cudaMemcpyDeviceToDevice, st));
+        const T* field = reinterpret_cast<const T*>(src);
+        if (!on_dev || !r.has_real_rows) {
+            SPDBA_CUDA(cudaMemcpyAsync(r.real, src, sizeof(T) * tot, kind, st));
+            field = r.real;
         }
-    } else if (!r.long_nls) {
-        SPDBA_CUDA(cudaMemcpyAsync(wslot, src, sizeof(cx_t<T>) * r.n, kind, st));
-        if ((s = r.fft1.exec(wslot, slot, SPDBA_FORWARD, st)) != SPDBA_OK) return s;
+        if (r.hs) {
+            // rows of the half array from the real rows, then y and z
+            if ((s = launch_pass<T>(r.r2c, field, r.work, st)) != SPDBA_OK) return s;
+            if ((s = launch_pass<T>(r.h_fwd_y, r.work, r.work, st)) != SPDBA_OK) return s;
+            if ((s = launch_pass<T>(r.h_mirror, r.work, r.c_hat, st)) != SPDBA_OK) return s;
+        } else {
+            FftEngine<T>& e = rcd ? r.rcd_fft : r.fft1;
+            if (r.has_real_rows) {
+                // the engine's first pass (the rows) reads the real field
+                if ((s = launch_pass<T>(r.r2c, field, slot, st)) != SPDBA_OK) return s;
+                for (size_t k = 1; k < e.fwd.size(); ++k)
+                    if ((s = launch_pass<T>(e.fwd[k], slot, slot, st)) != SPDBA_OK) return s;
+            } else {
+                pdl_launch(real_to_complex_kernel<T>, grid_for(tot, 256), 256, 0, st, field, wslot, tot);
+                if ((s = e.exec(wslot, slot, SPDBA_FORWARD, st)) != SPDBA_OK) return s;
+            }
+        }
     } else {
-        // E (natural time order) -> column pass (forward) -> row pass (forward): S in transposed order
-        SPDBA_CUDA(cudaMemcpyAsync(slot, src, sizeof(cx_t<T>) * r.n, kind, st));
-        NLSArgs<T> a = nls_args<T>(p, r, slot, 1, 1);
-        a.tw = r.tw_col;
-        a.do_inv = 0; a.do_kerr = 0; a.do_fwd = 1;
-        if ((s = nls_col_pass<T>(a, r.nl, st)) != SPDBA_OK) return s;
-        a.tw = r.tw_row;
-        a.do_fwd = 1; a.do_close = 0; a.do_open = 0; a.do_inv = 0;
-        if ((s = nls_row_pass<T>(a, r.nl, st)) != SPDBA_OK) return s;
+        // a device signal on a 16-byte boundary is read where it lies
+        const cx_t<T>* from = reinterpret_cast<const cx_t<T>*>(src);
+        if (!on_dev || ((uintptr_t)src & 15)) {
+            SPDBA_CUDA(cudaMemcpyAsync(wslot, src, sizeof(cx_t<T>) * r.n, kind, st));
+            from = wslot;
+        }
+        if (!r.long_nls) {
+            if ((s = r.fft1.exec(from, slot, SPDBA_FORWARD, st)) != SPDBA_OK) return s;
+        } else {
+            // E (natural time order) -> column pass (forward) -> row pass (forward): S in transposed order
+            NLSArgs<T> a = nls_args<T>(p, r, slot, 1, 1);
+            a.in = from;
+            a.tw = r.tw_col;
+            a.do_inv = 0; a.do_kerr = 0; a.do_fwd = 1;
+            if ((s = nls_col_pass<T>(a, r.nl, st)) != SPDBA_OK) return s;
+            a.in = slot;
+            a.tw = r.tw_row;
+            a.do_fwd = 1; a.do_close = 0; a.do_open = 0; a.do_inv = 0;
+            if ((s = nls_row_pass<T>(a, r.nl, st)) != SPDBA_OK) return s;
+        }
     }
     r.step = 0;
     r.assessed = false;
     r.has_snap = false;
     r.has_pred = false;
-    pdl_launch(stats_reset_kernel, 1, 32, 0, st, r.stats + sub, 1, p->threshold);
+    pdl_launch(stats_reset_kernel, grid_for(r.g.bpr(), 256 * 16), 256, 0, st, r.stats + sub, 1, p->threshold,
+               r.states + sub * r.g.bpr(), r.g.bpr());
     SPDBA_CUDA(cudaGetLastError());
-    SPDBA_CUDA(cudaMemsetAsync(r.states + sub * r.g.bpr(), SPDBA_ACTIVE, r.g.bpr(), st));
     return SPDBA_OK;
 }
 
@@ -1712,34 +1730,47 @@ static spdba_status run_get_field(spdba_plan* p, Group<T>& r, long long sub, voi
     cx_t<T>* slot = r.c_hat + sub * r.n;
     cx_t<T>* wslot = r.work + sub * r.n;
     const cudaMemcpyKind kind = on_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
-    if (p->opt.model == SPDBA_MODEL_RCD) {
+    if (p->opt.model != SPDBA_MODEL_NLS) {
+        const bool rcd = p->opt.model == SPDBA_MODEL_RCD;
         const long long tot = r.n * r.ncomp;
-        if ((s = r.rcd_fft.exec(r.c_hat, r.work, SPDBA_INVERSE, st)) != SPDBA_OK) return s;
-        pdl_launch(complex_real_part_kernel<T>, grid_for(tot, 256), 256, 0, st, r.work, r.real, tot);
-        SPDBA_CUDA(cudaMemcpyAsync(dst, r.real, sizeof(T) * tot, kind, st));
-    } else if (p->opt.model == SPDBA_MODEL_CH) {
+        // the row passes write the real field: to the caller's buffer, or staged for the host
+        T* field = on_dev && r.has_real_rows ? reinterpret_cast<T*>(dst) : r.real;
         if (r.hs) {
-            pdl_launch(half_storage_extend_kernel<T>, grid_for(r.n, 256), 256, 0, st, 
-                r.c_hat, r.work, (int)r.dims[0], (int)r.dims[1], (int)r.dims[2], (int)r.hs_nhp);
-            if ((s = r.fft1.exec(r.work, wslot, SPDBA_INVERSE, st)) != SPDBA_OK) return s;
-        } else if ((s = r.fft1.exec(slot, wslot, SPDBA_INVERSE, st)) != SPDBA_OK) {
-            return s;
+            if ((s = launch_pass<T>(r.h_inv_z, r.c_hat, r.work, st)) != SPDBA_OK) return s;
+            if ((s = launch_pass<T>(r.h_inv_y, r.work, r.work, st)) != SPDBA_OK) return s;
+            if ((s = launch_pass<T>(r.c2r, r.work, field, st)) != SPDBA_OK) return s;
+        } else {
+            FftEngine<T>& e = rcd ? r.rcd_fft : r.fft1;
+            if (r.has_real_rows) {
+                const cx_t<T>* from = slot;
+                for (size_t k = 0; k + 1 < e.inv.size(); ++k) {
+                    if ((s = launch_pass<T>(e.inv[k], from, wslot, st)) != SPDBA_OK) return s;
+                    from = wslot;
+                }
+                if ((s = launch_pass<T>(r.c2r, from, field, st)) != SPDBA_OK) return s;
+            } else {
+                if ((s = e.exec(slot, wslot, SPDBA_INVERSE, st)) != SPDBA_OK) return s;
+                pdl_launch(complex_real_part_kernel<T>, grid_for(tot, 256), 256, 0, st, wslot, r.real, tot);
+            }
         }
-        pdl_launch(complex_real_part_kernel<T>, grid_for(r.n, 256), 256, 0, st, wslot, r.real, r.n);
-        SPDBA_CUDA(cudaMemcpyAsync(dst, r.real, sizeof(T) * r.n, kind, st));
-    } else if (!r.long_nls) {
-        if ((s = r.fft1.exec(slot, wslot, SPDBA_INVERSE, st)) != SPDBA_OK) return s;
-        SPDBA_CUDA(cudaMemcpyAsync(dst, wslot, sizeof(cx_t<T>) * r.n, kind, st));
+        if (field == r.real) SPDBA_CUDA(cudaMemcpyAsync(dst, r.real, sizeof(T) * tot, kind, st));
     } else {
-        SPDBA_CUDA(cudaMemcpyAsync(wslot, slot, sizeof(cx_t<T>) * r.n, cudaMemcpyDeviceToDevice, st));
-        NLSArgs<T> a = nls_args<T>(p, r, wslot, 1, 1);
-        a.tw = r.tw_row;
-        a.do_fwd = 0; a.do_close = 0; a.do_open = 0; a.do_inv = 1;
-        if ((s = nls_row_pass<T>(a, r.nl, st)) != SPDBA_OK) return s;
-        a.tw = r.tw_col;
-        a.do_inv = 1; a.do_kerr = 0; a.do_fwd = 0;
-        if ((s = nls_col_pass<T>(a, r.nl, st)) != SPDBA_OK) return s;
-        SPDBA_CUDA(cudaMemcpyAsync(dst, wslot, sizeof(cx_t<T>) * r.n, kind, st));
+        cx_t<T>* to = on_dev && ((uintptr_t)dst & 15) == 0 ? reinterpret_cast<cx_t<T>*>(dst) : wslot;
+        if (!r.long_nls) {
+            if ((s = r.fft1.exec(slot, to, SPDBA_INVERSE, st)) != SPDBA_OK) return s;
+        } else {
+            NLSArgs<T> a = nls_args<T>(p, r, wslot, 1, 1);
+            a.in = slot;
+            a.tw = r.tw_row;
+            a.do_fwd = 0; a.do_close = 0; a.do_open = 0; a.do_inv = 1;
+            if ((s = nls_row_pass<T>(a, r.nl, st)) != SPDBA_OK) return s;
+            a.in = wslot;
+            a.S = to;
+            a.tw = r.tw_col;
+            a.do_inv = 1; a.do_kerr = 0; a.do_fwd = 0;
+            if ((s = nls_col_pass<T>(a, r.nl, st)) != SPDBA_OK) return s;
+        }
+        if (to == wslot) SPDBA_CUDA(cudaMemcpyAsync(dst, wslot, sizeof(cx_t<T>) * r.n, kind, st));
     }
     SPDBA_CUDA(cudaStreamSynchronize(st));
     return SPDBA_OK;
