@@ -29,6 +29,7 @@ template <typename T> struct NLSArgs {
     T gamma_h, inv_n;
     double* power;              // per-signal FP64 sum |E|^2 accumulators (strided) or null
     int power_stride;
+    DevStats* stats = nullptr;  // the runs' statistics, counted by the step's column (or single) kernel, or null
     int do_fwd, do_close, do_open, do_inv, do_kerr;
 };
 

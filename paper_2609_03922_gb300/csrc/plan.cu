@@ -36,19 +36,6 @@ __global__ void zero_strided_kernel(double* p, long long n, int stride) {
     pdl_wait();
     for (long long i = threadIdx.x; i < n; i += blockDim.x) p[i * stride] = 0.0;
 }
-// per-run share of non-frozen blocks for one step (1 on all-active steps)
-__global__ void ratio_kernel(DevStats* stats, long long nruns, long long bpr, long long bmodes, int dense) {
-    pdl_wait();
-    for (long long r = threadIdx.x; r < nruns; r += blockDim.x) {
-        double nf = dense ? (double)bpr : (double)(stats[r].n_active + stats[r].n_transition);
-        stats[r].ratio_sum += nf / (double)bpr;
-        if (!dense) {
-            stats[r].list_modes += nf * (double)bmodes;
-            stats[r].ctl_nf += stats[r].n_active + stats[r].n_transition;   // control interval
-            stats[r].ctl_steps += 1;
-        }
-    }
-}
 // Statistics of runs [0, n) reset, with the threshold coefficient in force set to eps.
 // and their block states, if given, all ACTIVE (nst of them).
 __global__ void stats_reset_kernel(DevStats* stats, long long n, double eps, uint8_t* states, long long nst) {
@@ -1254,6 +1241,7 @@ template <typename T> static spdba_status group_nls_steps(spdba_plan* p, Group<T
             if ((s = row_pass<T>(p, r, a, merge ? 1 : 0, merge ? 1 : 0, 1, 1)) != SPDBA_OK) return s;
             NLSArgs<T> c = a;
             c.tw = r.tw_col;
+            c.stats = r.stats;
             if (reassess) {
                 pdl_launch(zero_strided_kernel, 1, 256, 0, st, &r.stats[0].mass, r.batch, a.power_stride);
                 c.power = &r.stats[0].mass;
@@ -1265,13 +1253,11 @@ template <typename T> static spdba_status group_nls_steps(spdba_plan* p, Group<T
                 pdl_launch(zero_strided_kernel, 1, 256, 0, st, &r.stats[0].mass, r.batch, a.power_stride);
                 a.power = &r.stats[0].mass;
             }
+            a.stats = r.stats;
             ProfScope pr(p, K_NLS_STEP, 2.0 * sizeof(cx_t<T>) * (double)(r.batch * r.n));
             if ((s = nls_small_step<T>(a, r.nl, st)) != SPDBA_OK) return s;
             p->launches += 1;
         }
-        pdl_launch(ratio_kernel, 1, 256, 0, st, r.stats, r.batch, r.g.bpr(), r.g.block_modes(), dense);
-        SPDBA_CUDA(cudaGetLastError());
-        p->launches += 1;
         prev_dense = dense;
         r.step += 1;
     }
