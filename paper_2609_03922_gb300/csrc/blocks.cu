@@ -62,11 +62,18 @@ __device__ __forceinline__ double bitsd(unsigned long long b) { return __longlon
 // before or after it); below 2^-99 every nonzero mode is evaluated, and
 // exactly-zero modes never need it.  The running max rises in few chunks, so
 // about one mode in a chunk reaches the slow FP64 pipe; the rest costs two
-// FP32 operations and a compare, and nothing crosses lanes until the end.  The
+// FP32 operations and a compare, and nothing crosses lanes until the end.  Nor is
+// every such mode evaluated at once: where a chunk has a single candidate that
+// exceeds everything before it by more than the screen's error, it becomes the
+// lane's pending mode and the former one is dropped unevaluated (it cannot be the
+// maximum); the pending mode is evaluated at the end.  FP64 work is left for near
+// ties and for modes below 2^-99.  The
 // field's k = 0 mode is kept out of the screen and taken apart, so that the
 // max over k != 0 is exact as well.
 __device__ __forceinline__ float screen_sq(float2 q) { return fmaf(q.x, q.x, q.y * q.y); }
 constexpr float kScreen99 = 1.5777218104420236e-30f;   // 2^-99
+// (1 + 2^-18): a screen value above another by more exceeds it exactly
+constexpr float kScreenAbove = 1.0f + 3.814697265625e-06f;
 __device__ __forceinline__ bool nonzero_mode(float2 v) {
     return ((__float_as_uint(v.x) | __float_as_uint(v.y)) << 1) != 0u;
 }
@@ -84,7 +91,7 @@ __global__ void __launch_bounds__(256) block_activity_kernel(Geom g, const cx_t<
     const long long run = blk / g.bpr();
     const long long dc = run * g.fmodes();   // the field's k = 0 mode
     const long long base = ((b0 * B0) * g.n[1] + b1 * B1) * g.n[2] + b2 * B2;
-    double mx = 0.0, mxnd = 0.0, sm = 0.0;
+    double mx = 0.0, mxnd = 0.0, sm = 0.0, sm1 = 0.0;
     if constexpr (sizeof(cx_t<T>) == 8) {
         // chunks of up to 16 modes per lane, as 8 16-byte loads of mode pairs along
         // the fast axis (B2 is even for every supported block), all issued before
@@ -94,6 +101,7 @@ __global__ void __launch_bounds__(256) block_activity_kernel(Geom g, const cx_t<
         const int npair = B0 * B1 * H;
         constexpr int K2 = 8;
         float S = 0.f;
+        float2 pend = make_float2(0.f, 0.f);   // pending candidate
         double Ddc = 0.0;   // |q(k = 0)|^2: pair 0 of the block holding it (lane 0)
         if (lane == 0 && base == dc) Ddc = mode_sq(q[dc]);
         for (int m0 = 0; m0 < npair; m0 += 32 * K2) {
@@ -119,8 +127,10 @@ __global__ void __launch_bounds__(256) block_activity_kernel(Geom g, const cx_t<
                 v[2 * k] = make_float2(w[k].x, w[k].y);
                 v[2 * k + 1] = make_float2(w[k].z, w[k].w);
                 if (ENERGY) {
-                    sm += mode_sq(v[2 * k]);
-                    sm += mode_sq(v[2 * k + 1]);
+                    // exact products: a mode's two squares are added with a rounding each, as before
+                    const double x0 = v[2 * k].x, y0 = v[2 * k].y, x1 = v[2 * k + 1].x, y1 = v[2 * k + 1].y;
+                    sm = __fma_rn(x0, x0, __fma_rn(y0, y0, sm));
+                    sm1 = __fma_rn(x1, x1, __fma_rn(y1, y1, sm1));
                 }
                 if (isdc[k]) v[2 * k] = make_float2(0.f, 0.f);   // k = 0: out of the screen
             }
@@ -130,12 +140,14 @@ __global__ void __launch_bounds__(256) block_activity_kernel(Geom g, const cx_t<
                 p32[k] = screen_sq(v[k]);
                 cm = fmaxf(cm, p32[k]);
             }
+            const float before = S;
             S = cm;
             const float cut = S >= kScreen99 ? S * (1.0f - 9.5367431640625e-07f) : 0.f;
             unsigned mask = 0;
 #pragma unroll
             for (int k = 0; k < 2 * K2; ++k)
                 if (p32[k] >= cut && nonzero_mode(v[k])) mask |= 1u << k;   // exact zeros cannot raise the max
+            const bool alone = S >= kScreen99 && cm > before * kScreenAbove && (mask & (mask - 1)) == 0;
             while (mask) {
                 const int i = __ffs(mask) - 1;
                 mask &= mask - 1;
@@ -143,9 +155,11 @@ __global__ void __launch_bounds__(256) block_activity_kernel(Geom g, const cx_t<
 #pragma unroll
                 for (int k = 1; k < 2 * K2; ++k)
                     if (i == k) c = v[k];
-                mxnd = fmax(mxnd, mode_sq(c));
+                if (alone) pend = c;
+                else mxnd = fmax(mxnd, mode_sq(c));
             }
         }
+        mxnd = fmax(mxnd, mode_sq(pend));
         mx = fmax(mxnd, Ddc);
     } else {
         const int nmodes = B0 * B1 * B2;
@@ -161,7 +175,7 @@ __global__ void __launch_bounds__(256) block_activity_kernel(Geom g, const cx_t<
     }
     mx = bitsd(warp_max_u64(dbits(mx)));
     mxnd = bitsd(warp_max_u64(dbits(mxnd)));
-    if (ENERGY) sm = warp_sum(sm);
+    if (ENERGY) sm = warp_sum(sm + sm1);
     if (lane == 0) {
         maxsq[blk] = mx;
         if (ENERGY) sumsq[blk] = sm;
@@ -176,14 +190,20 @@ __global__ void __launch_bounds__(256) block_activity_kernel(Geom g, const cx_t<
 // one mode pair column 2u, so it stays in one block bx = 2u / B2 throughout;
 // its modes are one part of the block for the screen above.  The G = B2 / 2
 // lanes of a block and the row groups combine at the end.
+// Two CTA sizes: seven CTAs of 128 threads are resident per SM, so a map of 1024 rows
+// of blocks runs in one round over 152 SMs, where three CTAs of 256 take three
+// rounds, the last a quarter full; the launch takes the one of fewer row trips.
 constexpr int ROWACT_NT = 256;
-__global__ void __launch_bounds__(ROWACT_NT) block_activity_rows_kernel(Geom g, const float2* __restrict__ q,
-                                                                         double* __restrict__ maxsq,
-                                                                         double* __restrict__ gmax) {
+constexpr int ROWACT_U = 8;   // row trips in flight
+template <int NT> constexpr int rowact_ctas() { return NT == 256 ? 3 : 7; }
+template <int NT>
+__global__ void __launch_bounds__(NT, rowact_ctas<NT>()) block_activity_rows_kernel(Geom g, const float2* __restrict__ q,
+                                                                                    double* __restrict__ maxsq,
+                                                                                    double* __restrict__ gmax) {
     pdl_wait();
-    __shared__ unsigned long long s_mx[ROWACT_NT], s_mxnd[ROWACT_NT];
+    __shared__ unsigned long long s_mx[NT], s_mxnd[NT];
     const int n2 = (int)g.n[2], half = n2 >> 1;          // mode pairs per row
-    const int rpi = ROWACT_NT / half;                      // rows per iteration (threads beyond rpi rows idle)
+    const int rpi = NT / half;                             // rows per iteration (threads beyond rpi rows idle)
     const int u = threadIdx.x % half, rho = threadIdx.x / half;
     const int b0 = blockIdx.x / (int)g.nb[1], b1 = blockIdx.x - b0 * (int)g.nb[1];
     const int B0 = g.b[0], B1 = g.b[1], B2 = g.b[2];
@@ -198,7 +218,8 @@ __global__ void __launch_bounds__(ROWACT_NT) block_activity_rows_kernel(Geom g, 
     double D = 0.0;       // exact max of this lane's k != 0 modes
     double Ddc = 0.0;     // |q(k = 0)|^2, in the lane that holds it (row 0, pair 0)
     if (rho == 0 && rowbase == dc) Ddc = mode_sq(q[dc]);
-    constexpr int U = 8;
+    constexpr int U = ROWACT_U;
+    float2 pend = make_float2(0.f, 0.f);   // pending candidate (screen value at most S)
     for (int r0 = rho; rho < rpi && r0 < rows; r0 += U * rpi) {
         float4 w[U];
         bool isdc[U];
@@ -229,12 +250,14 @@ __global__ void __launch_bounds__(ROWACT_NT) block_activity_rows_kernel(Geom g, 
             p[k] = screen_sq(v[k]);
             cm = fmaxf(cm, p[k]);
         }
+        const float before = S;
         S = cm;
         const float cut = S >= kScreen99 ? S * (1.0f - 9.5367431640625e-07f) : 0.f;
         unsigned mask = 0;
 #pragma unroll
         for (int k = 0; k < 2 * U; ++k)
             if (p[k] >= cut && nonzero_mode(v[k])) mask |= 1u << k;   // exact zeros (padding) cannot raise the max
+        const bool alone = S >= kScreen99 && cm > before * kScreenAbove && (mask & (mask - 1)) == 0;
         while (mask) {
             const int i = __ffs(mask) - 1;
             mask &= mask - 1;
@@ -243,9 +266,11 @@ __global__ void __launch_bounds__(ROWACT_NT) block_activity_rows_kernel(Geom g, 
 #pragma unroll
             for (int k = 1; k < 2 * U; ++k)
                 if (i == k) c = v[k];
-            D = fmax(D, mode_sq(c));
+            if (alone) pend = c;
+            else D = fmax(D, mode_sq(c));
         }
     }
+    D = fmax(D, mode_sq(pend));
     // combine the G lanes of one block (aligned lane groups), then the row groups
     unsigned long long bm = dbits(fmax(D, Ddc)), bmnd = dbits(D);
     for (int o = G >> 1; o > 0; o >>= 1) {
@@ -271,6 +296,11 @@ __global__ void __launch_bounds__(ROWACT_NT) block_activity_rows_kernel(Geom g, 
     }
 }
 
+__global__ void zero_gmax_kernel(double* gmax) {
+    pdl_wait();
+    if (threadIdx.x < 2) gmax[threadIdx.x] = 0.0;
+}
+
 static bool rows_kernel_fits(const Geom& g) {
     const long long n2 = g.n[2];
     if (n2 % 2 != 0 || n2 / 2 > ROWACT_NT) return false;
@@ -283,14 +313,25 @@ static bool rows_kernel_fits(const Geom& g) {
     return true;
 }
 
+// Serial row trips of the rows kernel: rounds of CTAs over the SMs times trips per CTA.
+template <int NT> static long long rowact_trips(const Geom& g) {
+    const long long slots = 152LL * rowact_ctas<NT>(), ctas = g.nb[0] * g.nb[1];
+    const int per = ROWACT_U * (NT / (int)(g.n[2] / 2));
+    return ((ctas + slots - 1) / slots) * ((g.b[0] * g.b[1] + per - 1) / per);
+}
+
 template <typename T>
 spdba_status launch_block_activity(const Geom& g, const cx_t<T>* q, double* maxsq, double* sumsq, double* gmax,
                                    cudaStream_t st) {
     long long nb = g.blocks();
     if constexpr (sizeof(cx_t<T>) == 8) {
         if (!sumsq && rows_kernel_fits(g)) {
-            pdl_launch(block_activity_rows_kernel, (unsigned)(g.nb[0] * g.nb[1]), ROWACT_NT, 0, st, 
-                g, reinterpret_cast<const float2*>(q), maxsq, gmax);
+            const long long rows = g.nb[0] * g.nb[1];
+            const float2* qf = reinterpret_cast<const float2*>(q);
+            if (g.n[2] / 2 <= 128 && rowact_trips<128>(g) < rowact_trips<256>(g))
+                pdl_launch(block_activity_rows_kernel<128>, (unsigned)rows, 128, 0, st, g, qf, maxsq, gmax);
+            else
+                pdl_launch(block_activity_rows_kernel<256>, (unsigned)rows, 256, 0, st, g, qf, maxsq, gmax);
             SPDBA_CUDA(cudaGetLastError());
             return SPDBA_OK;
         }
@@ -329,7 +370,9 @@ spdba_status launch_tau(const double* gmax, int nruns, double threshold, int tau
 }
 
 // ------------------------------------------------------------------ states
-constexpr int CLS_NT = 1024;
+// 256 blocks per CTA: a 32^3 map then reaches 128 SMs (with 1024 it ran on 32, and
+// on 18 for the stored half of 256^3: 12.7 us).
+constexpr int CLS_NT = 256;
 
 // Block coordinates (32-bit: block maps hold fewer than 2^31 blocks).
 struct BCoord {
@@ -355,7 +398,9 @@ __device__ __forceinline__ int bindex(const Geom& g, const BCoord& c) {
 // the symmetry boundary) or hx - 2 (whose modes are the conjugates of those
 // right of kx = N/2).
 __device__ __forceinline__ void mirror_other_axes(const Geom& g, BCoord& c) {
-    for (int a = 3 - g.ndim; a < 2; ++a) c.c[a] = (int)g.nb[a] - 1 - c.c[a];
+    // constant indices: a loop from 3 - ndim would move the coordinates to local memory
+    if (g.ndim == 3) c.c[0] = (int)g.nb[0] - 1 - c.c[0];
+    if (g.ndim >= 2) c.c[1] = (int)g.nb[1] - 1 - c.c[1];
 }
 __device__ __forceinline__ BCoord bnbr(const Geom& g, BCoord c, int axis, int dir) {
     if (axis == 2 && g.hx > 0) {
@@ -477,6 +522,9 @@ __global__ void __launch_bounds__(CLS_NT) state_kernel(Geom g, const uint8_t* __
     // the activity maxima were consumed by the previous kernel: zero them for the next scan
     if (gmax_reset != nullptr && blockIdx.x == 0)
         for (int r = threadIdx.x; r < 2 * nruns; r += CLS_NT) gmax_reset[r] = 0.0;
+    // and the mass (or power) accumulators for the pass that follows a state setting
+    if (stats && blockIdx.x == 0)
+        for (long long r = threadIdx.x; r < g.runs(); r += CLS_NT) stats[r].mass = 0.0;
     int st = 0;
     uint8_t cb = 0;
     if (b < nb) {
@@ -634,7 +682,7 @@ extern "C" spdba_status spdba_block_activity(int32_t precision, int32_t ndim, co
     spdba_status s = make_geom(&g, ndim, dims, block);
     if (s != SPDBA_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
-    SPDBA_CUDA(cudaMemsetAsync(gmax, 0, 2 * sizeof(double), st));
+    pdl_launch(zero_gmax_kernel, 1, 32, 0, st, gmax);   // a kernel: a memset between two kernels costs both their ticks
     if (precision == SPDBA_C64) return launch_block_activity<float>(g, (const float2*)q, maxsq, sumsq, gmax, st);
     if (precision == SPDBA_C128) return launch_block_activity<double>(g, (const double2*)q, maxsq, sumsq, gmax, st);
     return fail(SPDBA_ERR_ARG, "bad precision %d", precision);
@@ -669,7 +717,7 @@ extern "C" spdba_status spdba_classify(int32_t ndim, const int64_t* nblocks, con
 #include <mutex>
 
 #define SPDBA_STATIC_SCRATCH_BYTES ((size_t)SPDBA_CLASSIFY_STATIC_MAX_BLOCKS + \
-                                    sizeof(int) * (size_t)(SPDBA_CLASSIFY_STATIC_MAX_BLOCKS / 1024))
+                                    sizeof(int) * (size_t)(SPDBA_CLASSIFY_STATIC_MAX_BLOCKS / spdba::CLS_NT))
 
 static __device__ __align__(256) unsigned char g_classify_scratch[SPDBA_STATIC_SCRATCH_BYTES];
 

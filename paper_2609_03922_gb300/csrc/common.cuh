@@ -285,10 +285,12 @@ __device__ __forceinline__ void atomic_max_nonneg(double* addr, double v) {
 }
 
 // |q|^2 in FP64 as re*re + im*im with each product rounded, then the sum rounded
-// (no contraction), the same evaluation the oracle uses.
+// (no contraction), the same evaluation the oracle uses.  Products of FP32 values
+// are exact in FP64, so there the fused form gives the same bits in two
+// instructions of the slow FP64 pipe instead of three.
 __device__ __forceinline__ double mode_sq(float2 q) {
     double re = (double)q.x, im = (double)q.y;
-    return __dadd_rn(__dmul_rn(re, re), __dmul_rn(im, im));
+    return __fma_rn(re, re, __dmul_rn(im, im));
 }
 __device__ __forceinline__ double mode_sq(double2 q) {
     return __dadd_rn(__dmul_rn(q.x, q.x), __dmul_rn(q.y, q.y));

@@ -139,29 +139,34 @@ __global__ void __launch_bounds__(1024) half_col_live_kernel(const uint8_t* __re
 // states: zlive[y * NHP + x] = some block of z pencil (y, x) is not FROZEN
 // (the z forward's outputs are read only by the update of non-frozen blocks);
 // xlive[x] = some z pencil of column x is live (the y forward's outputs in the
-// other columns are read by no live z pencil).  xlive is zero on entry.
+// other columns are read by no live z pencil).  One CTA per block column x / B2:
+// the liveness of its nb1 pencil rows once, then the bytes of its columns.
 __global__ void __launch_bounds__(256) hs_live_kernel(const uint8_t* __restrict__ states, int nb0, int nb1, int nb2,
-                                                      int B1, int B2, int N1, int NHP, uint8_t* __restrict__ zlive,
+                                                      int B1, int B2, int NHP, uint8_t* __restrict__ zlive,
                                                       uint8_t* __restrict__ xlive) {
     pdl_wait();
-    const long long n = (long long)N1 * NHP;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)(i / NHP), x = (int)(i - (long long)y * NHP);
-        const long long b0 = (long long)(y / B1) * nb2 + x / B2;
+    __shared__ uint8_t s_row[1024];   // nb1 <= 512 (the longest axis)
+    const int bx = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int by = warp; by < nb1; by += 8) {
         unsigned live = 0;
-#pragma unroll 8
-        for (int bz = 0; bz < nb0; ++bz) live |= states[(long long)bz * nb1 * nb2 + b0];
-        zlive[i] = live != 0;
-        if (live) xlive[x] = 1;
+        for (int bz = lane; bz < nb0; bz += 32) live |= states[((long long)bz * nb1 + by) * nb2 + bx];
+        const unsigned any = __ballot_sync(0xffffffffu, live != 0);
+        if (lane == 0) s_row[by] = any != 0;
     }
+    __syncthreads();
+    int some = 0;
+    for (int by = threadIdx.x; by < nb1; by += blockDim.x) some |= s_row[by];
+    some = __syncthreads_or(some);
+    for (int k = threadIdx.x; k < nb1 * B1 * B2; k += blockDim.x) {
+        const int y = k / B2, l = k - y * B2;
+        zlive[(long long)y * NHP + bx * B2 + l] = s_row[y / B1];
+    }
+    for (int l = threadIdx.x; l < B2; l += blockDim.x) xlive[bx * B2 + l] = some != 0;
 }
 
 spdba_status launch_hs_live(const Geom& g, const uint8_t* states, uint8_t* zlive, uint8_t* xlive, cudaStream_t st) {
-    const long long n = g.n[1] * g.n[2];
-    SPDBA_CUDA(cudaMemsetAsync(xlive, 0, (size_t)g.n[2], st));
-    const long long grid = std::min<long long>((n + 255) / 256, 152 * 8);
-    pdl_launch(hs_live_kernel, (unsigned)grid, 256, 0, st, states, (int)g.nb[0], (int)g.nb[1], (int)g.nb[2], g.b[1], g.b[2],
-                                                   (int)g.n[1], (int)g.n[2], zlive, xlive);
+    pdl_launch(hs_live_kernel, (unsigned)g.nb[2], 256, 0, st, states, (int)g.nb[0], (int)g.nb[1], (int)g.nb[2],
+               g.b[1], g.b[2], (int)g.n[2], zlive, xlive);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
 }

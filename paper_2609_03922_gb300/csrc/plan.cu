@@ -32,10 +32,6 @@ template <typename T> __global__ void complex_real_part_kernel(const cx_t<T>* __
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         r[i] = c[i].x;
 }
-__global__ void zero_strided_kernel(double* p, long long n, int stride) {
-    pdl_wait();
-    for (long long i = threadIdx.x; i < n; i += blockDim.x) p[i * stride] = 0.0;
-}
 // Statistics of runs [0, n) reset, with the threshold coefficient in force set to eps.
 // and their block states, if given, all ACTIVE (nst of them).
 __global__ void stats_reset_kernel(DevStats* stats, long long n, double eps, uint8_t* states, long long nst) {
@@ -1002,8 +998,6 @@ template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>&
         Pass<T> nl = r.h_nl;
         if (reassess) {
             nl.p.mass = &r.stats[0].mass;
-            pdl_launch(zero_strided_kernel, 1, 256, 0, st, &r.stats[0].mass, r.batch, nl.p.mass_stride);
-            p->launches += 1;
         }
         {
             ProfScope pr(p, K_FUSED_NL, 2.0 * hb);
@@ -1060,8 +1054,6 @@ template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>&
         Pass<T> nl = r.h_nl;
         if (reassess) {
             nl.p.mass = &r.stats[0].mass;
-            pdl_launch(zero_strided_kernel, 1, 256, 0, st, &r.stats[0].mass, r.batch, nl.p.mass_stride);
-            p->launches += 1;
         }
         {
             ProfScope pr(p, K_FUSED_NL, 2.0 * half_b);
@@ -1113,8 +1105,6 @@ template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>&
     Pass<T> fused = r.fused;
     if (reassess) {
         fused.p.mass = &r.stats[0].mass;
-        pdl_launch(zero_strided_kernel, 1, 256, 0, st, &r.stats[0].mass, r.batch, fused.p.mass_stride);
-        p->launches += 1;
     }
     {
         ProfScope pr(p, K_FUSED_NL, pass_bytes);
@@ -1243,14 +1233,12 @@ template <typename T> static spdba_status group_nls_steps(spdba_plan* p, Group<T
             c.tw = r.tw_col;
             c.stats = r.stats;
             if (reassess) {
-                pdl_launch(zero_strided_kernel, 1, 256, 0, st, &r.stats[0].mass, r.batch, a.power_stride);
                 c.power = &r.stats[0].mass;
             }
             if ((s = col_pass<T>(p, r, c, 1, 1, 1)) != SPDBA_OK) return s;
         } else {
             if (reassess && (s = group_assess<T>(p, r)) != SPDBA_OK) return s;
             if (reassess) {
-                pdl_launch(zero_strided_kernel, 1, 256, 0, st, &r.stats[0].mass, r.batch, a.power_stride);
                 a.power = &r.stats[0].mass;
             }
             a.stats = r.stats;
@@ -1455,8 +1443,6 @@ static spdba_status multi_ch_step(spdba_plan* p, const MultiForm& mf) {
         if (control_step(p, r.step) && (s = group_control<float>(p, r)) != SPDBA_OK) return s;
         if (reassess) {
             if ((s = group_assess<float>(p, r)) != SPDBA_OK) return s;
-            pdl_launch(zero_strided_kernel, 1, 256, 0, st, &r.stats[0].mass, r.batch, r.fused.p.mass_stride);
-            p->launches += 1;
             mass_mask |= 1u << i;
         }
         if (!adaptive || all_active_step(p, r.step)) dense_mask |= 1u << i;
