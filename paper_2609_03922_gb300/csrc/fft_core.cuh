@@ -161,6 +161,10 @@ template <typename T> struct PassParams {
     // unmarked columns are never read), or null to transform every tile
     const uint8_t* col_live = nullptr;
     int stream_chat = 0;   // step chain: c_hat is streamed past the L2
+    // two-pencil step chain on a stored half: the last tiles take the one used column
+    // right of the whole tiles of several rows (pair_tile), fd_seg dividing by the whole
+    // tiles of a row
+    int edge = 0;
     // plain passes whose outer index o (strided) or row (rows) runs over fields of
     // seg_n such indices: a tile is skipped when its entries of seg_live are zero
     const uint8_t* seg_live = nullptr;
@@ -886,6 +890,7 @@ struct UpdTile {
     int o, i0, cy, x0, bx0, nbx, l_out;
     long long boff;   // block id offset of (block row 0, x-block bx0)
     int bstride;      // block id step per block row of the pass axis
+    int bxstep;       // block id step per table column (1, or a row of blocks in an edge tile)
     bool rows;
 };
 template <typename T, int P>
@@ -904,6 +909,7 @@ __device__ __forceinline__ UpdTile upd_tile(const PassParams<T>& a, int q0) {
         u.x0 = u.i0;
     }
     u.rows = d3 && u.x0 + P > (int)g.n[2];
+    u.bxstep = 1;
     u.bx0 = (int)f.fd_b2.div((uint32_t)u.x0);
     u.nbx = (int)f.fd_b2.div((uint32_t)(u.x0 + P - 1)) - u.bx0 + 1;
     if (d3) {
@@ -1100,7 +1106,7 @@ __device__ __forceinline__ void ch_update_table(uint8_t* tab, const PassParams<T
     const int npass = (int)(f.g.ndim == 3 ? f.g.nb[0] : f.g.nb[1]);
     for (int k = threadIdx.x; k < npass * u.nbx; k += NT) {
         const int bp = k / u.nbx, bx = k - bp * u.nbx;
-        const long long id = u.boff + (long long)bp * u.bstride + bx;
+        const long long id = u.boff + (long long)bp * u.bstride + bx * u.bxstep;
         tab[k] = f.dense ? (uint8_t)SPDBA_ACTIVE : (uint8_t)(f.states[id] | (f.chi[id] << 2));
     }
 }

@@ -53,11 +53,6 @@ struct GlobalPairIn {
         return pair_of(*reinterpret_cast<const float4*>(base + (2 * p + m * sJ)));
     }
 };
-// The same while the thread's cp.async copies land: complete, and visible to
-// every thread after the stage's barrier.
-struct GlobalPairInWait : GlobalPairIn {
-    __device__ __forceinline__ void before_write() const { cp_async_wait<0>(); }
-};
 // Raw (interleaved) tile in shared memory, pairs of row m at m * H + p.
 template <int H, bool X = false> struct RawPairIn {
     static constexpr bool EXT = X;   // X: the raw tile is not the buffer the transform works in
@@ -158,20 +153,30 @@ template <int L, int H, int Q> struct ChainMid2 {
     const uint8_t* te;
     float2* ce;
     unsigned long long pol;
-    __device__ __forceinline__ ChainMid2(const PassParams<float>& a, const UpdTile& u, const uint8_t* tab_,
-                                         const float* kp_, const float4* cs_, unsigned long long pol_)
+    // edge: pair p is at columns x0 + 2 (p & 1) of row cy + p / 2, else x0 + 2 p of row cy
+    __device__ __forceinline__ ChainMid2(const PassParams<float>& a, const UpdTile& u, bool edge, long long at,
+                                         const uint8_t* tab_, const float* kp_, const float4* cs_,
+                                         unsigned long long pol_)
         : f(a.fu), tab(tab_), kp(kp_), cs(cs_) {
         d3 = f.g.ndim == 3;
         nbx = u.nbx;
-        const int p = 2 * (int)(threadIdx.x % H);
-        const int x = u.x0 + p, bx = (int)f.fd_b2.div((uint32_t)x);
-        tab += bx - u.bx0;
+        const int p = (int)(threadIdx.x % H);
+        const int x = u.x0 + 2 * (edge ? p & 1 : p), bx = (int)f.fd_b2.div((uint32_t)x);
+        int cy = u.cy;
+        l_out = u.l_out;
+        if (edge) {
+            cy += p >> 1;
+            const int by = (int)f.fd_b1.div((uint32_t)cy);
+            l_out = cy - by * f.g.b[1];
+            tab += by - (int)f.fd_b1.div((uint32_t)u.cy);
+        } else {
+            tab += bx - u.bx0;
+        }
         bstep = (int)f.fd_bp.div((uint32_t)Q) * nbx;
         lx = x - bx * f.g.b[2];
         kx = f32x2(f.k2ax[2][x], f.k2ax[2][x + 1]);
-        kc = d3 ? f.k2ax[1][u.cy] : f.k2ax[0][u.cy];
-        l_out = u.l_out;
-        cb = f.c_hat + ((long long)u.o * a.osO + (u.i0 + p));
+        kc = d3 ? f.k2ax[1][cy] : f.k2ax[0][cy];
+        cb = f.c_hat + at;
         osJ = (int)a.osJ;
         ndt = f32x2(-f.dt);
         dtk = f32x2(f.dtkappa);
@@ -209,6 +214,53 @@ template <int L, int H, int Q> struct ChainMid2 {
     }
 };
 
+// A thread's one pencil pair (base: its element 0) in the pass's arrays, read while the
+// thread's cp.async copies land: complete, and visible to every thread after the
+// stage's barrier.
+struct ThreadPairIn {
+    static constexpr bool EXT = true;
+    const float2* base;
+    int sJ;
+    __device__ __forceinline__ void before_write() const { cp_async_wait<0>(); }
+    __device__ __forceinline__ cf32x2 operator()(int, int m) const {
+        return pair_of(*reinterpret_cast<const float4*>(base + m * sJ));
+    }
+};
+template <int L> struct ThreadPairOut {
+    static constexpr bool SYNC = false;
+    float2* base;
+    int sJ;
+    f32x2 scale;
+    __device__ __forceinline__ void pre() {}
+    __device__ __forceinline__ void begin(int, int, int) {}
+    template <int R> __device__ __forceinline__ void emit(int, int, int j, cf32x2 (&v)[R]) {
+        float2* po = base + j * sJ;
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            *reinterpret_cast<float4*>(po + r * (L / R) * sJ) = quad_of(cscale(v[r], scale));
+    }
+};
+
+// Pencil pair p of a tile of the chain: columns q0 + 2 p and the next of one row, or in an
+// edge tile the columns q0 .. q0 + 3 of P / 4 rows, two pairs a row.  A stored half has
+// one used column right of its whole tiles (129 of 144 at 256 points, 33 of 48 at 64);
+// a tile per row would transform and move 15 columns of padding beside it.  Four columns
+// are a sector of 32 bytes: with two, half sectors were written, and 256^3 took 3 us a
+// step more, not less.
+struct PairTile {
+    int q0, row;   // row: 0, or the row width of an edge tile
+    __device__ __forceinline__ int pencil(int p) const {
+        return row == 0 ? q0 + 2 * p : q0 + (p >> 1) * row + 2 * (p & 1);
+    }
+};
+template <int P> __device__ __forceinline__ PairTile pair_tile(const PassParams<float>& a, int t) {
+    if (!a.edge) return PairTile{t * P, 0};
+    const int w = (int)a.fu.g.n[2], per_row = (int)a.fd_seg.d, t0 = (int)a.fu.g.n[1] * per_row;
+    if (t >= t0) return PairTile{(t - t0) * (P / 4) * w + per_row * P, w};
+    const int row = (int)a.fd_seg.div((uint32_t)t);
+    return PairTile{row * w + (t - row * per_row) * P, 0};
+}
+
 template <int L, int P, int NT, int OCC>
 __global__ void __launch_bounds__(NT, OCC) fft_chain2_kernel(PassParams<float> a) {
     pdl_wait();
@@ -222,14 +274,23 @@ __global__ void __launch_bounds__(NT, OCC) fft_chain2_kernel(PassParams<float> a
     __shared__ float s_kp[L];
     __shared__ cf32x2 s_tw[L];
     const CHFuse<float>& f = a.fu;
-    const long long q0 = (long long)blockIdx.x * P;
-    const UpdTile u = upd_tile<float, P>(a, (int)q0);
+    const PairTile pt = pair_tile<P>(a, (int)blockIdx.x);
+    const bool edge = pt.row != 0;
+    UpdTile u = upd_tile<float, P>(a, pt.q0);
+    if (edge) {
+        // one table column per row of blocks that the tile's rows meet
+        u.nbx = (int)f.fd_b1.div((uint32_t)(u.cy + P / 4 - 1)) - (int)f.fd_b1.div((uint32_t)u.cy) + 1;
+        u.bxstep = (int)f.g.nb[2];
+    }
     const unsigned long long pol = chat_policy(a.stream_chat);
-    const float2* cbase = f.c_hat + ((long long)u.o * a.osO + u.i0);
+    const int p = (int)(threadIdx.x % H);
+    const int q = pt.pencil(p), o = (int)a.fd_I.div((uint32_t)q);
+    const long long at = o * a.osO + (q - o * a.I);   // in place: input strides are the output's
     {
-        const int p = (int)(threadIdx.x % H), j0 = (int)(threadIdx.x / H), sJ = (int)a.osJ;
+        const int j0 = (int)(threadIdx.x / H), sJ = (int)a.osJ;
+        const float2* cbase = f.c_hat + at;
 #pragma unroll 8
-        for (int j = j0; j < L; j += NT / H) cp_async16_hint(cs + j * H + p, cbase + (2 * p + j * sJ), pol);
+        for (int j = j0; j < L; j += NT / H) cp_async16_hint(cs + j * H + p, cbase + j * sJ, pol);
         cp_async_commit();
     }
     ch_update_table<float, L, P, NT>(s_tab, a, u);
@@ -245,10 +306,10 @@ __global__ void __launch_bounds__(NT, OCC) fft_chain2_kernel(PassParams<float> a
         for (int k = threadIdx.x; k < nent; k += NT) any |= (s_tab[k] & 3) != SPDBA_FROZEN;
         live = __syncthreads_or(any) != 0;
     }
-    GlobalPairOut<L> out{a.out + ((long long)u.o * a.osO + u.i0), (int)a.osJ, f32x2(1.f)};
+    ThreadPairOut<L> out{a.out + at, (int)a.osJ, f32x2(1.f)};
     if (live) {
-        GlobalPairInWait in{{a.in + ((long long)u.o * a.isO + u.i0), (int)a.isJ}};
-        ChainMid2<L, H, L / Radices_last<f32x2, L>::value> mid(a, u, s_tab, s_kp, cs, pol);
+        ThreadPairIn in{a.in + at, (int)a.isJ};
+        ChainMid2<L, H, L / Radices_last<f32x2, L>::value> mid(a, u, edge, at, s_tab, s_kp, cs, pol);
         transform_pair_in<f32x2, L, H, NT, -1, +1, LY>(sm, s_tw, in, mid, out);
     } else {
         cp_async_wait<0>();

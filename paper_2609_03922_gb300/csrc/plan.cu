@@ -140,7 +140,7 @@ template <typename T> struct Group {
     // step chain: upd_pass and the next step's first inverse pass in one kernel, used
     // between two steps of one call where the fused update is in force
     Pass<T> chain;
-    bool has_chain = false;
+    bool has_chain = false, chain_pairs = false;   // chain_pairs: the two-pencil kernel
     bool pre_done = false;          // `work` holds the first inverse pass of c_hat (set by the chain, within a call)
     FftEngine<T> fft1;              // one run's transforms for set/get_field
     // ... whose passes along the rows take the real field in and give it out (complex64; the
@@ -433,6 +433,7 @@ static spdba_status setup_chain(spdba_plan* p, Group<T>& r, int ndim, const int6
         if (get_chain2_kernel(d[0], c.P < 8, &k2) && r.g.b[2] % 2 == 0 && d[ndim - 1] % k2.P == 0 &&
             chain2_step(d[0]) % bpass == 0) {
             if ((s = set_pass_kernel(&c, k2)) != SPDBA_OK) return s;
+            r.chain_pairs = true;
         }
     }
     if (d[ndim - 1] % c.P != 0 || (d[0] / bpass) * (int64_t)upd_table_cols(c.P, r.g.b[2]) > kUpdTable) return SPDBA_OK;
@@ -586,6 +587,22 @@ static spdba_status group_init_ch_hs(spdba_plan* p, Group<float>& r, const int64
         r.has_fused = true;
         r.fused_update = p->opt.fuse_update != 0;
         if ((s = setup_chain<float>(p, r, 3, dh, 1)) != SPDBA_OK) return s;
+        if (r.has_chain) {
+            // edge tiles: whole tiles up to N2 / 2, then P / 4 rows a tile (its state table has a
+            // column per row of blocks among them).  64^3, 40 steps: 726 -> 702 us (192 tiles become
+            // 144, one round of the SMs); 256^3, 20 steps: 2757 -> 2739 us; 384^3, which lies outside
+            // the L2 and pays for the scattered sectors in HBM accesses: 6320 -> 6372 us, so not there.
+            const int P = r.chain.P, rows = P / 4;
+            int l2 = 0, dev = 0;
+            SPDBA_CUDA(cudaGetDevice(&dev));
+            SPDBA_CUDA(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
+            if ((int64_t)sizeof(float2) * r.hs_n <= l2 && r.chain_pairs && M % P == 0 && N1 % rows == 0 &&
+                (N0 / r.g.b[0]) * (int64_t)upd_table_cols(rows, r.g.b[1]) <= kUpdTable) {
+                r.chain.p.edge = 1;
+                r.chain.p.fd_seg.init((uint32_t)(M / P));
+                r.chain.grid = N1 * (M / P) + N1 / rows;
+            }
+        }
     } else if (s != SPDBA_OK && s != SPDBA_ERR_UNSUPPORTED) {
         return s;
     }
