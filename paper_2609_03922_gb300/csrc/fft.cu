@@ -391,7 +391,6 @@ spdba_status make_half_pass(Pass<float>* out, int mode, const HalfGeo& hg, Twidd
     a.mass_ppr = (long long)hg.N0 * hg.N1;
     a.fd_I.init((uint32_t)a.I);
     a.hg = hg;
-    a.hg.fd_HN.init((uint32_t)(hg.NHP / 2));
     *out = ps;
     return SPDBA_OK;
 }

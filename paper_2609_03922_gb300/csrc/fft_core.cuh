@@ -30,7 +30,6 @@ namespace spdba {
 // Twiddle load: from a CTA's shared copy of the table (the compiler sees the
 // shared address space after inlining) or through the read-only cache.
 template <class C> __device__ __forceinline__ C tw_load(const C* p) { return __isShared(p) ? *p : __ldg(p); }
-__device__ __forceinline__ cf32x2 tw_load(const cf32x2* p) { return *p; }   // always a shared table
 
 // Radix schedule per element type and pencil length (product of radices == L).
 // FP32: few stages, as registers allow.  FP64: radices of at most 8.  An SM takes an
@@ -85,6 +84,26 @@ template <typename T, int L> __host__ __device__ constexpr int ns_at(int i) {
 }
 template <typename T, int L> struct Radices_last { static constexpr int value = LastOf<typename Radices<T, L>::type>::value; };
 
+// Twiddle exp(-SIGN 2 pi i r jm / (NS R)) of a stage.  One pencil per thread: from the
+// table of exp(-2 pi i m / L).  Two pencils: from a shared table that holds one stage
+// after the other, (r - 1) NS + jm within a stage (stage_twiddles).  In the first table
+// a warp's entries lie r L / (NS R) apart and up to eight of them fall on one bank; in
+// the second they are consecutive.
+template <typename T> struct TwOf { using type = cx_t<T>; };
+template <> struct TwOf<f32x2> { using type = float2; };
+template <typename T> using tw_t = typename TwOf<T>::type;
+template <typename T, int L, int NS, int R, int SIGN>
+__device__ __forceinline__ cx_t<T> tw_at(const tw_t<T>* tw, int r, int jm) {
+    if constexpr (std::is_same<T, f32x2>::value) {
+        const float2 w = tw[NS - radix_at<T, L>(0) + (r - 1) * NS + jm];
+        return mk<cf32x2>(f32x2(w.x), f32x2(SIGN > 0 ? -w.y : w.y));
+    } else {
+        cx_t<T> w = tw_load(tw + r * jm * (L / (NS * R)));
+        if constexpr (SIGN > 0) w.y = -w.y;
+        return w;
+    }
+}
+
 // Layout A; ODD selects an odd pencil stride (needed when pencils are read
 // transposed, pencil-fastest), otherwise the stride stays even so that a pair
 // (j, j+1) is one aligned 16-byte shared-memory word.
@@ -132,7 +151,7 @@ struct HalfGeo {
     // as a complex-to-real transform does (their planes need not be
     // conjugate-symmetric within themselves)
     int r2c = 0;
-    FastDiv fd_N2, fd_NHP, fd_M, fd_HN;   // fd_M: division by N2 / 2; fd_HN: by NHP / 2
+    FastDiv fd_N2, fd_NHP, fd_M;   // fd_M: division by N2 / 2
 };
 
 template <typename T> struct PassParams {
@@ -410,7 +429,7 @@ template <typename T, class LY> struct SmemIn {
 };
 
 template <typename T, int L, int P, int NT, int SIGN, int NS, int R, class LY, class IN>
-__device__ __forceinline__ void stockham_stage_in(cx_t<T>* sm, const cx_t<T>* __restrict__ tw, const IN& in) {
+__device__ __forceinline__ void stockham_stage_in(cx_t<T>* sm, const tw_t<T>* __restrict__ tw, const IN& in) {
     using C = cx_t<T>;
     constexpr int Q = L / R;
     constexpr int NB = P * Q;
@@ -429,9 +448,7 @@ __device__ __forceinline__ void stockham_stage_in(cx_t<T>* sm, const cx_t<T>* __
                 int jm = j % NS;
 #pragma unroll
                 for (int r = 1; r < R; ++r) {
-                    C w = tw_load(tw + r * jm * (L / (NS * R)));
-                    if constexpr (SIGN > 0) w.y = -w.y;
-                    v[k][r] = cmul(v[k][r], w);
+                    v[k][r] = cmul(v[k][r], tw_at<T, L, NS, R, SIGN>(tw, r, jm));
                 }
             }
             Dft<R, SIGN, C>::run(v[k]);
@@ -456,22 +473,22 @@ __device__ __forceinline__ void stockham_stage_in(cx_t<T>* sm, const cx_t<T>* __
 }
 
 template <typename T, int L, int P, int NT, int SIGN, int NS, int R, class LY>
-__device__ __forceinline__ void stockham_stage(cx_t<T>* sm, const cx_t<T>* __restrict__ tw) {
+__device__ __forceinline__ void stockham_stage(cx_t<T>* sm, const tw_t<T>* __restrict__ tw) {
     stockham_stage_in<T, L, P, NT, SIGN, NS, R, LY>(sm, tw, SmemIn<T, LY>{sm});
 }
 
 template <typename T, int L, int P, int NT, int SIGN, class LY, int NS, int R, int... Rest>
-__device__ __forceinline__ void run_stages_impl(cx_t<T>* sm, const cx_t<T>* tw) {
+__device__ __forceinline__ void run_stages_impl(cx_t<T>* sm, const tw_t<T>* tw) {
     stockham_stage<T, L, P, NT, SIGN, NS, R, LY>(sm, tw);
     if constexpr (sizeof...(Rest) > 0) run_stages_impl<T, L, P, NT, SIGN, LY, NS * R, Rest...>(sm, tw);
 }
 template <typename T, int L, int P, int NT, int SIGN, class LY, int... Rs>
-__device__ __forceinline__ void run_stages_list(cx_t<T>* sm, const cx_t<T>* tw, RList<Rs...>) {
+__device__ __forceinline__ void run_stages_list(cx_t<T>* sm, const tw_t<T>* tw, RList<Rs...>) {
     run_stages_impl<T, L, P, NT, SIGN, LY, 1, Rs...>(sm, tw);
 }
 // All stages of a length-L transform with kernel exp(SIGN 2 pi i n k / L).
 template <typename T, int L, int P, int NT, int SIGN, class LY>
-__device__ __forceinline__ void run_stages(cx_t<T>* sm, const cx_t<T>* tw) {
+__device__ __forceinline__ void run_stages(cx_t<T>* sm, const tw_t<T>* tw) {
     run_stages_list<T, L, P, NT, SIGN, LY>(sm, tw, typename Radices<T, L>::type{});
 }
 
@@ -482,7 +499,7 @@ __device__ __forceinline__ void run_stages(cx_t<T>* sm, const cx_t<T>* tw) {
 // the butterflies); out.emit(k, p, j, v) receives the R outputs.  An output
 // that writes shared memory sets OUT::SYNC (all reads finish first).
 template <typename T, int L, int P, int NT, int SIGN, int NS, int R, class LY, class OUT>
-__device__ __forceinline__ void stockham_stage_out(cx_t<T>* sm, const cx_t<T>* __restrict__ tw, OUT& out) {
+__device__ __forceinline__ void stockham_stage_out(cx_t<T>* sm, const tw_t<T>* __restrict__ tw, OUT& out) {
     using C = cx_t<T>;
     static_assert(NS * R == L, "direct output is for the last stage");
     constexpr int Q = L / R;
@@ -512,9 +529,7 @@ __device__ __forceinline__ void stockham_stage_out(cx_t<T>* sm, const cx_t<T>* _
             if constexpr (NS > 1) {
 #pragma unroll
                 for (int r = 1; r < R; ++r) {
-                    C w = tw_load(tw + r * j);
-                    if constexpr (SIGN > 0) w.y = -w.y;
-                    v[k][r] = cmul(v[k][r], w);
+                    v[k][r] = cmul(v[k][r], tw_at<T, L, NS, R, SIGN>(tw, r, j));
                 }
             }
             Dft<R, SIGN, C>::run(v[k]);
@@ -534,7 +549,7 @@ __device__ __forceinline__ void stockham_stage_out(cx_t<T>* sm, const cx_t<T>* _
 }
 
 template <typename T, int L, int P, int NT, int SIGN, class LY, class OUT, int NS, int R, int... Rest>
-__device__ __forceinline__ void run_stages_out_impl(cx_t<T>* sm, const cx_t<T>* tw, OUT& out) {
+__device__ __forceinline__ void run_stages_out_impl(cx_t<T>* sm, const tw_t<T>* tw, OUT& out) {
     if constexpr (sizeof...(Rest) == 0) {
         stockham_stage_out<T, L, P, NT, SIGN, NS, R, LY, OUT>(sm, tw, out);
     } else {
@@ -543,12 +558,12 @@ __device__ __forceinline__ void run_stages_out_impl(cx_t<T>* sm, const cx_t<T>* 
     }
 }
 template <typename T, int L, int P, int NT, int SIGN, class LY, class OUT, int... Rs>
-__device__ __forceinline__ void run_stages_out_list(cx_t<T>* sm, const cx_t<T>* tw, OUT& out, RList<Rs...>) {
+__device__ __forceinline__ void run_stages_out_list(cx_t<T>* sm, const tw_t<T>* tw, OUT& out, RList<Rs...>) {
     run_stages_out_impl<T, L, P, NT, SIGN, LY, OUT, 1, Rs...>(sm, tw, out);
 }
 // All stages of a length-L transform, the last one emitting through `out`.
 template <typename T, int L, int P, int NT, int SIGN, class LY, class OUT>
-__device__ __forceinline__ void run_stages_out(cx_t<T>* sm, const cx_t<T>* tw, OUT& out) {
+__device__ __forceinline__ void run_stages_out(cx_t<T>* sm, const tw_t<T>* tw, OUT& out) {
     run_stages_out_list<T, L, P, NT, SIGN, LY, OUT>(sm, tw, out, typename Radices<T, L>::type{});
 }
 
@@ -584,7 +599,7 @@ template <typename T> struct ChNlMid {
 
 // Stages I .. E-1 of a length-L transform (in shared memory).
 template <typename T, int L, int P, int NT, int SIGN, class LY, int I, int E>
-__device__ __forceinline__ void run_stage_range(cx_t<T>* sm, const cx_t<T>* tw) {
+__device__ __forceinline__ void run_stage_range(cx_t<T>* sm, const tw_t<T>* tw) {
     if constexpr (I < E) {
         stockham_stage<T, L, P, NT, SIGN, ns_at<T, L>(I), radix_at<T, L>(I), LY>(sm, tw);
         run_stage_range<T, L, P, NT, SIGN, LY, I + 1, E>(sm, tw);
@@ -646,7 +661,7 @@ template <typename T, int L, int R, class LY> struct FirstStageOut {
 // run in registers.  The
 // second stage's outputs go to `out` (j R + r for a stage that others follow).
 template <typename T, int L, int P, int NT, int SA, int SB, int NS, int R, class LY, class MID, class OUT>
-__device__ __forceinline__ void fused_mid_stage(cx_t<T>* sm, const cx_t<T>* __restrict__ tw, MID& mid, OUT& out) {
+__device__ __forceinline__ void fused_mid_stage(cx_t<T>* sm, const tw_t<T>* __restrict__ tw, MID& mid, OUT& out) {
     using C = cx_t<T>;
     static_assert(NS * R == L, "the first of the two stages closes its transform");
     constexpr int Q = L / R;
@@ -666,9 +681,7 @@ __device__ __forceinline__ void fused_mid_stage(cx_t<T>* sm, const cx_t<T>* __re
             if constexpr (NS > 1) {
 #pragma unroll
                 for (int r = 1; r < R; ++r) {
-                    C w = tw_load(tw + r * j);
-                    if constexpr (SA > 0) w.y = -w.y;
-                    v[k][r] = cmul(v[k][r], w);
+                    v[k][r] = cmul(v[k][r], tw_at<T, L, NS, R, SA>(tw, r, j));
                 }
             }
             mid.begin(p, j);
@@ -698,7 +711,7 @@ __device__ __forceinline__ void fused_mid_stage(cx_t<T>* sm, const cx_t<T>* __re
 // One transform whose first stage reads through `in` and whose last stage
 // emits through `out` (at least two stages).
 template <typename T, int L, int P, int NT, int SIGN, class LY, class IN, class OUT>
-__device__ __forceinline__ void run_stages_in_out(cx_t<T>* sm, const cx_t<T>* tw, const IN& in, OUT& out) {
+__device__ __forceinline__ void run_stages_in_out(cx_t<T>* sm, const tw_t<T>* tw, const IN& in, OUT& out) {
     constexpr int NST = NSTAGES<T, L>::value;
     static_assert(NST >= 2, "a separate first and last stage");
     stockham_stage_in<T, L, P, NT, SIGN, 1, radix_at<T, L>(0), LY>(sm, tw, in);
@@ -707,13 +720,13 @@ __device__ __forceinline__ void run_stages_in_out(cx_t<T>* sm, const cx_t<T>* tw
 }
 
 template <typename T, int L, int P, int NT, int SA, int SB, class LY, class MID, class OUT>
-__device__ __forceinline__ void transform_pair(cx_t<T>* sm, const cx_t<T>* tw, MID& mid, OUT& out);
+__device__ __forceinline__ void transform_pair(cx_t<T>* sm, const tw_t<T>* tw, MID& mid, OUT& out);
 
 // transform_pair whose first stage reads its inputs through `in` (an
 // elementwise preparation folded into the first stage's loads); at least
 // three stages in all.
 template <typename T, int L, int P, int NT, int SA, int SB, class LY, class IN, class MID, class OUT>
-__device__ __forceinline__ void transform_pair_in(cx_t<T>* sm, const cx_t<T>* tw, const IN& in, MID& mid, OUT& out) {
+__device__ __forceinline__ void transform_pair_in(cx_t<T>* sm, const tw_t<T>* tw, const IN& in, MID& mid, OUT& out) {
     constexpr int NST = NSTAGES<T, L>::value;
     constexpr int R0 = radix_at<T, L>(0), RL = radix_at<T, L>(NST - 1);
     static_assert(NST >= 2, "the first stage must not be the meeting stage");
@@ -735,7 +748,7 @@ __device__ __forceinline__ void transform_pair_in(cx_t<T>* sm, const cx_t<T>* tw
 }
 
 template <typename T, int L, int P, int NT, int SA, int SB, class LY, class MID, class OUT>
-__device__ __forceinline__ void transform_pair(cx_t<T>* sm, const cx_t<T>* tw, MID& mid, OUT& out) {
+__device__ __forceinline__ void transform_pair(cx_t<T>* sm, const tw_t<T>* tw, MID& mid, OUT& out) {
     constexpr int NST = NSTAGES<T, L>::value;
     constexpr int R0 = radix_at<T, L>(0), RL = radix_at<T, L>(NST - 1);
     if constexpr (R0 == RL) {

@@ -17,13 +17,21 @@ namespace spdba {
 __device__ __forceinline__ cf32x2 pair_of(float4 q) { return mk<cf32x2>(f32x2(q.x, q.z), f32x2(q.y, q.w)); }
 __device__ __forceinline__ float4 quad_of(cf32x2 c) { return make_float4(c.x.lo(), c.y.lo(), c.x.hi(), c.y.hi()); }
 
-// The length-L twiddle table with each factor duplicated for the two pencils.
-template <int L, int NT> __device__ __forceinline__ void dup_twiddles(cf32x2* s_tw, const float2* __restrict__ tw) {
+// The shared twiddle table of tw_at, stage after stage (L minus the first radix entries).
+// A table in index order with each factor stored twice (16 bytes) made half of the row
+// kernels' shared wavefronts: strides of the last stages put up to eight lanes on one
+// bank.  As it is now, with fields in and out: 256^3 half 2739 -> 2646 us (20 steps),
+// 384^3 6372 -> 6100 us (10), the 64-run ensemble 6258 -> 5865 us, 64 NLS signals 4709 ->
+// 4181 us, 32 transforms of 2^18 forward and back 140 -> 130 us.
+template <int L, int NT, int I = 1> __device__ __forceinline__ void stage_twiddles(float2* s_tw, const float2* __restrict__ tw) {
+    constexpr int NS = ns_at<f32x2, L>(I), R = radix_at<f32x2, L>(I);
+    float2* dst = s_tw + (NS - radix_at<f32x2, L>(0));
 #pragma unroll
-    for (int j = threadIdx.x; j < L; j += NT) {
-        const float2 w = __ldg(tw + j);
-        s_tw[j] = mk<cf32x2>(f32x2(w.x), f32x2(w.y));
+    for (int e = threadIdx.x; e < (R - 1) * NS; e += NT) {
+        const int r = e / NS + 1, jm = e % NS;
+        dst[e] = __ldg(tw + r * jm * (L / (NS * R)));
     }
+    if constexpr (I + 1 < NSTAGES<f32x2, L>::value) stage_twiddles<L, NT, I + 1>(s_tw, tw);
 }
 
 // L2 priority of c_hat's lines in the chain.  stream: they are dropped first, so
@@ -88,8 +96,8 @@ __global__ void __launch_bounds__(NT, OCC) fft_pipe2_kernel(PassParams<float> a)
     using LY = LayoutB<L, H>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cf32x2* const b0 = reinterpret_cast<cf32x2*>(smem_raw);
-    __shared__ cf32x2 s_tw[L];
-    dup_twiddles<L, NT>(s_tw, a.tw);   // visible after the loop's first barrier
+    __shared__ float2 s_tw[L];
+    stage_twiddles<L, NT>(s_tw, a.tw);   // visible after the loop's first barrier
     const int ntiles = (int)((a.O * a.I) / P), G = (int)gridDim.x, sJ = (int)a.isJ;
     const int p = (int)(threadIdx.x % H), j0 = (int)(threadIdx.x / H);
     static_assert(NT % H == 0, "each thread copies one pencil pair");
@@ -272,7 +280,7 @@ __global__ void __launch_bounds__(NT, OCC) fft_chain2_kernel(PassParams<float> a
     float4* const cs = reinterpret_cast<float4*>(sm + LY::SIZE);
     __shared__ uint8_t s_tab[kUpdTable];
     __shared__ float s_kp[L];
-    __shared__ cf32x2 s_tw[L];
+    __shared__ float2 s_tw[L];
     const CHFuse<float>& f = a.fu;
     const PairTile pt = pair_tile<P>(a, (int)blockIdx.x);
     const bool edge = pt.row != 0;
@@ -296,7 +304,7 @@ __global__ void __launch_bounds__(NT, OCC) fft_chain2_kernel(PassParams<float> a
     ch_update_table<float, L, P, NT>(s_tab, a, u);
     const float* kpg = f.g.ndim == 3 ? f.k2ax[0] : f.k2ax[1];
     for (int j = threadIdx.x; j < L; j += NT) s_kp[j] = kpg[j];
-    dup_twiddles<L, NT>(s_tw, a.tw);
+    stage_twiddles<L, NT>(s_tw, a.tw);
     ch_update_stats<float, NT>(f, f.dense);
     bool live = true;
     if (!f.dense) {
@@ -392,7 +400,7 @@ __global__ void __launch_bounds__(NT, OCC) fft_rows2_kernel(PassParams<float> a)
     using LY = RowLayout<L, H>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cf32x2* const sm = reinterpret_cast<cf32x2*>(smem_raw);
-    __shared__ cf32x2 s_tw[L];
+    __shared__ float2 s_tw[L];
     const long long q0 = (long long)blockIdx.x * P;
     const long long o = a.fd_I.div((uint32_t)q0), i0 = q0 - o * a.I;
     if (MODE == PASS_PLAIN && a.seg_live != nullptr) {
@@ -403,7 +411,7 @@ __global__ void __launch_bounds__(NT, OCC) fft_rows2_kernel(PassParams<float> a)
         for (int p = 0; p < P; ++p) live |= a.seg_live[r0 + p] != 0;
         if (!live) return;
     }
-    dup_twiddles<L, NT>(s_tw, a.tw);
+    stage_twiddles<L, NT>(s_tw, a.tw);
     RowPairIn in{a.in + (o * a.isO + i0 * a.isI), (int)a.isI};
     RowPairOut<L> out{a.out + (o * a.osO + i0 * a.osI), (int)a.osI, f32x2(a.scale)};
     if constexpr (MODE == PASS_CH_NL) {
@@ -450,10 +458,10 @@ __global__ void __launch_bounds__(NT, OCC) fft_rows_transpose2_kernel(PassParams
     using LY = LayoutA<L, H, true>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cf32x2* const sm = reinterpret_cast<cf32x2*>(smem_raw);
-    __shared__ cf32x2 s_tw[L];
+    __shared__ float2 s_tw[L];
     const long long q0 = (long long)blockIdx.x * P;
     const long long o = a.fd_I.div((uint32_t)q0), i0 = q0 - o * a.I;
-    dup_twiddles<L, NT>(s_tw, a.tw);
+    stage_twiddles<L, NT>(s_tw, a.tw);
     RowPairIn in{a.in + (o * a.isO + i0 * a.isI), (int)a.isI};
     SmemOut2<L, LY> so{sm};
     run_stages_in_out<f32x2, L, H, NT, SIGN, LY>(sm, s_tw, in, so);
@@ -541,10 +549,10 @@ __global__ void __launch_bounds__(NT, OCC) fft_nl_half2_kernel(PassParams<float>
     using LY = RowLayout<L, H>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cf32x2* const sm = reinterpret_cast<cf32x2*>(smem_raw);
-    __shared__ cf32x2 s_tw[L];
+    __shared__ float2 s_tw[L];
     const int NHP = a.hg.NHP;
     const long long q0 = (long long)blockIdx.x * P;
-    dup_twiddles<L, NT>(s_tw, a.tw);
+    stage_twiddles<L, NT>(s_tw, a.tw);
     const float2* src = a.in + q0 * NHP;
     float2* rows = reinterpret_cast<float2*>(smem_raw);
     if constexpr (ST && MODE != PASS_R2C_HALF) {
@@ -569,32 +577,26 @@ __global__ void __launch_bounds__(NT, OCC) fft_nl_half2_kernel(PassParams<float>
     }
     __syncthreads();
     // the two rows' half spectra of each transform: G1[k] = (W[k] + conj W[-k]) / 2,
-    // G2[k] = (W[k] - conj W[-k]) / (2i), two entries of four rows an item (padding
-    // entries zero)
+    // G2[k] = (W[k] - conj W[-k]) / (2i), an entry of four rows an item (padding
+    // entries zero).  Two neighbouring entries an item (16-byte stores) would read the
+    // tile at every other element, two wavefronts for one.
     float2* dst = a.out + q0 * NHP;
-    const int HN = NHP / 2;
     const f32x2 half(0.5f), nhalf(-0.5f);
-    auto split = [&](int p, int k, float2 (&g)[4]) {
+    for (int it = threadIdx.x; it < H * NHP; it += NT) {
+        const int p = (int)a.hg.fd_NHP.div((uint32_t)it), k = it - p * NHP;
+        float2* d = dst + (4 * p * NHP + k);
         if (k > M) {
-            g[0] = g[1] = g[2] = g[3] = make_float2(0.f, 0.f);
-            return;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) d[i * NHP] = make_float2(0.f, 0.f);
+            continue;
         }
         const cf32x2 w = sm[LY::idx(p, k)], v = sm[LY::idx(p, k == 0 ? 0 : L - k)];
         const f32x2 g1x = mul_rn(half, w.x + v.x), g1y = mul_rn(half, w.y - v.y);
         const f32x2 g2x = mul_rn(half, w.y + v.y), g2y = mul_rn(nhalf, w.x - v.x);
-        g[0] = make_float2(g1x.lo(), g1y.lo());
-        g[1] = make_float2(g2x.lo(), g2y.lo());
-        g[2] = make_float2(g1x.hi(), g1y.hi());
-        g[3] = make_float2(g2x.hi(), g2y.hi());
-    };
-    for (int it = threadIdx.x; it < H * HN; it += NT) {
-        const int p = (int)a.hg.fd_HN.div((uint32_t)it), k = 2 * (it - p * HN);
-        float2 g0[4], g1[4];
-        split(p, k, g0);
-        split(p, k + 1, g1);
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            *reinterpret_cast<float4*>(dst + (4 * p + i) * NHP + k) = make_float4(g0[i].x, g0[i].y, g1[i].x, g1[i].y);
+        d[0] = make_float2(g1x.lo(), g1y.lo());
+        d[NHP] = make_float2(g2x.lo(), g2y.lo());
+        d[2 * NHP] = make_float2(g1x.hi(), g1y.hi());
+        d[3 * NHP] = make_float2(g2x.hi(), g2y.hi());
     }
     if (a.mass != nullptr) {
         const double ms = warp_sum((double)mid.msum.lo() + (double)mid.msum.hi());

@@ -114,12 +114,12 @@ __global__ void __launch_bounds__(NT, OCC) nls_row2_kernel(NLSArgs<float> a, Fas
     using LY = RowLayout<L, H>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cf32x2* const sm = reinterpret_cast<cf32x2*>(smem_raw);
-    __shared__ cf32x2 s_tw[L];
+    __shared__ float2 s_tw[L];
     __shared__ uint8_t s_sc[512];
     const uint32_t q0 = blockIdx.x * (uint32_t)P;
     const uint32_t sig = fd_n1.div(q0);   // a tile lies within one signal (P divides n1)
     const int k1p = (int)(q0 - sig * (uint32_t)a.n1);
-    dup_twiddles<L, NT>(s_tw, a.tw);
+    stage_twiddles<L, NT>(s_tw, a.tw);
     const bool halves = a.do_close || a.do_open;
     if (halves) {
         for (int b = threadIdx.x; b < a.nblk; b += NT) {
@@ -190,12 +190,12 @@ __global__ void __launch_bounds__(NT, OCC) nls_col2_kernel(NLSArgs<float> a) {
     using LY = LayoutB<L, H>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cf32x2* const sm = reinterpret_cast<cf32x2*>(smem_raw);
-    __shared__ cf32x2 s_tw[L];
+    __shared__ float2 s_tw[L];
     constexpr int TPS = 512 / P;   // tiles per signal
     const long long sig = blockIdx.x / TPS;
     const int n20 = (int)(blockIdx.x % TPS) * P;
     if constexpr (INV && FWD) nls_step_stats<float>(a);
-    dup_twiddles<L, NT>(s_tw, a.tw);
+    stage_twiddles<L, NT>(s_tw, a.tw);
     GlobalPairIn in{a.in + (sig * a.n + n20), 512};
     float2* dst = a.S + (sig * a.n + n20);
     if constexpr (INV && FWD) {

@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(NT, OCC)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* const rows = reinterpret_cast<float2*>(smem_raw);           // 4 H rows
     cf32x2* const sm = reinterpret_cast<cf32x2*>(rows + 4 * H * L);
-    __shared__ cf32x2 s_tw[L];
+    __shared__ float2 s_tw[L];
     __shared__ RowPair s_pr[H];
     const int c = (int)fd_tiles.div(blockIdx.x), q0 = ((int)blockIdx.x - c * tiles) * H;
     const long long n = (long long)N0 * N1 * L;
@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(NT, OCC)
     const bool pair = 2 * c + 1 < M;   // an odd last component stands alone
     if (threadIdx.x < H)
         s_pr[threadIdx.x] = q0 + (int)threadIdx.x < npairs ? rcd_row_pair(q0 + threadIdx.x, N0, N1) : RowPair{-1, -1};
-    dup_twiddles<L, NT>(s_tw, tw);
+    stage_twiddles<L, NT>(s_tw, tw);
     __syncthreads();
     constexpr int U = L / 2;   // 16-byte units per row
     for (int w = threadIdx.x; w < 4 * H * U; w += NT) {
