@@ -152,11 +152,11 @@ def check(status):
 
 
 def _i64(vals):
-    return (ctypes.c_int64 * len(vals))(*[int(v) for v in vals])
+    return (ctypes.c_int64 * len(vals))(*map(int, vals))
 
 
 def _i32(vals):
-    return (ctypes.c_int32 * len(vals))(*[int(v) for v in vals])
+    return (ctypes.c_int32 * len(vals))(*map(int, vals))
 
 
 def _ptr(x):
@@ -174,8 +174,10 @@ def _ptr(x):
 
 
 def current_stream():
+    """Handle of torch's current stream (without the Stream object around it, which costs
+    as much as a kernel launch)."""
     import torch
-    return torch.cuda.current_stream().cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def options_default(**kw):
