@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(256) hs_live_kernel(const uint8_t* __restrict_
                                                       int B1, int B2, int NHP, uint8_t* __restrict__ zlive,
                                                       uint8_t* __restrict__ xlive) {
     pdl_wait();
-    __shared__ uint8_t s_row[1024];   // nb1 <= 512 (the longest axis)
+    extern __shared__ uint8_t s_row[];   // nb1 entries
     const int bx = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int by = warp; by < nb1; by += 8) {
         unsigned live = 0;
@@ -165,7 +165,9 @@ __global__ void __launch_bounds__(256) hs_live_kernel(const uint8_t* __restrict_
 }
 
 spdba_status launch_hs_live(const Geom& g, const uint8_t* states, uint8_t* zlive, uint8_t* xlive, cudaStream_t st) {
-    pdl_launch(hs_live_kernel, (unsigned)g.nb[2], 256, 0, st, states, (int)g.nb[0], (int)g.nb[1], (int)g.nb[2],
+    // y has at most 4096 points (the longest pass), so that a byte per block row always fits
+    if (g.nb[1] > 4096) return fail(SPDBA_ERR_UNSUPPORTED, "half-spectrum storage over 4096 block rows");
+    pdl_launch(hs_live_kernel, (unsigned)g.nb[2], 256, (size_t)g.nb[1], st, states, (int)g.nb[0], (int)g.nb[1], (int)g.nb[2],
                g.b[1], g.b[2], (int)g.n[2], zlive, xlive);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;

@@ -52,3 +52,19 @@ def test_one_call_equals_single_steps(dims, block, mode):
     assert np.array_equal(a[1], b[1])
     assert a[2] == b[2]
     assert np.array_equal(a[3], b[3])
+
+
+def test_many_block_rows():
+    """2048 rows of blocks along y: the pencil liveness that prunes the forward passes. Fused steps use
+    the x columns' part of it, staged ones also the z pencils'."""
+    from paper_2609_03922_gb300 import spdba
+    dims, block = (16, 2048, 64), (4, 1, 8)
+    x = _field(dims)
+    outs = []
+    for fuse in (1, 0):
+        with spdba.Plan(dims, block, half_storage=1, threshold=0.6, reassess=5, mode=1, dt=0.02, fuse_update=fuse) as p:
+            p.set_field(x)
+            p.step(8)
+            outs.append((p.get_spectrum(), p.get_mask()))
+    assert np.array_equal(outs[0][0].view(np.float32), outs[1][0].view(np.float32))
+    assert np.array_equal(outs[0][1], outs[1][1])
