@@ -7,6 +7,8 @@
 // conj W(-k)) / (2 i), which the update does as it reads W.  Every pass between the
 // two moves half the data, the reaction too.  The inverse starts with the rows, where
 // Z is formed (this file); rows r and -r are needed together, and share a thread.
+#include <algorithm>
+
 #include "fft_f32x2.cuh"
 #include "rcd.h"
 
@@ -38,9 +40,10 @@ __device__ __forceinline__ RowPair rcd_row_pair(int q, int N0, int N1) {
 }
 
 // Packed element m of row pair p: Z at (row d, m) and (row m, m) from the staged
-// rows a_d, b_d, a_m, b_m.
+// rows a_d, b_d, a_m, b_m (the transform works over them once its inputs are in
+// registers).
 template <int L> struct RcdPackIn {
-    static constexpr bool EXT = true;
+    static constexpr bool EXT = false;
     const float2* rows;   // pair p: four rows of L
     __device__ __forceinline__ void before_write() const {}
     __device__ __forceinline__ cf32x2 operator()(int p, int m) const {
@@ -85,7 +88,7 @@ __global__ void __launch_bounds__(NT, OCC)
     using LY = RowLayout<L, H>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* const rows = reinterpret_cast<float2*>(smem_raw);           // 4 H rows
-    cf32x2* const sm = reinterpret_cast<cf32x2*>(rows + 4 * H * L);
+    cf32x2* const sm = reinterpret_cast<cf32x2*>(smem_raw);
     __shared__ float2 s_tw[L];
     __shared__ RowPair s_pr[H];
     const int c = (int)fd_tiles.div(blockIdx.x), q0 = ((int)blockIdx.x - c * tiles) * H;
@@ -182,7 +185,7 @@ namespace {
 template <int L, int H, int NT, int OCC> void pack_info(RcdPack* o) {
     o->H = H;
     o->nt = NT;
-    o->smem = (4 * H * L * (int)sizeof(float2)) + RowLayout<L, H>::SIZE * (int)sizeof(cf32x2);
+    o->smem = std::max(4 * H * L * (int)sizeof(float2), RowLayout<L, H>::SIZE * (int)sizeof(cf32x2));
     o->func = (const void*)rcd_pack_rows_kernel<L, H, NT, OCC>;
 }
 }  // namespace
@@ -200,8 +203,8 @@ spdba_status rcd_pack_prepare(RcdPack* o, int ndim, const int64_t* d, int M, Twi
         case 256: pack_info<256, 4, 64, 6>(o); break;
         default: return SPDBA_OK;
     }
-    if (o->smem > 48 * 1024)
-        SPDBA_CUDA(cudaFuncSetAttribute(o->func, cudaFuncAttributeMaxDynamicSharedMemorySize, o->smem));
+    // at most 34 KB; the whole carveout, so that as many CTAs fit as the registers allow
+    SPDBA_CUDA(cudaFuncSetAttribute(o->func, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     const int smem = 2 * ((M + 1) / 2) * RCD_PRX_NT * (int)sizeof(float);
     if (smem > 48 * 1024)
         SPDBA_CUDA(cudaFuncSetAttribute((const void*)rcd_reaction_packed_kernel,
