@@ -67,35 +67,35 @@ def prof_every(k):
 
 
 # DRAM bytes (read + write) per launch from ncu captures of the current kernels
-# on the 256^3 field with half-spectrum storage, one launch each at step 505 of
-# the staged run (cold L2 at the start of each launch;
+# on the 256^3 field with half-spectrum storage (averages over the first steps after
+# time 5, cold L2 at the start of each launch;
 # profiles/ch3d256_half_storage_step_kernels.md):
 TOUCHED_BYTES = {
-    # x pass (two real rows per transform, one output loop over all row pairs): 75.53 MB read,
-    # 14.55 MB written
-    "fft_fused_nl": 75.53e6 + 14.55e6,
-    # z inverse 75.56 + 20.36 MB and y inverse 75.55 + 11.44 MB on the stored half, averaged
-    "fft_pass": (75.56e6 + 20.36e6 + 75.55e6 + 11.44e6) / 2,
-    # y forward pruned to the live x columns: 58.78 MB read, 2.29 MB written
-    "fft_y_forward_pruned": 58.78e6 + 2.29e6,
-    # z forward pruned to the live z pencils: 38.63 MB read, 0.12 MB written (its output stays in L2
-    # for the list update)
+    # x pass (two real rows per transform, two transforms per thread)
+    "fft_fused_nl": 75.54e6 + 12.42e6,
+    # z inverse and y inverse on the stored half, averaged
+    "fft_pass": 75.53e6 + 12.45e6,
+    # y forward pruned to the live x columns
+    "fft_y_forward_pruned": 61.33e6 + 4.32e6,
+    # z forward + update + the next step's z inverse
+    "fft_update_inverse": 115.49e6 + 33.99e6,
+    # z forward pruned to the live z pencils (its output stays in L2 for the list update)
     "fft_z_forward": 38.63e6 + 0.12e6,
-    # list-driven update of the half map's non-frozen blocks: 41.67 MB read, 0.02 MB written
+    # list-driven update of the half map's non-frozen blocks
     "update_list": 41.67e6 + 0.02e6,
-    # activity scan of the stored half (rows kernel, per-lane screen): 75.52 MB read, 0.56 MB written
-    "assess": 75.52e6 + 0.56e6,
+    # activity scan of the stored half (rows kernel, per-lane screen)
+    "assess": 75.52e6 + 0.02e6,
 }
+_LAUNCH = "ncu DRAM read + write per launch (cold L2)"
 TOUCHED_NOTE = {
-    "fft_fused_nl": "ncu DRAM read + write of one launch at step 505 (cold L2)",
-    "fft_pass": "ncu DRAM read + write per launch at step 505, averaged over the z inverse and the y inverse "
-                "(cold L2)",
-    "fft_y_forward_pruned": "ncu DRAM read + write of one launch at step 505 (cold L2)",
-    "fft_z_forward": "ncu DRAM read + write of one launch at step 505 (cold L2)",
-    "update_list": "ncu DRAM read + write of one launch at step 505 (cold L2; most writes leave the launch "
-                   "in L2)",
-    "assess": "ncu DRAM read + write of one scan at step 510 (the scan launch only; the classification's three "
-              "small launches and the pencil-liveness launch are in the same kind)",
+    "fft_fused_nl": _LAUNCH,
+    "fft_pass": _LAUNCH + ", averaged over the z inverse and the y inverse",
+    "fft_y_forward_pruned": _LAUNCH,
+    "fft_update_inverse": _LAUNCH,
+    "fft_z_forward": _LAUNCH,
+    "update_list": _LAUNCH + "; most writes leave the launch in L2",
+    "assess": _LAUNCH + " of the scan only; the classification's three small launches and the "
+              "pencil-liveness launch are in the same kind",
 }
 CONTROL_TARGETS = (0.05, 0.1, 0.2)   # dynamic threshold control targets (S1.3: 5-20 %)
 CONTROL_EVERY = 50                   # control interval (S3.2, S4.2, S5.3)
@@ -270,7 +270,7 @@ def run_ours(args, rank, world, local_rank, parity=None):
         return spdba.Plan(DIMS, BLOCK, threshold=THRESHOLD, reassess=REASSESS, precision=spdba.SPDBA_C64,
                           mode=mode, dt=DT, kappa=KAPPA, fuse_update=fuse, half_storage=hs, **kw)
 
-    def prepare(plan):
+    def prepare(plan, tune_it=True):
         """From c0 to step TUNE_AT (blocks have frozen there), where the plan's
         autotuner picks its launch configuration; then the run again from c0,
         keeping c_hat at the window starts: steps 0, FULL_RUN/NSNAP, ...
@@ -279,7 +279,7 @@ def run_ours(args, rank, world, local_rank, parity=None):
         itself).  Returns the tuner's report and the states (device)."""
         plan.set_field(c0_dev)
         plan.step(TUNE_AT)
-        tune = plan.autotune(2 * REASSESS)
+        tune = plan.autotune(2 * REASSESS) if tune_it else {}
         tune["at_step"] = TUNE_AT
         starts = snapshot_steps(K)
         plan.set_field(c0_dev)
@@ -462,7 +462,7 @@ def run_ours(args, rank, world, local_rank, parity=None):
     staged = {}
     for name, mode in (("adaptive", spdba.SPDBA_MODE_ADAPTIVE), ("dense", spdba.SPDBA_MODE_REGULAR)):
         pl = make(mode, 0)
-        _, snap = prepare(pl)
+        _, snap = prepare(pl, tune_it=False)   # the tuner may choose the fused update
         ms, _, _, _ = window(pl, snap)
         _, _, _, pr = window(pl, snap, profile=True, reps=prof_reps)
         nsteps = max(1, pr[0]["fft_fused_nl"]["launches"])
@@ -540,6 +540,11 @@ def run_ours(args, rank, world, local_rank, parity=None):
                 # reads the y forward's output, reads and writes c_hat of the non-frozen blocks
                 alg = 8.0 * n_half + 16.0 * n_half * ratio
                 dense_b = 24.0 * n_half
+            elif k == "fft_update_inverse":
+                # reads the y forward's output and c_hat, writes c_hat of the non-frozen blocks and
+                # the next step's z inverse
+                alg = 24.0 * n_half + 8.0 * n_half * ratio
+                dense_b = 32.0 * n_half
             elif k == "update_list":
                 dense_b = 24.0 * n_half
             elif k in ("fft_y_forward_pruned", "fft_z_forward"):
@@ -575,6 +580,8 @@ def run_ours(args, rank, world, local_rank, parity=None):
                 "avg_us": v["avg_us"]}
 
     labels = {"fft_update": "z forward FFT pass on the stored half + fused CH update (L=256, c64)",
+              "fft_update_inverse": "z forward FFT + CH update + the next step's z inverse on the stored half "
+                                    "(L=256, c64)",
               "fft_z_forward": "z forward FFT pass on the stored half, pruned to live pencils (L=256, c64)",
               "update_list": "list-driven CH update of the half map's non-frozen blocks (c64)",
               "fft_fused_nl": "x pass: two real rows per transform, c^3 - c (L=256, c64)",
@@ -582,11 +589,14 @@ def run_ours(args, rank, world, local_rank, parity=None):
               "assess": "activity scan of the stored half + classification on the half map (every R steps)"}
     roofs = {k: roof(k, kinds, lab) for k, lab in labels.items()}
     # the dominant kernel: the longest average launch among the step's kernels that run once per step
-    cands = [(kinds[k]["avg_us"], roofs[k]) for k in ("fft_update", "fft_z_forward", "update_list", "fft_fused_nl")
-             if k in kinds and roofs.get(k)]
+    cands = [(kinds[k]["avg_us"], roofs[k]) for k in ("fft_update", "fft_update_inverse", "fft_z_forward",
+                                                           "update_list", "fft_fused_nl")
+             if k in kinds and roofs.get(k) and
+             2 * kinds[k]["launches"] > kinds.get("fft_fused_nl", {"launches": 1})["launches"]]
     dominant = max(cands, key=lambda c: c[0])[1] if cands else roofs.get("fft_pass")
     transforms_us = sum(kinds[k]["avg_us"] * kinds[k]["launches"] for k in ("fft_pass", "fft_fused_nl",
                                                                              "fft_z_forward", "fft_update",
+                                                                             "fft_update_inverse",
                                                                              "fft_y_forward_pruned")
                         if k in kinds) / max(1, kinds.get("fft_fused_nl", {"launches": 1})["launches"])
     sa, sd = staged["adaptive"]["update_stage_ms_per_step"], staged["dense"]["update_stage_ms_per_step"]
