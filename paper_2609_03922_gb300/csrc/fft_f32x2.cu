@@ -34,6 +34,7 @@ template <int L, int P, int NT, int OCC> static bool rows(int sign, int mode, Ke
 bool get_pass2_kernel(int64_t L, int sign, int mode, bool strided_axis, bool narrow, KernelInfo* ki) {
     if (strided_axis) {
         if (mode != PASS_PLAIN || narrow) return false;
+        if (L == 128) return strided<128, 16, 64, 6>(sign, ki);
         if (L == 256) return strided<256, 16, 128, 3>(sign, ki);
         if (L == 384) return strided<384, 16, 192, 2>(sign, ki);
         return false;

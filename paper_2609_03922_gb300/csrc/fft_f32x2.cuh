@@ -23,7 +23,8 @@ __device__ __forceinline__ float4 quad_of(cf32x2 c) { return make_float4(c.x.lo(
 // bank.  As it is now, with fields in and out: 256^3 half 2739 -> 2646 us (20 steps),
 // 384^3 6372 -> 6100 us (10), the 64-run ensemble 6258 -> 5865 us, 64 NLS signals 4709 ->
 // 4181 us, 32 transforms of 2^18 forward and back 140 -> 130 us.
-template <int L, int NT, int I = 1> __device__ __forceinline__ void stage_twiddles(float2* s_tw, const float2* __restrict__ tw) {
+template <int L, int NT, int I = 1>
+__device__ __forceinline__ void stage_twiddles(float2* s_tw, const float2* __restrict__ tw) {
     constexpr int NS = ns_at<f32x2, L>(I), R = radix_at<f32x2, L>(I);
     float2* dst = s_tw + (NS - radix_at<f32x2, L>(0));
 #pragma unroll
@@ -88,7 +89,8 @@ template <int L> struct GlobalPairOut {
 // second buffer with cp.async while the current one is transformed in place.
 // HBM and the L2 bound it.  256 points over a 256 x 256 x 144 array in place:
 // 20.9 us with one pencil per thread, 19.2 us with two (7.9 TB/s read + written);
-// 384 points over 384 x 384 x 208: 143 us (8-pencil tiles) and 87 us.
+// 384 points over 384 x 384 x 208: 143 us (8-pencil tiles) and 87 us.  With 128 points so
+// too: RCD 128^3 x 48 with fields in and out 12373 -> 12129 us, 192 x 128 x 256 1999 -> 1946 us.
 template <int L, int P, int NT, int SIGN, int OCC>
 __global__ void __launch_bounds__(NT, OCC) fft_pipe2_kernel(PassParams<float> a) {
     pdl_wait();
@@ -389,7 +391,8 @@ template <int L> struct RealRowPairOut {
     }
 };
 
-// MODE: PASS_PLAIN, PASS_R2C / PASS_C2R (real rows in / real parts out), or PASS_CH_NL (inverse, c = Re / N and g = c^3 - c, forward).
+// MODE: PASS_PLAIN, PASS_R2C / PASS_C2R (real rows in / real parts out), or PASS_CH_NL
+// (inverse, c = Re / N and g = c^3 - c, forward).
 // Measured (rows x length, in place; pipelined one-pencil kernel before): plain
 // 65536 x 256 56.8 -> 51.9 us, 147456 x 384 323 -> 194 us, 32768 x 64 7.6 -> 5.6 us;
 // nonlinear 70.2 -> 60.1, 455 -> 285, 10.0 -> 7.5 us.
