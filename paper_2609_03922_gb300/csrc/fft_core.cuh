@@ -184,6 +184,7 @@ template <typename T> struct PassParams {
     // right of the whole tiles of several rows (pair_tile), fd_seg dividing by the whole
     // tiles of a row
     int edge = 0;
+    int last = 0;   // two-pencil step chain: stop after the update
     // plain passes whose outer index o (strided) or row (rows) runs over fields of
     // seg_n such indices: a tile is skipped when its entries of seg_live are zero
     const uint8_t* seg_live = nullptr;
@@ -724,9 +725,10 @@ __device__ __forceinline__ void transform_pair(cx_t<T>* sm, const tw_t<T>* tw, M
 
 // transform_pair whose first stage reads its inputs through `in` (an
 // elementwise preparation folded into the first stage's loads); at least
-// three stages in all.
+// three stages in all.  only_first: stop after `mid`.
 template <typename T, int L, int P, int NT, int SA, int SB, class LY, class IN, class MID, class OUT>
-__device__ __forceinline__ void transform_pair_in(cx_t<T>* sm, const tw_t<T>* tw, const IN& in, MID& mid, OUT& out) {
+__device__ __forceinline__ void transform_pair_in(cx_t<T>* sm, const tw_t<T>* tw, const IN& in, MID& mid, OUT& out,
+                                                  bool only_first = false) {
     constexpr int NST = NSTAGES<T, L>::value;
     constexpr int R0 = radix_at<T, L>(0), RL = radix_at<T, L>(NST - 1);
     static_assert(NST >= 2, "the first stage must not be the meeting stage");
@@ -735,6 +737,7 @@ __device__ __forceinline__ void transform_pair_in(cx_t<T>* sm, const tw_t<T>* tw
         run_stage_range<T, L, P, NT, SA, LY, 1, NST - 1>(sm, tw);
         FirstStageOut<T, L, R0, LY> fo{sm};
         fused_mid_stage<T, L, P, NT, SA, SB, L / R0, R0, LY>(sm, tw, mid, fo);
+        if (only_first) return;
         __syncthreads();
         run_stage_range<T, L, P, NT, SB, LY, 1, NST - 1>(sm, tw);
         stockham_stage_out<T, L, P, NT, SB, ns_at<T, L>(NST - 1), RL, LY>(sm, tw, out);
@@ -742,6 +745,7 @@ __device__ __forceinline__ void transform_pair_in(cx_t<T>* sm, const tw_t<T>* tw
         run_stage_range<T, L, P, NT, SA, LY, 1, NST - 1>(sm, tw);
         MidOut<T, L, LY, MID> mo{sm, mid};
         stockham_stage_out<T, L, P, NT, SA, ns_at<T, L>(NST - 1), RL, LY>(sm, tw, mo);
+        if (only_first) return;
         __syncthreads();
         run_stages_out<T, L, P, NT, SB, LY>(sm, tw, out);
     }

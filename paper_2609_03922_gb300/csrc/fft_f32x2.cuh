@@ -320,9 +320,10 @@ __global__ void __launch_bounds__(NT, OCC) fft_chain2_kernel(PassParams<float> a
     if (live) {
         ThreadPairIn in{a.in + at, (int)a.isJ};
         ChainMid2<L, H, L / Radices_last<f32x2, L>::value> mid(a, u, edge, at, s_tab, s_kp, cs, pol);
-        transform_pair_in<f32x2, L, H, NT, -1, +1, LY>(sm, s_tw, in, mid, out);
+        transform_pair_in<f32x2, L, H, NT, -1, +1, LY>(sm, s_tw, in, mid, out, a.last != 0);
     } else {
         cp_async_wait<0>();
+        if (a.last) return;
         __syncthreads();
         RawPairIn<H, true> in{cs};
         run_stages_in_out<f32x2, L, H, NT, +1, LY>(sm, s_tw, in, out);

@@ -141,6 +141,7 @@ template <typename T> struct Group {
     // between two steps of one call where the fused update is in force
     Pass<T> chain;
     bool has_chain = false, chain_pairs = false;   // chain_pairs: the two-pencil kernel
+    bool chain_last = false;   // it also takes the update of a call's last step
     bool pre_done = false;          // `work` holds the first inverse pass of c_hat (set by the chain, within a call)
     FftEngine<T> fft1;              // one run's transforms for set/get_field
     // ... whose passes along the rows take the real field in and give it out (complex64; the
@@ -446,6 +447,11 @@ static spdba_status setup_chain(spdba_plan* p, Group<T>& r, int ndim, const int6
     c.p.stream_chat = field <= l2 && 2 * field > l2;
     r.chain = c;
     r.has_chain = true;
+    // At 192 and 384 points the one-pencil update pass is slower than the whole chain (66
+    // against 50 us over 192 x 128 x 256, 356 against 229 over 384 x 384 x 208); at powers of
+    // two it is the faster one (46 against 57 over 256 x 256 x 144).  With fields in and out:
+    // 192 x 128 x 256, 20 steps 1946 -> 1919 us; 384^3 half, 10 steps 6103 -> 5949 us.
+    r.chain_last = r.chain_pairs && d[0] % 3 == 0;
     return SPDBA_OK;
 }
 
@@ -965,6 +971,15 @@ template <typename T> static spdba_status ch_chain(spdba_plan* p, Group<T>& r, i
     return SPDBA_OK;
 }
 
+// The fused update of a step that no other follows: `upd`, or where r.chain_last the
+// chain's kernel stopped after the update.
+template <typename T> static Pass<T> last_update(const Group<T>& r, const Pass<T>& upd) {
+    if (!r.chain_last) return upd;
+    Pass<T> ps = r.chain;
+    ps.p.last = 1;
+    return ps;
+}
+
 // more: another step of this group follows in the same call (or captured segment).
 template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>& r, bool more) {
     cudaStream_t st = p->st;
@@ -1031,7 +1046,7 @@ template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>&
         p->launches += 4;
         if (chain) return ch_chain<T>(p, r, dense, 4.0 * hb);
         if (r.fused_update) {
-            Pass<T> ps = r.h_upd;
+            Pass<T> ps = last_update<T>(r, r.h_upd);
             ps.p.fu.dense = dense;
             ProfScope pr(p, K_FFT_UPDATE, 3.0 * hb);
             if ((s = launch_pass<T>(ps, r.work, r.work, st)) != SPDBA_OK) return s;
@@ -1133,7 +1148,7 @@ template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>&
         if (last_fused && chain) return ch_chain<T>(p, r, dense, 2.0 * pass_bytes);
         if (last_fused) {
             // forward transform of the first axis + update; traffic depends on the states
-            Pass<T> ps = r.upd_pass;
+            Pass<T> ps = last_update<T>(r, r.upd_pass);
             ps.p.fu.dense = dense;
             ProfScope pr(p, K_FFT_UPDATE, pass_bytes + sizeof(cx_t<T>) * (double)(r.batch * r.n));
             if ((s = launch_pass<T>(ps, r.work, r.work, st)) != SPDBA_OK) return s;

@@ -68,3 +68,24 @@ def test_many_block_rows():
             outs.append((p.get_spectrum(), p.get_mask()))
     assert np.array_equal(outs[0][0].view(np.float32), outs[1][0].view(np.float32))
     assert np.array_equal(outs[0][1], outs[1][1])
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("dims,block,kw", [((192, 64), (8, 16), {}), ((384, 128), (16, 8), {"force_dc": 0}),
+                                           ((192, 16, 64), (8, 8, 8), {"half_spectrum": 0}),
+                                           ((384, 64, 64), (16, 4, 8), {"half_storage": 1})])
+def test_last_update_equals_staged(dims, block, kw, mode):
+    """The fused update of a call's last step at 192 and 384 points (the chain's kernel without its
+    inverse) against the staged update, bit for bit."""
+    from paper_2609_03922_gb300 import spdba
+    x = _field(dims)
+    outs = []
+    for fuse in (1, 0):
+        with spdba.Plan(dims, block, threshold=0.6, reassess=3, mode=mode, dt=0.02, fuse_update=fuse, **kw) as p:
+            p.set_field(x)
+            for n in (1, 1, 3, 2):
+                p.step(n)
+            outs.append((p.get_spectrum(), p.get_mask(), p.get_stats()["active_ratio_sum"]))
+    assert np.array_equal(outs[0][0].view(np.float32), outs[1][0].view(np.float32))
+    assert np.array_equal(outs[0][1], outs[1][1])
+    assert outs[0][2] == outs[1][2]
