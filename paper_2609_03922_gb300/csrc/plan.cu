@@ -256,6 +256,7 @@ struct SegGraph {
 
 struct spdba_plan {
     spdba_options opt;
+    int device = 0;         // the GPU that holds the buffers and runs the kernels
     MultiForm multi[2];     // tile tables of 4096 and 2048 elements
     int multi_sel = 0;      // form in force: 0 = per group, 1 / 2 = multi[0] / multi[1]
     std::vector<void*> multi_bufs;   // device buffers of the multi-size forms
@@ -1663,10 +1664,24 @@ template <typename T> static spdba_status plan_step(spdba_plan* p, int64_t n) {
     return SPDBA_OK;
 }
 
+// Whether the plan's kernels may take the caller's buffer themselves: device memory of the plan's
+// GPU.  Any other (another GPU's, readable by a copy with or without peer access, or managed
+// memory) is copied from or to.
+static bool takes_pointer(const spdba_plan* p, const void* ptr, int on_dev) {
+    if (!on_dev) return false;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess) {
+        cudaGetLastError();   // the copy that follows reports a bad pointer
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == p->device;
+}
+
 template <typename T>
 static spdba_status run_set_field(spdba_plan* p, Group<T>& r, long long sub, const void* src, int on_dev) {
     cudaStream_t st = p->st;
     spdba_status s;
+    const bool direct = takes_pointer(p, src, on_dev);
     cx_t<T>* slot = r.c_hat + sub * r.n;
     cx_t<T>* wslot = r.work + sub * r.n;
     const cudaMemcpyKind kind = on_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
@@ -1674,7 +1689,7 @@ static spdba_status run_set_field(spdba_plan* p, Group<T>& r, long long sub, con
         const bool rcd = p->opt.model == SPDBA_MODEL_RCD;
         const long long tot = r.n * r.ncomp;
         const T* field = reinterpret_cast<const T*>(src);
-        if (!on_dev || !r.has_real_rows) {
+        if (!direct || !r.has_real_rows) {
             SPDBA_CUDA(cudaMemcpyAsync(r.real, src, sizeof(T) * tot, kind, st));
             field = r.real;
         }
@@ -1696,9 +1711,9 @@ static spdba_status run_set_field(spdba_plan* p, Group<T>& r, long long sub, con
             }
         }
     } else {
-        // a device signal on a 16-byte boundary is read where it lies
+        // a signal of this GPU on a 16-byte boundary is read where it lies
         const cx_t<T>* from = reinterpret_cast<const cx_t<T>*>(src);
-        if (!on_dev || ((uintptr_t)src & 15)) {
+        if (!direct || ((uintptr_t)src & 15)) {
             SPDBA_CUDA(cudaMemcpyAsync(wslot, src, sizeof(cx_t<T>) * r.n, kind, st));
             from = wslot;
         }
@@ -1731,6 +1746,7 @@ template <typename T>
 static spdba_status run_get_field(spdba_plan* p, Group<T>& r, long long sub, void* dst, int on_dev) {
     cudaStream_t st = p->st;
     spdba_status s;
+    const bool direct = takes_pointer(p, dst, on_dev);
     cx_t<T>* slot = r.c_hat + sub * r.n;
     cx_t<T>* wslot = r.work + sub * r.n;
     const cudaMemcpyKind kind = on_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
@@ -1738,7 +1754,7 @@ static spdba_status run_get_field(spdba_plan* p, Group<T>& r, long long sub, voi
         const bool rcd = p->opt.model == SPDBA_MODEL_RCD;
         const long long tot = r.n * r.ncomp;
         // the row passes write the real field: to the caller's buffer, or staged for the host
-        T* field = on_dev && r.has_real_rows ? reinterpret_cast<T*>(dst) : r.real;
+        T* field = direct && r.has_real_rows ? reinterpret_cast<T*>(dst) : r.real;
         if (r.hs) {
             if ((s = launch_pass<T>(r.h_inv_z, r.c_hat, r.work, st)) != SPDBA_OK) return s;
             if ((s = launch_pass<T>(r.h_inv_y, r.work, r.work, st)) != SPDBA_OK) return s;
@@ -1759,7 +1775,7 @@ static spdba_status run_get_field(spdba_plan* p, Group<T>& r, long long sub, voi
         }
         if (field == r.real) SPDBA_CUDA(cudaMemcpyAsync(dst, r.real, sizeof(T) * tot, kind, st));
     } else {
-        cx_t<T>* to = on_dev && ((uintptr_t)dst & 15) == 0 ? reinterpret_cast<cx_t<T>*>(dst) : wslot;
+        cx_t<T>* to = direct && ((uintptr_t)dst & 15) == 0 ? reinterpret_cast<cx_t<T>*>(dst) : wslot;
         if (!r.long_nls) {
             if ((s = r.fft1.exec(slot, to, SPDBA_INVERSE, st)) != SPDBA_OK) return s;
         } else {
@@ -1966,6 +1982,7 @@ extern "C" spdba_status spdba_batch_create(spdba_plan** out, int32_t nruns, int3
     p->reassess = reassess;
     p->precision = o.precision;
     p->st = (cudaStream_t)o.stream;
+    if (cudaGetDevice(&p->device) != cudaSuccess) cudaGetLastError();   // the allocations report a missing GPU
     s = p->precision == SPDBA_C64 ? build_groups<float>(p, nruns, ndim, dims, block)
                                   : build_groups<double>(p, nruns, ndim, dims, block);
     if (s == SPDBA_OK && p->precision == SPDBA_C64 && ndim == 2) {
