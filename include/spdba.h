@@ -169,8 +169,9 @@ void spdba_options_default(spdba_options* opt);
 /*
  * Create a plan for one field (spdba_init of S2.1).
  *   ndim        1, 2 or 3 (NLS: 1; CH: 2 or 3)
- *   dims[ndim]  grid extents; CH axes in {16, 32, 64, 128, 192, 256, 384, 512};
- *               NLS lengths 64..4096 (powers of two) and n1 * 512 with n1 in
+ *   dims[ndim]  grid extents; CH axes in {16, 32, 64, 128, 192, 256, 384, 512}, with
+ *               half storage also 1024 and 2048 along the first two; NLS lengths
+ *               64..4096 (powers of two) and n1 * 512 with n1 in
  *               {16, 32, ..., 512} (up to 2^18); other lengths of the form
  *               2^a 3^b return SPDBA_ERR_UNSUPPORTED
  *   block[ndim] block edge per axis; must divide dims; the block map is
