@@ -1,6 +1,7 @@
 // Host side of the Stockham FFT: FP64 twiddle tables, pass planning, the
 // kernel-level FFT entry points, and the library's error reporting.
 #include <atomic>
+#include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
 
@@ -150,12 +151,15 @@ spdba_status make_pass(Pass<T>* out, int64_t L, int sign, int mode, long long O,
     };
     // A pass of fewer wide tiles than SMs takes narrow ones (128 x 128: 8 against
     // 32 tiles).  complex128 passes, bound by the SMs' FP64 rate, do so up to four
-    // wide tiles an SM, to spread evenly.
-    const long long few = (sizeof(T) == 8 ? 4 : 1) * (long long)nsm;
+    // wide tiles an SM where that is the shorter way: wide tiles take whole rounds of the
+    // SMs, narrow ones spread evenly at ki.cost times the work.  Rows of 128 points, wide
+    // against narrow: 0.5 tiles an SM 16.6 / 12.7 us, 2 30.2 / 42.4, 4 58.1 / 81.5; of 64
+    // points 14.3 / 8.7, 1.5 26.0 / 20.2, 3.5 49.8 / 46.7.
     bool ok = get(TILE_WIDE);
-    if (ok && O * I < few * ki.P) {
+    if (ok && O * I < (sizeof(T) == 8 ? 4 : 1) * (long long)nsm * ki.P) {
         const KernelInfo wide = ki;
-        if (!get(TILE_NARROW) || I % ki.P != 0) ki = wide;
+        const double tiles = (double)(O * I) / ((double)nsm * wide.P);   // wide tiles an SM
+        if (!get(TILE_NARROW) || I % ki.P != 0 || ki.cost * tiles >= ceil(tiles)) ki = wide;
     }
     bool generic = !ok || I % ki.P != 0;
     if (sizeof(T) == 4 && !chain && mode == PASS_PLAIN && !loadp && storep) {
@@ -180,6 +184,20 @@ spdba_status make_pass(Pass<T>* out, int64_t L, int sign, int mode, long long O,
         SPDBA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ki.func, ki.NT, ki.smem));
         if (per_sm < 1) per_sm = 1;
         long long resident = (long long)per_sm * nsm;
+        if (sizeof(T) == 8 && grid > resident) {
+            // The FP64 rate of the SM with the most tiles bounds a pass: as many CTAs per SM as
+            // leave the fewest tiles on any.  The CTAs of the last round are the first ones, of
+            // which some SMs hold two (4 of 152): 608 tiles on 3 CTAs an SM are 5 on those, on 2
+            // they are 4: 81.9 and 66.5 us for rows of 256 points.  Fewer than eight warps an SM
+            // lose an eighth of the rate (strided passes of 256 over 65536 pencils: 1275 us on 3
+            // CTAs, 1373 on one).
+            auto load = [&](long long k) {
+                const long long g = k * nsm, last = ntiles % g, spread = nsm - nsm / 16;
+                return (double)(k * (ntiles / g) + (last + spread - 1) / spread) * (k * ki.NT < 256 ? 1.125 : 1.0);
+            };
+            for (long long k = per_sm - 1; k * ki.NT >= 128; --k)
+                if (load(k) < load(resident / nsm)) resident = k * nsm;
+        }
         if (grid > resident) grid = resident;
     }
     s = SPDBA_OK;

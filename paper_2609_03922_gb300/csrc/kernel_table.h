@@ -7,6 +7,7 @@ struct KernelInfo {
     const void* func = nullptr;
     int P = 0, NT = 0, smem = 0;
     bool pipe = false;  // persistent, double-buffered kernel: grid = resident CTAs
+    double cost = 1;    // of a narrow tile: time of a pencil against the wide tile's, the SMs full
 };
 // Tile sizes of a pass: TILE_WIDE fills 128-byte rows and a CTA; TILE_NARROW is for
 // passes of fewer wide tiles than the GPU has SMs; TILE_GENERIC takes any
