@@ -1021,10 +1021,10 @@ constexpr int kUpdTable = 4096;
 constexpr int kPairTable = 1024;
 __host__ __device__ __forceinline__ int upd_table_cols(int P, int bx) { return (P + bx - 2) / bx + 1; }
 // The update pass stages c_hat in a third tile buffer for row-major tiles of
-// L <= 256 whose last stage emits directly (not the radix-3 tail of 192).
-template <typename T, int L> __host__ __device__ constexpr bool upd_stages_chat() {
-    return L <= 256 && Radices_last<T, L>::value != 3;
-}
+// L <= 256, where its CTAs still overlap. Not at 192 points, where the buffer costs a CTA: a step
+// over 192 x 128 x 256 takes 116 us with it and 106 without (complex128 2179 and 2147), over
+// 192 x 192 x 64 52.9 and 46.8 (844 and 827).
+template <typename T, int L> __host__ __device__ constexpr bool upd_stages_chat() { return L <= 256 && L != 192; }
 
 // Update emitted from the forward transform's last stage (tile within one row):
 // each output is updated and stored from registers.  With CS the tile's
@@ -1257,9 +1257,7 @@ __device__ __forceinline__ void pipe_tile(cx_t<T>* sm, cx_t<T>* chat, const Pass
     using LY = PipeLayout<L, P, PFAST>;
     // direct stores from the last stage stay coalesced when a warp's lanes
     // cover at least 32 contiguous bytes of each output row
-    // (the radix-3 tails of 192 and 384 hold too many registers to emit directly)
-    constexpr bool DIRECT = (LY::PMAP || (L / Radices_last<T, L>::value) * (int)sizeof(C) >= 32) &&
-                            Radices_last<T, L>::value != 3;
+    constexpr bool DIRECT = LY::PMAP || (L / Radices_last<T, L>::value) * (int)sizeof(C) >= 32;
     if constexpr (MODE == PASS_PLAIN && PFAST) {
         if (a.tw4 != nullptr) {
             FourStepOut<T, L, SIGN> out(a, q0);
