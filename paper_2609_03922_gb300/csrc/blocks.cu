@@ -373,6 +373,11 @@ spdba_status launch_tau(const double* gmax, int nruns, double threshold, int tau
 // 256 blocks per CTA: a 32^3 map then reaches 128 SMs (with 1024 it ran on 32, and
 // on 18 for the stored half of 256^3: 12.7 us).
 constexpr int CLS_NT = 256;
+// A CTA of the compaction adds up the counts of all CTAs before it, which grows with their
+// number squared: maps above this many blocks take CTAs of 1024.  A classification with CTAs
+// of 256 and of 1024 blocks: 2^21 blocks 79.8 and 80.0 us, 2^22 121 and 115, 2^24 998 and 652.
+constexpr int CLS_NT_LARGE = 1024;
+constexpr long long CLS_LARGE = 2LL << 20;
 
 // Block coordinates (32-bit: block maps hold fewer than 2^31 blocks).
 struct BCoord {
@@ -512,19 +517,20 @@ __device__ __forceinline__ bool has_active_nbr(const Geom& g, const uint8_t* act
 // TRANSITION iff not active and a face neighbour (periodic) is active; chi bit
 // 2a / 2a+1 marks a FROZEN lower / upper neighbour along local axis a (axis 0
 // = slowest axis of the field).  One CTA-sized count per CTA goes to scratch.
-__global__ void __launch_bounds__(CLS_NT) state_kernel(Geom g, const uint8_t* __restrict__ active, int transitions,
-                                                       uint8_t* __restrict__ states, uint8_t* __restrict__ chi,
-                                                       int* __restrict__ cta_count, DevStats* stats,
-                                                       double* gmax_reset, int nruns) {
+template <int NT>
+__global__ void __launch_bounds__(NT) state_kernel(Geom g, const uint8_t* __restrict__ active, int transitions,
+                                                   uint8_t* __restrict__ states, uint8_t* __restrict__ chi,
+                                                   int* __restrict__ cta_count, DevStats* stats, double* gmax_reset,
+                                                   int nruns) {
     pdl_wait();
-    long long b = (long long)blockIdx.x * CLS_NT + threadIdx.x;
+    long long b = (long long)blockIdx.x * NT + threadIdx.x;
     long long nb = g.blocks();
     // the activity maxima were consumed by the previous kernel: zero them for the next scan
     if (gmax_reset != nullptr && blockIdx.x == 0)
-        for (int r = threadIdx.x; r < 2 * nruns; r += CLS_NT) gmax_reset[r] = 0.0;
+        for (int r = threadIdx.x; r < 2 * nruns; r += NT) gmax_reset[r] = 0.0;
     // and the mass (or power) accumulators for the pass that follows a state setting
     if (stats && blockIdx.x == 0)
-        for (long long r = threadIdx.x; r < g.runs(); r += CLS_NT) stats[r].mass = 0.0;
+        for (long long r = threadIdx.x; r < g.runs(); r += NT) stats[r].mass = 0.0;
     int st = 0;
     uint8_t cb = 0;
     if (b < nb) {
@@ -562,13 +568,13 @@ __global__ void __launch_bounds__(CLS_NT) state_kernel(Geom g, const uint8_t* __
         // per-run counts: one atomic per CTA when a CTA never straddles runs (the
         // counters of a run are one address: per-warp atomics would queue on it),
         // else one per warp when a warp never straddles runs
-        if (bpr % CLS_NT == 0) {
+        if (bpr % NT == 0) {
             if ((threadIdx.x & 31) == 0) {
                 atomicAdd(&s_na, __popc(na));
                 atomicAdd(&s_nt, __popc(nt));
             }
             __syncthreads();
-            const long long b0 = (long long)blockIdx.x * CLS_NT;
+            const long long b0 = (long long)blockIdx.x * NT;
             if (threadIdx.x == 0 && b0 < nb) {
                 const long long run = b0 / bpr;
                 if (s_na) atomicAdd(&stats[run].n_active, (unsigned long long)s_na);
@@ -592,12 +598,13 @@ __global__ void __launch_bounds__(CLS_NT) state_kernel(Geom g, const uint8_t* __
 
 // Ordered compaction: CTA c starts at the sum of the counts of CTAs before it
 // and places its non-frozen ids with a warp-ballot prefix and a block scan.
-__global__ void __launch_bounds__(CLS_NT) compact_kernel(Geom g, const uint8_t* __restrict__ states,
-                                                         const int* __restrict__ cta_count, int ncta,
-                                                         int32_t* __restrict__ list, int32_t* __restrict__ count) {
+template <int NT>
+__global__ void __launch_bounds__(NT) compact_kernel(Geom g, const uint8_t* __restrict__ states,
+                                                     const int* __restrict__ cta_count, int ncta,
+                                                     int32_t* __restrict__ list, int32_t* __restrict__ count) {
     pdl_wait();
     __shared__ int s_base;
-    __shared__ int s_warp[CLS_NT / 32];
+    __shared__ int s_warp[NT / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (w == 0) {
         int acc = 0;
@@ -606,20 +613,20 @@ __global__ void __launch_bounds__(CLS_NT) compact_kernel(Geom g, const uint8_t* 
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (lane == 0) s_base = acc;
     }
-    long long b = (long long)blockIdx.x * CLS_NT + threadIdx.x;
+    long long b = (long long)blockIdx.x * NT + threadIdx.x;
     bool keep = b < g.blocks() && states[b] != 0;
     unsigned m = __ballot_sync(0xffffffffu, keep);
     if (lane == 0) s_warp[w] = __popc(m);
     __syncthreads();
     if (w == 0) {
-        int v = lane < CLS_NT / 32 ? s_warp[lane] : 0;
+        int v = lane < NT / 32 ? s_warp[lane] : 0;
         int incl = v;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             int t = __shfl_up_sync(0xffffffffu, incl, o);
             if (lane >= o) incl += t;
         }
-        if (lane < CLS_NT / 32) s_warp[lane] = incl - v;
+        if (lane < NT / 32) s_warp[lane] = incl - v;
         if (blockIdx.x == (unsigned)(ncta - 1) && lane == 31) *count = s_base + incl;
     }
     __syncthreads();
@@ -627,6 +634,23 @@ __global__ void __launch_bounds__(CLS_NT) compact_kernel(Geom g, const uint8_t* 
         int pos = s_base + s_warp[w] + __popc(m & ((1u << lane) - 1u));
         list[pos] = (int32_t)b;
     }
+}
+
+// States and the list of non-frozen blocks from the active flags.
+template <int NT>
+static void launch_states(const Geom& g, const uint8_t* active, int transitions, uint8_t* states, uint8_t* chi,
+                          int32_t* list, int32_t* count, int* cta_count, DevStats* stats, double* gmax_reset,
+                          cudaStream_t st) {
+    const int ncta = (int)((g.blocks() + NT - 1) / NT);
+    pdl_launch(state_kernel<NT>, ncta, NT, 0, st, g, active, transitions, states, chi, cta_count, stats, gmax_reset,
+               (int)g.runs());
+    pdl_launch(compact_kernel<NT>, ncta, NT, 0, st, g, states, cta_count, ncta, list, count);
+}
+static void launch_states(const Geom& g, const uint8_t* active, int transitions, uint8_t* states, uint8_t* chi,
+                          int32_t* list, int32_t* count, int* cta_count, DevStats* stats, double* gmax_reset,
+                          cudaStream_t st) {
+    (g.blocks() > CLS_LARGE ? launch_states<CLS_NT_LARGE> : launch_states<CLS_NT>)(
+        g, active, transitions, states, chi, list, count, cta_count, stats, gmax_reset, st);
 }
 
 __global__ void zero_counts_kernel(DevStats* stats, long long nruns) {
@@ -644,12 +668,10 @@ spdba_status launch_classify(const Geom& g, const double* msq, int msq_is_square
                              int transitions, int all_active, uint8_t* active, uint8_t* states, uint8_t* chi,
                              int32_t* list, int32_t* count, void* scratch, DevStats* stats, cudaStream_t st) {
     long long nb = g.blocks();
-    int ncta = (int)((nb + CLS_NT - 1) / CLS_NT);
     if (stats) pdl_launch(zero_counts_kernel, 1, 256, 0, st, stats, g.runs());
     pdl_launch(active_kernel, (unsigned)((nb + 255) / 256), 256, 0, st, g, msq, msq_is_square, tau, force_dc, all_active,
                                                                  active);
-    pdl_launch(state_kernel, ncta, CLS_NT, 0, st, g, active, transitions, states, chi, (int*)scratch, stats, nullptr, 0);
-    pdl_launch(compact_kernel, ncta, CLS_NT, 0, st, g, states, (const int*)scratch, ncta, list, count);
+    launch_states(g, active, transitions, states, chi, list, count, (int*)scratch, stats, nullptr, st);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
 }
@@ -659,12 +681,9 @@ spdba_status launch_classify_from_scan(const Geom& g, const double* msq, int msq
                                        double* tau, uint8_t* active, uint8_t* states, uint8_t* chi, int32_t* list,
                                        int32_t* count, void* scratch, DevStats* stats, cudaStream_t st) {
     long long nb = g.blocks();
-    int ncta = (int)((nb + CLS_NT - 1) / CLS_NT);
     pdl_launch(active_tau_kernel, (unsigned)((nb + 255) / 256), 256, 0, st, g, msq, msq_is_square, gmax, threshold, tau_rule,
                                                                       exclude_dc, force_dc, tau, stats, active);
-    pdl_launch(state_kernel, ncta, CLS_NT, 0, st, g, active, transitions, states, chi, (int*)scratch, stats, gmax,
-                                          (int)g.runs());
-    pdl_launch(compact_kernel, ncta, CLS_NT, 0, st, g, states, (const int*)scratch, ncta, list, count);
+    launch_states(g, active, transitions, states, chi, list, count, (int*)scratch, stats, gmax, st);
     SPDBA_CUDA(cudaGetLastError());
     return SPDBA_OK;
 }
