@@ -981,13 +981,16 @@ template <typename T> static Pass<T> last_update(const Group<T>& r, const Pass<T
     return ps;
 }
 
+// Whether the steps of a group chain where another follows (fixed by the launch configuration).
+template <typename T> static bool chains(const Group<T>& r) { return r.has_chain && r.fused_update && !r.use_half; }
+
 // more: another step of this group follows in the same call (or captured segment).
 template <typename T> static spdba_status group_ch_step(spdba_plan* p, Group<T>& r, bool more) {
     cudaStream_t st = p->st;
     spdba_status s;
     prof_select(p, r.step);
     // between two steps the fused update runs as a chain into the next step's first inverse pass
-    const bool chain = more && r.has_chain && r.fused_update && !r.use_half;
+    const bool chain = more && chains<T>(r);
     const bool adaptive = p->opt.mode == SPDBA_MODE_ADAPTIVE;
     const int interval = p->pred ? p->horizon : p->reassess;
     const bool reassess = adaptive && (!r.assessed || r.step % interval == 0);
@@ -1601,7 +1604,16 @@ template <typename T> static bool segment_ready(spdba_plan* p) {
     return true;
 }
 
-// Whether every CH group holds its first inverse pass (a chain ended the last step).
+// Whether any group's steps chain, and whether one holds its first inverse pass (a chain ended the
+// last step).  Which groups chain is fixed while the plan's graphs live (a change of the launch
+// configuration releases them), so that one bit tells the state of all.  The multi-size form's do
+// not.
+template <typename T> static bool any_chains(spdba_plan* p) {
+    if (p->multi_sel > 0) return false;
+    for (auto& g : groups<T>(p))
+        if (chains<T>(*g)) return true;
+    return false;
+}
 template <typename T> static bool chained(spdba_plan* p) {
     for (auto& g : groups<T>(p))
         if (g->pre_done) return true;
@@ -1618,9 +1630,9 @@ template <typename T> static spdba_status plan_step(spdba_plan* p, int64_t n) {
     int64_t i = 0;
     while (i < n) {
         if (n - i >= R && segment_ready<T>(p)) {
-            // the launches differ with the step before (chained into this segment or not)
-            // and with whether steps follow: one graph each
-            const bool more = n - i > R;
+            // where steps chain, the launches differ with the step before (chained into this
+            // segment or not) and with whether steps follow: one graph each
+            const bool more = n - i > R && any_chains<T>(p);
             SegGraph& sg = p->seg[(chained<T>(p) ? 1 : 0) + (more ? 2 : 0)];
             if (!sg.exec) {
                 const long long l0 = p->launches, u0 = p->list_updates;
@@ -1649,7 +1661,7 @@ template <typename T> static spdba_status plan_step(spdba_plan* p, int64_t n) {
                 for (auto& g : groups<T>(p)) {
                     g->step += R;
                     if (p->opt.mode == SPDBA_MODE_ADAPTIVE) g->assessed = true;
-                    g->pre_done = sg.chain_out && g->has_chain && g->fused_update && !g->use_half;
+                    g->pre_done = sg.chain_out && chains<T>(*g);
                 }
                 p->launches += sg.launches;
                 p->list_updates += sg.list_updates;
