@@ -174,10 +174,12 @@ def _ptr(x):
 
 
 def current_stream():
-    """Handle of torch's current stream (without the Stream object around it, which costs
-    as much as a kernel launch)."""
+    """Handle of torch's current stream.  torch's own accessor leaves out the Stream object, which
+    costs as much as a kernel launch; it is not part of torch's public interface, so a torch
+    without it is asked for the object."""
     import torch
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return torch.cuda.current_stream().cuda_stream if raw is None else raw(torch.cuda.current_device())
 
 
 def options_default(**kw):
