@@ -130,7 +130,7 @@ static spdba_status ensure_smem_attr(const void* f, int smem, bool max_carveout)
 template <typename T>
 spdba_status make_pass(Pass<T>* out, int64_t L, int sign, int mode, long long O, long long I, long long isO,
                        long long isI, long long isJ, long long osO, long long osI, long long osJ,
-                       TwiddleCache<T>& tw, cudaStream_t st, bool fourstep) {
+                       TwiddleCache<T>& tw, cudaStream_t st, bool fourstep, long long field) {
     bool loadp = (isJ != 1), storep = (osJ != 1);
     if (loadp && isI != 1) return fail(SPDBA_ERR_UNSUPPORTED, "pass without a unit-stride input direction");
     if (storep && osI != 1) return fail(SPDBA_ERR_UNSUPPORTED, "pass without a unit-stride output direction");
@@ -156,10 +156,11 @@ spdba_status make_pass(Pass<T>* out, int64_t L, int sign, int mode, long long O,
     // against narrow: 0.5 tiles an SM 16.6 / 12.7 us, 2 30.2 / 42.4, 4 58.1 / 81.5; of 64
     // points 14.3 / 8.7, 1.5 26.0 / 20.2, 3.5 49.8 / 46.7.
     bool ok = get(TILE_WIDE);
-    if (ok && O * I < (sizeof(T) == 8 ? 4 : 1) * (long long)nsm * ki.P) {
+    const bool straddles = ok && field > 0 && field % ki.P != 0;
+    if (ok && (straddles || O * I < (sizeof(T) == 8 ? 4 : 1) * (long long)nsm * ki.P)) {
         const KernelInfo wide = ki;
         const double tiles = (double)(O * I) / ((double)nsm * wide.P);   // wide tiles an SM
-        if (!get(TILE_NARROW) || I % ki.P != 0 || ki.cost * tiles >= ceil(tiles)) ki = wide;
+        if (!get(TILE_NARROW) || I % ki.P != 0 || (!straddles && ki.cost * tiles >= ceil(tiles))) ki = wide;
     }
     bool generic = !ok || I % ki.P != 0;
     if (sizeof(T) == 4 && !chain && mode == PASS_PLAIN && !loadp && storep) {
@@ -251,8 +252,9 @@ spdba_status make_axis_pass(Pass<T>* out, int ndim, const int64_t* dims, int64_t
     for (int a = 0; a < axis; ++a) O *= dims[a];
     for (int a = axis + 1; a < ndim; ++a) I *= dims[a];
     if (I == 1) {
-        // contiguous pencils: index them as the inner direction
-        return make_pass<T>(out, L, sign, mode, 1, O, 0, L, 1, 0, L, 1, tw, st);
+        // contiguous pencils: index them as the inner direction; the nonlinear pass adds up the
+        // mass of the one field its tile lies in
+        return make_pass<T>(out, L, sign, mode, 1, O, 0, L, 1, 0, L, 1, tw, st, false, mode == PASS_CH_NL ? O / batch : 0);
     }
     return make_pass<T>(out, L, sign, mode, O, I, L * I, 1, I, L * I, 1, I, tw, st);
 }
@@ -346,10 +348,10 @@ template struct FftEngine<float>;
 template struct FftEngine<double>;
 template spdba_status make_pass<float>(Pass<float>*, int64_t, int, int, long long, long long, long long, long long,
                                        long long, long long, long long, long long, TwiddleCache<float>&,
-                                       cudaStream_t, bool);
+                                       cudaStream_t, bool, long long);
 template spdba_status make_pass<double>(Pass<double>*, int64_t, int, int, long long, long long, long long, long long,
                                         long long, long long, long long, long long, TwiddleCache<double>&,
-                                        cudaStream_t, bool);
+                                        cudaStream_t, bool, long long);
 // Half-spectrum passes of a 3-D complex64 field (see fft_half.cuh).
 spdba_status make_half_pass(Pass<float>* out, int mode, const HalfGeo& hg, TwiddleCache<float>& tw, cudaStream_t st) {
     const bool rows = mode == PASS_NL_HALF || mode == PASS_R2C_HALF || mode == PASS_C2R_HALF;

@@ -58,11 +58,11 @@ template <typename T> struct Pass {
 };
 
 // Build a pass of length L over pencils (O, I) with the given strides; fourstep: the
-// caller adds four-step twiddles.
+// caller adds four-step twiddles; field: a tile's pencils belong to one run of so many (0: any).
 template <typename T>
 spdba_status make_pass(Pass<T>* out, int64_t L, int sign, int mode, long long O, long long I,
                        long long isO, long long isI, long long isJ, long long osO, long long osI,
-                       long long osJ, TwiddleCache<T>& tw, cudaStream_t st, bool fourstep = false);
+                       long long osJ, TwiddleCache<T>& tw, cudaStream_t st, bool fourstep = false, long long field = 0);
 template <typename T> spdba_status launch_pass(const Pass<T>& ps, const void* in, void* out, cudaStream_t st);
 
 // Puts another kernel under a pass (same pencils, one CTA per tile).
