@@ -68,8 +68,7 @@ def prof_every(k):
 
 # DRAM bytes (read + write) per launch from ncu captures of the current kernels
 # on the 256^3 field with half-spectrum storage (averages over the first steps after
-# time 5, cold L2 at the start of each launch;
-# profiles/case_launch_lists.md; the staged kernels' from ch3d256_half_storage_step_kernels.md):
+# time 5; the staged kernels' at step 505; cold L2 at the start of each launch):
 TOUCHED_BYTES = {
     # x pass (two real rows per transform, two transforms per thread)
     "fft_fused_nl": 75.54e6 + 12.42e6,

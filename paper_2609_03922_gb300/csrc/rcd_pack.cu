@@ -5,7 +5,13 @@
 // Z = h_a + i h_b is Re(IFFT(u_a)) + i Re(IFFT(u_b)), and the transform W of
 // R_a + i R_b separates into R_a(k) = (W(k) + conj W(-k)) / 2 and R_b(k) = (W(k) -
 // conj W(-k)) / (2 i), which the update does as it reads W.  Every pass between the
-// two moves half the data, the reaction too.  The inverse starts with the rows, where
+// two moves half the data, the reaction too.  The two components of a field share the rounding
+// of its transforms, relative to the larger one; so do all M in the update, whose product with
+// the eigenvectors of D mixes them.  Measured against complex128 over 1, 20 and 100 steps, with every
+// other component 1, 1e-3, 1e-6 or 0 of its neighbour (M = 2, 3, 8, 64 x 64 and 32 x 32 x 64, with and
+// without cross diffusion), each component's error is that of the M separate transforms; alone
+// two components without cross diffusion, one exactly zero, differ: it stays within 3e-12 of the other
+// one, 5e-17 before.  The inverse starts with the rows, where
 // Z is formed (this file); rows r and -r are needed together, and share a thread.
 #include <algorithm>
 
@@ -201,7 +207,7 @@ spdba_status rcd_pack_prepare(RcdPack* o, int ndim, const int64_t* d, int M, Twi
         case 64: pack_info<64, 8, 64, 8>(o); break;
         case 128: pack_info<128, 8, 64, 6>(o); break;
         case 256: pack_info<256, 4, 64, 6>(o); break;
-        default: return SPDBA_OK;
+        default: return SPDBA_OK;   // no packing kernel is built for other rows: they keep the M transforms
     }
     // at most 34 KB; the whole carveout, so that as many CTAs fit as the registers allow
     SPDBA_CUDA(cudaFuncSetAttribute(o->func, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
