@@ -448,10 +448,10 @@ static spdba_status setup_chain(spdba_plan* p, Group<T>& r, int ndim, const int6
     c.p.stream_chat = field <= l2 && 2 * field > l2;
     r.chain = c;
     r.has_chain = true;
-    // At 192 and 384 points the one-pencil update pass is slower than the whole chain (66
-    // against 50 us over 192 x 128 x 256, 356 against 229 over 384 x 384 x 208); at powers of
-    // two it is the faster one (46 against 57 over 256 x 256 x 144).  With fields in and out:
-    // 192 x 128 x 256, 20 steps 1946 -> 1919 us; 384^3 half, 10 steps 6103 -> 5949 us.
+    // At 192 and 384 points the one-pencil update pass is slower than the chain's kernel stopped
+    // after the update (56 against 34 us over 192 x 128 x 256, 356 against 169 over 384 x 384 x 208);
+    // at powers of two it is the faster one (46 against 57 for the whole chain over 256 x 256 x
+    // 144).  With fields in and out: 384^3 half, 10 steps 6103 -> 5949 us.
     r.chain_last = r.chain_pairs && d[0] % 3 == 0;
     return SPDBA_OK;
 }
@@ -596,8 +596,8 @@ static spdba_status group_init_ch_hs(spdba_plan* p, Group<float>& r, const int64
         if ((s = setup_chain<float>(p, r, 3, dh, 1)) != SPDBA_OK) return s;
         if (r.has_chain) {
             // edge tiles: whole tiles up to N2 / 2, then P / 4 rows a tile (its state table has a
-            // column per row of blocks among them).  64^3, 40 steps: 726 -> 702 us (192 tiles become
-            // 144, one round of the SMs); 256^3, 20 steps: 2757 -> 2739 us; 384^3, which lies outside
+            // column per row of blocks among them).  64^3, 40 steps: 711 -> 709 us (192 tiles become
+            // 144, one round of the SMs); 256^3, 20 steps: 2696 -> 2669 us; 384^3, which lies outside
             // the L2 and pays for the scattered sectors in HBM accesses: 6320 -> 6372 us, so not there.
             const int P = r.chain.P, rows = P / 4;
             int l2 = 0, dev = 0;
