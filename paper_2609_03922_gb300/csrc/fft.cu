@@ -190,8 +190,8 @@ spdba_status make_pass(Pass<T>* out, int64_t L, int sign, int mode, long long O,
             // leave the fewest tiles on any.  The CTAs of the last round are the first ones, of
             // which some SMs hold two (4 of 152): 608 tiles on 3 CTAs an SM are 5 on those, on 2
             // they are 4: 81.9 and 66.5 us for rows of 256 points.  Fewer than eight warps an SM
-            // lose an eighth of the rate (strided passes of 256 over 65536 pencils: 1275 us on 3
-            // CTAs, 1373 on one).
+            // lose an eighth of the rate (4096 transforms of 256 x 16, both passes: 1276 us, 1373
+            // on one CTA an SM).
             auto load = [&](long long k) {
                 const long long g = k * nsm, last = ntiles % g, spread = nsm - nsm / 16;
                 return (double)(k * (ntiles / g) + (last + spread - 1) / spread) * (k * ki.NT < 256 ? 1.125 : 1.0);
